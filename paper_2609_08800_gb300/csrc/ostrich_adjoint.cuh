@@ -44,8 +44,8 @@ template <class S> struct CGroup {
 // (a box edge's normal follows the rim centre at q-), the point the rim's deepest point
 // at q+ or the box corner; the same geometry as evaluate().
 template <class S, class Real>
-__device__ __forceinline__ void contact_group(const DevScene& sc, const WS<Real>& w, int sl, int b, const S* qm7,
-                                              const S* u6, double h, CGroup<S>& o) {
+__device__ __forceinline__ void contact_group(const KScene<Real>& sc, const WS<Real>& w, int sl, int b, const S* qm7,
+                                              const S* u6, const StepH<Real>& h, CGroup<S>& o) {
   const int local = sl - sc.slot_base[b];
   S qp[7];
   kin_body<S, S>(qm7, u6, h, qp);
@@ -75,8 +75,8 @@ __device__ __forceinline__ void contact_group(const DevScene& sc, const WS<Real>
 // vectors instead of to each row, (E a) . v = a . (E^T v); the same geometry as
 // contact_group.
 template <class S, class Real>
-__device__ __forceinline__ void contact_rows_dot(const DevScene& sc, const WS<Real>& w, int sl, int b, const S* qm7,
-                                                 const Real* u6, double h, vec3<Real> wlin, vec3<Real> wang, S& cn,
+__device__ __forceinline__ void contact_rows_dot(const KScene<Real>& sc, const WS<Real>& w, int sl, int b, const S* qm7,
+                                                 const Real* u6, const StepH<Real>& h, vec3<Real> wlin, vec3<Real> wang, S& cn,
                                                  S* vel, S* jw) {
   const int local = sl - sc.slot_base[b];
   S qp[7];
@@ -106,9 +106,9 @@ __device__ __forceinline__ void contact_rows_dot(const DevScene& sc, const WS<Re
 // friction residuals v_k + (W + kappa) lambda_fk, in S; lambda enters as S so that the
 // same code differentiates along lambda_n.
 template <class S, class Real>
-__device__ __forceinline__ S friction_rows(const DevScene& sc, S v1, S v2, S ln, Real l1, Real l2, Real hw, S mu,
+__device__ __forceinline__ S friction_rows(const KScene<Real>& sc, S v1, S v2, S ln, Real l1, Real l2, Real hw, S mu,
                                            S* rf) {
-  const Real eps = Real(sc.eps), kap = Real(sc.kappa);
+  const Real eps = sc.eps, kap = sc.kappa;
   const S vt = ssqrt(v1 * v1 + v2 * v2 + S(eps * eps));
   const Real lfn = ssqrt(l1 * l1 + l2 * l2 + eps * eps);
   const S lnp = sval(ln) > Real(0) ? ln : S(Real(0));
@@ -132,9 +132,9 @@ template <class S> struct JGroup {
 
 // Joint j between parent and child at q- and u+ (in S): the five position rows and the
 // servo row, as evaluate() forms them (same geometry helpers).
-template <class S>
-__device__ __forceinline__ void joint_group(const DevScene& sc, int j, const S* qmp, const S* up, const S* qmc,
-                                            const S* uc, double h, JGroup<S>& o) {
+template <class S, class Real>
+__device__ __forceinline__ void joint_group(const KScene<Real>& sc, int j, const S* qmp, const S* up, const S* qmc,
+                                            const S* uc, const StepH<Real>& h, JGroup<S>& o) {
   S qpp[7], qpc[7];
   kin_body<S, S>(qmp, up, h, qpp);
   kin_body<S, S>(qmc, uc, h, qpc);
@@ -157,8 +157,8 @@ __device__ __forceinline__ void joint_group(const DevScene& sc, int j, const S* 
 }
 
 // The joint coordinate at q- (in S), for a position servo's bias (x(q-) - target)/h.
-template <class S>
-__device__ __forceinline__ S joint_coord_qm(const DevScene& sc, int j, const S* qmp, const S* qmc) {
+template <class S, class Real>
+__device__ __forceinline__ S joint_coord_qm(const KScene<Real>& sc, int j, const S* qmp, const S* qmc) {
   return joint_coord<S>(sc, j, v3(qmp[0], qmp[1], qmp[2]), QuatRot<S>(qmp + 3), v3(qmc[0], qmc[1], qmc[2]),
                         QuatRot<S>(qmc + 3));
 }
@@ -175,9 +175,9 @@ template <class Real> struct ExWS {
   Real *V, *Hh, *cs, *sn, *gg, *y, *x, *r, *z, *t6, *wred, *scal;
 };
 
-template <class Real> __host__ __device__ inline int ex_n(const DevScene& s) { return 6 * s.nb + s.m_max; }
+template <class Real> __host__ __device__ inline int ex_n(const SceneLayout& s) { return 6 * s.nb + s.m_max; }
 
-template <class Real> __host__ __device__ ExWS<Real> ex_carve(char* base, const DevScene& s) {
+template <class Real> __host__ __device__ ExWS<Real> ex_carve(char* base, const SceneLayout& s) {
   ExWS<Real> e;
   char* p = base;
   const int nb = s.nb, n = ex_n<Real>(s), ns = s.n_slots > 0 ? s.n_slots : 1;
@@ -203,7 +203,7 @@ template <class Real> __host__ __device__ size_t ex_bytes(const DevScene& s) {
 }
 
 // Shared memory of one world in the adjoint kernel of a mode.
-template <class Real> __host__ __device__ size_t adj_smem_bytes(const DevScene& s, int mode) {
+template <class Real> size_t adj_smem_bytes(const DevScene& s, int mode) {
   size_t b = ws_bytes<Real>(s);
   if (mode == ADJ_EXACT) b = (b + ex_bytes<Real>(s) + 15) & ~(size_t)15;
   return b;
@@ -211,7 +211,7 @@ template <class Real> __host__ __device__ size_t adj_smem_bytes(const DevScene& 
 
 // Groups touching each body: slot indices (active slots of the body) then n_slots + j for
 // its joints, in a fixed order; built by one thread.
-template <class Real> __device__ void body_groups(const DevScene& sc, const WS<Real>& w, int* bgl, int* bgn) {
+template <class Real> __device__ void body_groups(const KScene<Real>& sc, const WS<Real>& w, int* bgl, int* bgn) {
   for (int b = 0; b < sc.nb; ++b) {
     int k = 0;
     for (int sl = sc.slot_base[b]; sl < sc.slot_base[b] + sc.slot_count[b]; ++sl)
@@ -223,7 +223,7 @@ template <class Real> __device__ void body_groups(const DevScene& sc, const WS<R
 }
 
 // Row index of the servo row of joint j (or -1) in the world's active-row order.
-template <class Real> __device__ __forceinline__ int servo_row(const DevScene& sc, const WS<Real>& w, int j) {
+template <class Real> __device__ __forceinline__ int servo_row(const KScene<Real>& sc, const WS<Real>& w, int j) {
   return sc.servo_of[j] >= 0 ? w.ints[1] + 5 * sc.nj + sc.servo_of[j] : -1;
 }
 
@@ -235,10 +235,10 @@ template <class Real> __device__ __forceinline__ int servo_row(const DevScene& s
 // fa / max(fa, 1e-12) in the exact mode as the row is).
 // ---------------------------------------------------------------------------
 template <class Real, int MODE>
-__device__ Real group_vjp_q(const DevScene& sc, const WS<Real>& w, const ExWS<Real>& ex, int grp, int db, int dc,
-                            const Real* wl, const Real* wu, bool trunc, double h) {
+__device__ Real group_vjp_q(const KScene<Real>& sc, const WS<Real>& w, const ExWS<Real>& ex, int grp, int db, int dc,
+                            const Real* wl, const Real* wu, bool trunc, const StepH<Real>& h) {
   typedef dual<Real> D;
-  const Real hR = Real(h);
+  const Real hR = h.h;
   if (grp < sc.n_slots) {
     const int sl = grp, b = sc.slot_body[sl], i = w.srow[sl];
     if (trunc) {
@@ -273,7 +273,7 @@ __device__ Real group_vjp_q(const DevScene& sc, const WS<Real>& w, const ExWS<Re
     if (MODE == ADJ_EXACT) {
       D rf[2];
       friction_rows<D, Real>(sc, vel[1], vel[2], D(w.lk[i]), w.lk[i + 1], w.lk[i + 2], hR * w.swhat[sl],
-                             D(Real(sc.mu)), rf);
+                             D(sc.mu), rf);
       acc = acc + D(wl[i + 1]) * rf[0] + D(wl[i + 2]) * rf[1];
     } else {
       acc = acc + D(wl[i + 1]) * vel[1] + D(wl[i + 2]) * vel[2];
@@ -332,10 +332,10 @@ __device__ Real group_vjp_q(const DevScene& sc, const WS<Real>& w, const ExWS<Re
 // b2 perturbed along c.  The task writes column c of body b2 in G (the rows' exact
 // derivatives) and in every K block (b, b2): each (row, column) entry belongs to one task.
 template <class Real>
-__device__ void exact_task(const DevScene& sc, const WS<Real>& w, const ExWS<Real>& ex, const int* bgl,
-                           const int* bgn, int b2, int c, double h) {
+__device__ void exact_task(const KScene<Real>& sc, const WS<Real>& w, const ExWS<Real>& ex, const int* bgl,
+                           const int* bgn, int b2, int c, const StepH<Real>& h) {
   typedef dual<Real> D;
-  const Real hR = Real(h);
+  const Real hR = h.h;
   const int nb = sc.nb;
   for (int b = 0; b < nb; ++b)
     for (int r = 0; r < 6; ++r) ex.K[(b * nb + b2) * 36 + r * 6 + c] = Real(0);
@@ -350,7 +350,7 @@ __device__ void exact_task(const DevScene& sc, const WS<Real>& w, const ExWS<Rea
       contact_group<D, Real>(sc, w, sl, b2, qm, u, h, g);
       D rf[2];
       friction_rows<D, Real>(sc, g.vel[1], g.vel[2], D(w.lk[i]), w.lk[i + 1], w.lk[i + 2], hR * w.swhat[sl],
-                             D(Real(sc.mu)), rf);
+                             D(sc.mu), rf);
       ex.G[12 * i + c] = ex.fsc[sl] * g.cn.d / hR;
       ex.G[12 * (i + 1) + c] = rf[0].d;
       ex.G[12 * (i + 2) + c] = rf[1].d;
@@ -399,10 +399,10 @@ __device__ void exact_task(const DevScene& sc, const WS<Real>& w, const ExWS<Rea
 
 // Per active slot: the normal row's derivative scale fa / max(fa, 1e-12) and the friction
 // rows' derivatives along lambda_n (through W), at the returned iterate.
-template <class Real> __device__ void exact_slot_terms(const DevScene& sc, const WS<Real>& w, const ExWS<Real>& ex,
-                                                       double h) {
+template <class Real> __device__ void exact_slot_terms(const KScene<Real>& sc, const WS<Real>& w, const ExWS<Real>& ex,
+                                                       const StepH<Real>& h) {
   typedef dual<Real> D;
-  const Real hR = Real(h), eps = Real(sc.eps), kap = Real(sc.kappa);
+  const Real hR = h.h, eps = sc.eps, kap = sc.kappa;
   for (int sl = threadIdx.x; sl < sc.n_slots; sl += blockDim.x) {
     if (!w.sact[sl]) continue;
     const int i = w.srow[sl], b = sc.slot_body[sl];
@@ -418,7 +418,7 @@ template <class Real> __device__ void exact_slot_terms(const DevScene& sc, const
     ex.fsc[sl] = fa / (fa > Real(1e-12) ? fa : Real(1e-12));
     D rf[2];
     friction_rows<D, Real>(sc, D(g.vel[1]), D(g.vel[2]), D(ln, Real(1)), w.lk[i + 1], w.lk[i + 2], hw,
-                           D(Real(sc.mu)), rf);
+                           D(sc.mu), rf);
     ex.cfn[2 * sl] = rf[0].d;
     ex.cfn[2 * sl + 1] = rf[1].d;
   }
@@ -434,10 +434,10 @@ template <class Real> __device__ void exact_slot_terms(const DevScene& sc, const
 // friction blocks plus, per contact, the friction rows' lambda_n column).  Compensated
 // sums: the two terms of out_l nearly cancel at the solution.
 template <class Real>
-__device__ void exact_apply(const DevScene& sc, const WS<Real>& w, const ExWS<Real>& ex, const Real* v, Real* out,
-                            double h, Real sigma) {
+__device__ void exact_apply(const KScene<Real>& sc, const WS<Real>& w, const ExWS<Real>& ex, const Real* v, Real* out,
+                            const StepH<Real>& h, Real sigma) {
   const int tid = threadIdx.x, nth = blockDim.x, nb = sc.nb, m = w.ints[0];
-  const Real hR = Real(h);
+  const Real hR = h.h;
   const Real* vu = v;
   const Real* vl = v + 6 * nb;
   const int ssd = sc.ss > 0 ? sc.ss : 1;
@@ -445,7 +445,7 @@ __device__ void exact_apply(const DevScene& sc, const WS<Real>& w, const ExWS<Re
     const int b = task / 6, k = task - 6 * b;
     acc2<Real> a;
     // M^T v_u (M symmetric: mass and world inertia at q-)
-    if (k < 3) a.add_prod(Real(sc.mass[b]), vu[6 * b + k]);
+    if (k < 3) a.add_prod(sc.mass[b], vu[6 * b + k]);
     else for (int q = 0; q < 3; ++q) a.add_prod(w.Iw[9 * b + 3 * (k - 3) + q], vu[6 * b + 3 + q]);
     // K^T v_u: column (b, k) of K over all row blocks
     for (int bb = 0; bb < nb; ++bb)
@@ -470,7 +470,7 @@ __device__ void exact_apply(const DevScene& sc, const WS<Real>& w, const ExWS<Re
     const int t = w.meta[4 * i] & 15, sub = w.meta[4 * i] >> 4;
     // normal rows: d(phi/scl)/dlambda_n = (fa kappa + fb h what)/scl; evaluate() keeps
     // kappa + fb h what/scl, equal unless the scale is clamped (fa < 1e-12)
-    const Real cii = t == ROW_NORMAL ? w.C[i] + (ex.fsc[w.ref[i]] - Real(1)) * Real(sc.kappa) : w.C[i];
+    const Real cii = t == ROW_NORMAL ? w.C[i] + (ex.fsc[w.ref[i]] - Real(1)) * sc.kappa : w.C[i];
     a.add_prod(cii, vl[i]);
     if (t == ROW_FRIC) {
       const Real* rd = w.srad + 3 * w.ref[i];
@@ -492,10 +492,10 @@ __device__ void exact_apply(const DevScene& sc, const WS<Real>& w, const ExWS<Re
 //   z_lambda = A^-1 (v_lambda / sigma + h J M^-1 v_u),  z_u = M^-1 (v_u - J^T z_lambda).
 // z may not alias v.  Uses w.mr, w.rhs and ex.t6 as scratch.
 template <class Real>
-__device__ void exact_precond(const DevScene& sc, WS<Real>& w, const ExWS<Real>& ex, const Real* v, Real* z, double h,
+__device__ void exact_precond(const KScene<Real>& sc, WS<Real>& w, const ExWS<Real>& ex, const Real* v, Real* z, const StepH<Real>& h,
                               Real sigma) {
   const int tid = threadIdx.x, nth = blockDim.x, nb = sc.nb, m = w.ints[0];
-  const Real hR = Real(h);
+  const Real hR = h.h;
   for (int b = tid; b < nb; b += nth) minv6(sc, w, b, v + 6 * b, w.mr + 6 * b);
   __syncthreads();
   for (int i = tid; i < m; i += nth) {
@@ -553,7 +553,7 @@ template <class Real> __device__ Real block_norm(const ExWS<Real>& ex, const Rea
 // mode's solution P^-T b.  Returns the Krylov iterations run; *conv_out says whether the
 // weighted residual fell below rel_tol times that of the starting point's right-hand side.
 template <class Real>
-__device__ int exact_gmres(const DevScene& sc, WS<Real>& w, const ExWS<Real>& ex, double h, Real sigma, Real rel_tol,
+__device__ int exact_gmres(const KScene<Real>& sc, WS<Real>& w, const ExWS<Real>& ex, const StepH<Real>& h, Real sigma, Real rel_tol,
                            int* conv_out) {
   const int tid = threadIdx.x, nth = blockDim.x, n = 6 * sc.nb + w.ints[0];
   Real* V = ex.V;

@@ -53,7 +53,7 @@ __device__ __forceinline__ f3 rrim_deepest(f3 c, f3 a, float r, f3 n) {
 struct Cand { int valid, ftype; f3 n; float d, ex, ez; };
 
 // Features of the box obstacle for one rim: 0 ground, 1 top, 2 near face, 3 near top edge.
-__device__ __forceinline__ Cand rbox_feature(const DevScene& s, int f, f3 c, f3 a, float r) {
+template <class Real> __device__ __forceinline__ Cand rbox_feature(const KScene<Real>& s, int f, f3 c, f3 a, float r) {
   Cand k; k.valid = 0; k.ftype = 0; k.n = mkf3(0.f, 0.f, 1.f); k.d = 0.f; k.ex = 0.f; k.ez = 0.f;
   float x0 = (float)s.box[0], x1 = (float)s.box[1], y0 = (float)s.box[2], y1 = (float)s.box[3], H = (float)s.box[4];
   float xm = rmul(0.5f, radd(x0, x1));
@@ -106,14 +106,14 @@ __device__ __forceinline__ bool rpredicate(f3 x, f3 n, float d, f3 p, f3 v, f3 w
 // (i, j)-(i+1, j+1) diagonal into face 0 {(i,j), (i+1,j), (i+1,j+1)} and face 1
 // {(i,j), (i+1,j+1), (i,j+1)}; face id = 2 ((n - 1) i + j) + t.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float hm_x(const DevScene& s, int i) { return radd((float)s.hox, rmul((float)i, (float)s.hsp)); }
-__device__ __forceinline__ float hm_y(const DevScene& s, int j) { return radd((float)s.hoy, rmul((float)j, (float)s.hsp)); }
-__device__ __forceinline__ f3 hm_vertex(const DevScene& s, int i, int j) {
+template <class Real> __device__ __forceinline__ float hm_x(const KScene<Real>& s, int i) { return radd((float)s.hox, rmul((float)i, (float)s.hsp)); }
+template <class Real> __device__ __forceinline__ float hm_y(const KScene<Real>& s, int j) { return radd((float)s.hoy, rmul((float)j, (float)s.hsp)); }
+template <class Real> __device__ __forceinline__ f3 hm_vertex(const KScene<Real>& s, int i, int j) {
   return mkf3(hm_x(s, i), hm_y(s, j), __ldg(s.heights + (size_t)i * s.hn + j));
 }
 
 // plane (n, d) of a face: n = normalised cross product of the two edges from (i, j)
-__device__ __forceinline__ void hm_face(const DevScene& s, int i, int j, int t, f3& n, float& d) {
+template <class Real> __device__ __forceinline__ void hm_face(const KScene<Real>& s, int i, int j, int t, f3& n, float& d) {
   f3 A = hm_vertex(s, i, j);
   f3 B = t == 0 ? hm_vertex(s, i + 1, j) : hm_vertex(s, i + 1, j + 1);
   f3 C = t == 0 ? hm_vertex(s, i + 1, j + 1) : hm_vertex(s, i, j + 1);
@@ -124,7 +124,7 @@ __device__ __forceinline__ void hm_face(const DevScene& s, int i, int j, int t, 
 }
 
 // cell under the horizontal position of x, clamped to the grid
-__device__ __forceinline__ void hm_cell(const DevScene& s, f3 x, int& i, int& j) {
+template <class Real> __device__ __forceinline__ void hm_cell(const KScene<Real>& s, f3 x, int& i, int& j) {
   float fi = floorf(__fdiv_rn(rsub(x.x, (float)s.hox), (float)s.hsp));
   float fj = floorf(__fdiv_rn(rsub(x.y, (float)s.hoy), (float)s.hsp));
   float top = (float)(s.hn - 2);
@@ -133,7 +133,7 @@ __device__ __forceinline__ void hm_cell(const DevScene& s, f3 x, int& i, int& j)
 }
 
 // does the horizontal position of x lie on face (i, j, t)?  (edges inclusive)
-__device__ __forceinline__ bool hm_on_face(const DevScene& s, f3 x, int i, int j, int t) {
+template <class Real> __device__ __forceinline__ bool hm_on_face(const KScene<Real>& s, f3 x, int i, int j, int t) {
   float x0 = hm_x(s, i), x1 = hm_x(s, i + 1), y0 = hm_y(s, j), y1 = hm_y(s, j + 1);
   if (!(x.x >= x0 && x.x <= x1 && x.y >= y0 && x.y <= y1)) return false;
   float u = rsub(x.x, x0), v = rsub(x.y, y0);
@@ -145,9 +145,10 @@ __device__ __forceinline__ bool hm_on_face(const DevScene& s, f3 x, int i, int j
 // centre cell of a 3 x 3 block; each face of the block whose own deepest rim point lies
 // on the face is a candidate, in scan order (cell row, cell column, face), filling the
 // rim's slots; returns true when candidates were left over (more than nf).
-__device__ __forceinline__ bool activate_rim_hm(const DevScene& s, int b, int rim, const float* q7, const float* u6,
-                                                double h, SlotAct* out) {
-  float hf = (float)h, hg = rmul(hf, (float)s.g), margin = (float)s.margin;
+template <class Real>
+__device__ __forceinline__ bool activate_rim_hm(const KScene<Real>& s, int b, int rim, const float* q7, const float* u6,
+                                                SlotAct* out) {
+  float hf = (float)s.hs.h, hg = rmul(hf, (float)s.g), margin = (float)s.margin;
   const float* q = q7 + 3;
   f3 p = mkf3(q7[0], q7[1], q7[2]);
   f3 v = mkf3(u6[0], u6[1], u6[2]);
@@ -190,10 +191,11 @@ __device__ __forceinline__ bool activate_rim_hm(const DevScene& s, int b, int ri
 
 // Activation of slot `sl` (global slot index) of one world, from the FP32 state of its body.
 // q7: position + quaternion, u6: linear + angular velocity (world frame).
-__device__ __forceinline__ SlotAct activate_slot(const DevScene& s, int b, int local, const float* q7, const float* u6,
-                                                 double h) {
+template <class Real>
+__device__ __forceinline__ SlotAct activate_slot(const KScene<Real>& s, int b, int local, const float* q7,
+                                                 const float* u6) {
   SlotAct o; o.active = 0; o.id = -1; o.ftype = 0; o.n[0] = 0.f; o.n[1] = 0.f; o.n[2] = 1.f; o.d = 0.f; o.ex = 0.f; o.ez = 0.f;
-  float hf = (float)h, hg = rmul(hf, (float)s.g), margin = (float)s.margin;
+  float hf = (float)s.hs.h, hg = rmul(hf, (float)s.g), margin = (float)s.margin;
   const float* q = q7 + 3;
   f3 p = mkf3(q7[0], q7[1], q7[2]);
   f3 v = mkf3(u6[0], u6[1], u6[2]);

@@ -65,7 +65,7 @@ template <class T> __host__ __device__ __forceinline__ T* carve(char*& p, int n)
 }
 
 
-template <class Real> __host__ __device__ WS<Real> ws_carve(char* base, const DevScene& s) {
+template <class Real> __host__ __device__ WS<Real> ws_carve(char* base, const SceneLayout& s) {
   WS<Real> w;
   char* p = base;
   int nb = s.nb, m = s.m_max, ns = s.n_slots > 0 ? s.n_slots : 1, ng = s.n_groups > 0 ? s.n_groups : 1;
@@ -103,12 +103,14 @@ template <class Real> __host__ __device__ WS<Real> ws_carve(char* base, const De
 // Dynamic shared memory of one world: the carve itself, run from a 16-byte aligned base
 // (the dynamic shared-memory base is 16-byte aligned and carve aligns to 8), rounded up
 // to 16 bytes.
-template <class Real> __host__ __device__ size_t ws_bytes(const DevScene& s) {
+template <class Real> __host__ __device__ size_t ws_layout_bytes(const SceneLayout& s) {
   char* base = reinterpret_cast<char*>(uintptr_t(16));
   WS<Real> w = ws_carve<Real>(base, s);
   size_t used = (size_t)(reinterpret_cast<char*>(w.pcr ? w.pcr + 7 * s.m_max : w.scal + 8) - base);
   return (used + 15) & ~(size_t)15;
 }
+
+template <class Real> size_t ws_bytes(const DevScene& s) { return ws_layout_bytes<Real>(s); }
 
 // deterministic block reduction (fixed tree); result broadcast through w.red[0]
 template <class Real> __device__ Real block_sum(WS<Real>& w, Real v) {
@@ -180,7 +182,7 @@ template <class Real> __device__ void block_max2(WS<Real>& w, Real& a, Real& b) 
 // geometry helpers in any scalar type S
 // ---------------------------------------------------------------------------
 template <class S> __device__ __forceinline__ void tangent_basis(vec3<S> n, vec3<S>& t1, vec3<S>& t2) {
-  vec3<S> e = fabs((double)sval(n.x)) < 0.9 ? v3(S(1), S(0), S(0)) : v3(S(0), S(1), S(0));
+  vec3<S> e = below_09(fabs(sval(n.x))) ? v3(S(1), S(0), S(0)) : v3(S(0), S(1), S(0));
   vec3<S> t = e - scale(n, dot3(n, e));
   S l = ssqrt(dot3(t, t));
   t1 = scale(t, S(1) / l);
@@ -189,7 +191,7 @@ template <class S> __device__ __forceinline__ void tangent_basis(vec3<S> n, vec3
 
 // contact point on body b at pose (p, q) for slot kind: box corner (material point) or
 // rim (deepest point of the rim circle along -n)
-template <class S> __device__ __forceinline__ vec3<S> slot_point(const DevScene& sc, int b, int local, vec3<S> p,
+template <class S, class Real> __device__ __forceinline__ vec3<S> slot_point(const KScene<Real>& sc, int b, int local, vec3<S> p,
                                                                  const S* q, vec3<S> n) {
   if (sc.shape[b] == SHAPE_BOX) {
     int k = local;
@@ -203,12 +205,12 @@ template <class S> __device__ __forceinline__ vec3<S> slot_point(const DevScene&
   S nd = dot3(n, a);
   vec3<S> perp = n - scale(a, nd);
   S pl = ssqrt(dot3(perp, perp));
-  if ((double)sval(pl) <= 1e-12) return cen;
+  if (upto_1em12(sval(pl))) return cen;
   return cen - scale(perp, S(sc.radius[b]) / pl);
 }
 
 // frame (n, d) of a slot: fixed plane, or box edge with normal toward the rim centre at q-
-template <class S, class Real> __device__ __forceinline__ void slot_frame2(const DevScene& sc, int b, int local, int ftype,
+template <class S, class Real> __device__ __forceinline__ void slot_frame2(const KScene<Real>& sc, int b, int local, int ftype,
                                                                            const S* qm7, const Real* nstore, Real dstore,
                                                                            const Real* edge, vec3<S>& n, S& d) {
   if (ftype == 1) {
@@ -252,7 +254,7 @@ template <class S> struct QuatRot {
   }
 };
 
-template <class S> __device__ __forceinline__ vec3<S> cvec(const double* a) { return v3(S(a[0]), S(a[1]), S(a[2])); }
+template <class S, class Real> __device__ __forceinline__ vec3<S> cvec(const Real* a) { return v3(S(a[0]), S(a[1]), S(a[2])); }
 
 // The five rows of joint j (Eq. (3)): Jacobian parts before the rotation-rate map E and the
 // constraint values, handed row by row (k = 0..4) to f(k, lin_p, ang_p, lin_c, ang_c, c) so
@@ -261,8 +263,8 @@ template <class S> __device__ __forceinline__ vec3<S> cvec(const double* a) { re
 // Revolute: anchor rows (p_p + r_p) - (p_c + r_c) by component, then the alignment rows
 // perp_k,p . axis_c.  Prismatic: b_k . d (b_k = R_p perp_k, d = (p_c + r_c) - (p_p + r_p)),
 // the alignment rows, and the twist lock perp2_p . perp1_c.
-template <class S, class RP, class RC, class F>
-__device__ __forceinline__ void joint_rows_each(const DevScene& sc, int j, vec3<S> pp, const RP& rotp, vec3<S> pc,
+template <class S, class RP, class RC, class F, class Real>
+__device__ __forceinline__ void joint_rows_each(const KScene<Real>& sc, int j, vec3<S> pp, const RP& rotp, vec3<S> pc,
                                                 const RC& rotc, F&& f) {
   const vec3<S> z = v3(S(0.0), S(0.0), S(0.0));
   if (sc.jtype[j] == JOINT_REVOLUTE) {
@@ -310,8 +312,8 @@ template <class S> struct JRows {
   S c[5];
 };
 
-template <class S, class RP, class RC>
-__device__ __forceinline__ void joint_rows_geom(const DevScene& sc, int j, vec3<S> pp, const RP& rotp, vec3<S> pc,
+template <class S, class RP, class RC, class Real>
+__device__ __forceinline__ void joint_rows_geom(const KScene<Real>& sc, int j, vec3<S> pp, const RP& rotp, vec3<S> pc,
                                                 const RC& rotc, JRows<S>& o) {
   joint_rows_each<S>(sc, j, pp, rotp, pc, rotc, [&](int k, vec3<S> lp, vec3<S> ap, vec3<S> lc, vec3<S> ac, S c) {
     o.lin_p[k] = lp; o.ang_p[k] = ap; o.lin_c[k] = lc; o.ang_c[k] = ac; o.c[k] = c;
@@ -323,8 +325,8 @@ __device__ __forceinline__ void joint_rows_geom(const DevScene& sc, int j, vec3<
 // (prismatic).
 template <class S> struct SRow { vec3<S> lin_p, ang_p, lin_c, ang_c; };
 
-template <class S, class RP, class RC>
-__device__ __forceinline__ void servo_row_geom(const DevScene& sc, int j, vec3<S> pp, const RP& rotp, vec3<S> pc,
+template <class S, class RP, class RC, class Real>
+__device__ __forceinline__ void servo_row_geom(const KScene<Real>& sc, int j, vec3<S> pp, const RP& rotp, vec3<S> pc,
                                                const RC& rotc, SRow<S>& o) {
   const vec3<S> a = rotp(cvec<S>(sc.axp[j]));
   if (sc.jtype[j] == JOINT_REVOLUTE) {
@@ -347,8 +349,8 @@ template <class T> __device__ __forceinline__ dual<T> satan2(dual<T> y, dual<T> 
   return dual<T>(satan2(y.v, x.v), (x.v * y.d - y.v * x.d) / r2);
 }
 
-template <class S, class RP, class RC>
-__device__ __forceinline__ S joint_coord(const DevScene& sc, int j, vec3<S> pp, const RP& rotp, vec3<S> pc,
+template <class S, class RP, class RC, class Real>
+__device__ __forceinline__ S joint_coord(const KScene<Real>& sc, int j, vec3<S> pp, const RP& rotp, vec3<S> pc,
                                          const RC& rotc) {
   const vec3<S> a = rotp(cvec<S>(sc.axp[j]));
   if (sc.jtype[j] == JOINT_REVOLUTE) {
@@ -360,13 +362,8 @@ __device__ __forceinline__ S joint_coord(const DevScene& sc, int j, vec3<S> pp, 
   return dot3(a, (pc + rc) - (pp + rp));
 }
 
-// Servo compliance alpha of Eq. (8): 1/kp (velocity target), 1/(kd + h kp) (position).
-__device__ __forceinline__ double servo_alpha(const DevScene& sc, int j, double h) {
-  return sc.smode[j] == SERVO_POSITION ? 1.0 / (sc.kd[j] + h * sc.kp[j]) : 1.0 / sc.kp[j];
-}
-
 // Joint of the k-th servo.
-__device__ __forceinline__ int servo_joint(const DevScene& sc, int k) {
+template <class Real> __device__ __forceinline__ int servo_joint(const KScene<Real>& sc, int k) {
   int j = 0, cnt = -1;
   for (j = 0; j < sc.nj; ++j) if (sc.servo_of[j] >= 0 && ++cnt == k) break;
   return j;
@@ -400,8 +397,8 @@ __device__ __forceinline__ int tape_to_int(double v) { return (int)v; }
 // record's slot table); ct_in: when not null, the table is read from there instead of
 // running the activation (the adjoint, at the taped step: the same set by construction).
 template <class Real>
-__device__ void world_setup(const DevScene& sc, WS<Real>& w, Src<Real> qmv, Src<Real> umv, Src<Real> ubarv,
-                            double h, Real* ct_out = nullptr, const Real* ct_in = nullptr) {
+__device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, Src<Real> umv, Src<Real> ubarv,
+                            const StepH<Real>& h, Real* ct_out = nullptr, const Real* ct_in = nullptr) {
   const int tid = threadIdx.x, nth = blockDim.x;
   const int nb = sc.nb;
   for (int i = tid; i < 7 * nb; i += nth) w.qm[i] = qmv.p[i * qmv.stride];
@@ -448,7 +445,7 @@ __device__ void world_setup(const DevScene& sc, WS<Real>& w, Src<Real> qmv, Src<
       for (int k = 0; k < 7; ++k) q7[k] = (float)w.qm[7 * b + k];
       for (int k = 0; k < 6; ++k) u6[k] = (float)w.um[6 * b + k];
       SlotAct acts[8];
-      if (activate_rim_hm(sc, b, rim, q7, u6, h, acts)) atomicOr(&w.ints[7], 4);
+      if (activate_rim_hm(sc, b, rim, q7, u6, acts)) atomicOr(&w.ints[7], 4);
       for (int f = 0; f < sc.nf; ++f) store_slot(sc.slot_base[b] + rim * sc.nf + f, b, rim * sc.nf + f, acts[f]);
     }
     for (int sl = tid; sl < sc.n_slots; sl += nth)      // box corners (no wheel rim)
@@ -457,7 +454,7 @@ __device__ void world_setup(const DevScene& sc, WS<Real>& w, Src<Real> qmv, Src<
         float q7[7], u6[6];
         for (int k = 0; k < 7; ++k) q7[k] = (float)w.qm[7 * b + k];
         for (int k = 0; k < 6; ++k) u6[k] = (float)w.um[6 * b + k];
-        store_slot(sl, b, sl - sc.slot_base[b], activate_slot(sc, b, sl - sc.slot_base[b], q7, u6, h));
+        store_slot(sl, b, sl - sc.slot_base[b], activate_slot(sc, b, sl - sc.slot_base[b], q7, u6));
       }
   } else {
     for (int sl = tid; sl < sc.n_slots; sl += nth) {
@@ -466,7 +463,7 @@ __device__ void world_setup(const DevScene& sc, WS<Real>& w, Src<Real> qmv, Src<
       float q7[7], u6[6];
       for (int k = 0; k < 7; ++k) q7[k] = (float)w.qm[7 * b + k];
       for (int k = 0; k < 6; ++k) u6[k] = (float)w.um[6 * b + k];
-      store_slot(sl, b, local, activate_slot(sc, b, local, q7, u6, h));
+      store_slot(sl, b, local, activate_slot(sc, b, local, q7, u6));
     }
   }
   // bodies: world inertia at q-, external force, warm-start velocity
@@ -478,24 +475,24 @@ __device__ void world_setup(const DevScene& sc, WS<Real>& w, Src<Real> qmv, Src<
       for (int j = 0; j < 3; ++j) {
         Real a = 0, ai = 0;
         for (int k = 0; k < 3; ++k) {
-          a += R[3 * i + k] * Real(sc.inertia[b][k]) * R[3 * j + k];
-          ai += R[3 * i + k] * (Real(1) / Real(sc.inertia[b][k])) * R[3 * j + k];
+          a += R[3 * i + k] * sc.inertia[b][k] * R[3 * j + k];
+          ai += R[3 * i + k] * sc.iinv[b][k] * R[3 * j + k];
         }
         w.Iw[9 * b + 3 * i + j] = a; w.Iwi[9 * b + 3 * i + j] = ai;
       }
-    Real m = Real(sc.mass[b]);
+    Real m = sc.mass[b];
     vec3<Real> om = v3(w.um[6 * b + 3], w.um[6 * b + 4], w.um[6 * b + 5]);
     vec3<Real> Io = mat3<Real>(w.Iw + 9 * b, om);
     vec3<Real> gy = cross3(om, Io);
-    w.f[6 * b] = 0; w.f[6 * b + 1] = 0; w.f[6 * b + 2] = m * Real(sc.g);
+    w.f[6 * b] = 0; w.f[6 * b + 1] = 0; w.f[6 * b + 2] = m * sc.g;
     w.f[6 * b + 3] = -gy.x; w.f[6 * b + 4] = -gy.y; w.f[6 * b + 5] = -gy.z;
     vec3<Real> dw = mat3<Real>(w.Iwi + 9 * b, v3(w.f[6 * b + 3], w.f[6 * b + 4], w.f[6 * b + 5]));
     w.uk[6 * b] = w.um[6 * b];
     w.uk[6 * b + 1] = w.um[6 * b + 1];
-    w.uk[6 * b + 2] = w.um[6 * b + 2] + Real(h) * Real(sc.g);
-    w.uk[6 * b + 3] = w.um[6 * b + 3] + Real(h) * dw.x;
-    w.uk[6 * b + 4] = w.um[6 * b + 4] + Real(h) * dw.y;
-    w.uk[6 * b + 5] = w.um[6 * b + 5] + Real(h) * dw.z;
+    w.uk[6 * b + 2] = w.um[6 * b + 2] + h.h * sc.g;
+    w.uk[6 * b + 3] = w.um[6 * b + 3] + h.h * dw.x;
+    w.uk[6 * b + 4] = w.um[6 * b + 4] + h.h * dw.y;
+    w.uk[6 * b + 5] = w.um[6 * b + 5] + h.h * dw.z;
   }
   __syncthreads();
   // servo biases b_c of Eq. (8): -target (velocity target) or (x(q-) - target)/h (position
@@ -506,7 +503,7 @@ __device__ void world_setup(const DevScene& sc, WS<Real>& w, Src<Real> qmv, Src<
       const Real x = joint_coord<Real>(sc, j, v3(w.qm[7 * bp], w.qm[7 * bp + 1], w.qm[7 * bp + 2]),
                                        MatRot<Real>{w.R + 9 * bp},
                                        v3(w.qm[7 * bc], w.qm[7 * bc + 1], w.qm[7 * bc + 2]), MatRot<Real>{w.R + 9 * bc});
-      w.sbc[k] = (x - w.ubar[k]) / Real(h);
+      w.sbc[k] = (x - w.ubar[k]) / h.h;
     } else {
       w.sbc[k] = -w.ubar[k];
     }
@@ -597,17 +594,17 @@ __device__ void world_setup(const DevScene& sc, WS<Real>& w, Src<Real> qmv, Src<
     vec3<Real> x = slot_point<Real>(sc, b, local, p, w.qm + 7 * b + 3, n);
     vec3<Real> a = cross3(x - p, n);
     vec3<Real> ia = mat3<Real>(w.Iwi + 9 * b, a);
-    w.swhat[sl] = Real(1) / Real(sc.mass[b]) + dot3(a, ia);
+    w.swhat[sl] = sc.minv[b] + dot3(a, ia);
   }
   __syncthreads();
 }
 
-template <class Real> __device__ __forceinline__ void clamp_cone(const DevScene& sc, WS<Real>& w, Real* lam) {
+template <class Real> __device__ __forceinline__ void clamp_cone(const KScene<Real>& sc, WS<Real>& w, Real* lam) {
   // first safeguard of Sec. III-B: |lambda_f| <= mu lambda_n
   for (int sl = threadIdx.x; sl < sc.n_slots; sl += blockDim.x) {
     if (!w.sact[sl]) continue;
     int i = w.srow[sl];
-    Real rad = Real(sc.mu) * (lam[i] > Real(0) ? lam[i] : Real(0));
+    Real rad = sc.mu * (lam[i] > Real(0) ? lam[i] : Real(0));
     Real nn = ssqrt(lam[i + 1] * lam[i + 1] + lam[i + 2] * lam[i + 2]);
     if (nn > rad) {
       Real f = nn > Real(0) ? rad / nn : Real(0);
@@ -623,14 +620,14 @@ template <class Real> __device__ __forceinline__ Real rowdot(const Real* Ja, int
 
 // y = M^-1 J_i^T for both body blocks of row i: (J_lin / m, Iw^-1 J_ang) per side (zero
 // for a side without a body); the same values Eq. (2)'s M~^-1 gives the row.
-template <class Real> __device__ __forceinline__ void minv_row(const DevScene& sc, const WS<Real>& w, int i, Real* y) {
+template <class Real> __device__ __forceinline__ void minv_row(const KScene<Real>& sc, const WS<Real>& w, int i, Real* y) {
   const Real* Jr = w.J + 12 * i;
   for (int side = 0; side < 2; ++side) {
     const int b = w.meta[4 * i + 1 + side];
     Real* ys = y + 6 * side;
     if (b < 0) { for (int q = 0; q < 6; ++q) ys[q] = Real(0); continue; }
     const Real* Js = Jr + 6 * side;
-    const Real mi = Real(1) / Real(sc.mass[b]);
+    const Real mi = sc.minv[b];
     ys[0] = Js[0] * mi; ys[1] = Js[1] * mi; ys[2] = Js[2] * mi;
     const vec3<Real> ia = mat3<Real>(w.Iwi + 9 * b, v3(Js[3], Js[4], Js[5]));
     ys[3] = ia.x; ys[4] = ia.y; ys[5] = ia.z;
@@ -643,10 +640,10 @@ template <class Real> __device__ __forceinline__ void minv_row(const DevScene& s
 // dyn = false (the adjoint): the rows, their compliance and delta only; the dynamics
 // residual and the merit are not formed (the returned merit is 0).
 template <class Real>
-__device__ Real evaluate(const DevScene& sc, WS<Real>& w, const Real* u, const Real* lam, double h, bool dyn = true) {
+__device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, const Real* lam, const StepH<Real>& h, bool dyn = true) {
   const int tid = threadIdx.x, nth = blockDim.x;
   const int nb = sc.nb, m = w.ints[0], mc = w.ints[1];
-  const Real hR = Real(h);
+  const Real hR = h.h;
   // poses at q+ = q- + h G(q-) u
   for (int b = tid; b < nb; b += nth) {
     kin_body<Real, Real>(w.qm + 7 * b, u + 6 * b, h, w.qp + 7 * b);
@@ -679,7 +676,7 @@ __device__ Real evaluate(const DevScene& sc, WS<Real>& w, const Real* u, const R
         vel[k] = dirs[k].x * u[6 * b] + dirs[k].y * u[6 * b + 1] + dirs[k].z * u[6 * b + 2] + ang.x * u[6 * b + 3] +
                  ang.y * u[6 * b + 4] + ang.z * u[6 * b + 5];
       }
-      const Real kap = Real(sc.kappa), eps = Real(sc.eps);
+      const Real kap = sc.kappa, eps = sc.eps;
       const Real hw = hR * w.swhat[sl];
       // normal row, Eq. (4): phi_eps(c_n/h + kappa lambda_n, h what lambda_n)
       Real cn = dot3(n, x) - w.sd[sl];
@@ -703,12 +700,12 @@ __device__ Real evaluate(const DevScene& sc, WS<Real>& w, const Real* u, const R
       Real vt = ssqrt(vel[1] * vel[1] + vel[2] * vel[2] + eps * eps);
       Real lfn = ssqrt(l1 * l1 + l2 * l2 + eps * eps);
       Real lnp = ln > Real(0) ? ln : Real(0);
-      Real g = hw * (Real(sc.mu) * lnp - lfn);
+      Real g = hw * (sc.mu * lnp - lfn);
       Real sg = ssqrt(vt * vt + g * g + eps * eps);
       // W's numerator max(0, vt - phi_eps(vt, g)) is sg - g >= 0; for g > 0 (sticking) it is
       // the small difference of two large numbers, taken as (vt^2 + eps^2)/(sg + g)
       Real num = g > Real(0) ? (vt * vt + eps * eps) / (sg + g) : sg - g;
-      Real den = Real(sc.mu) * lnp; if (den < Real(1e-12)) den = Real(1e-12);
+      Real den = sc.mu * lnp; if (den < Real(1e-12)) den = Real(1e-12);
       Real W = num / den;
       Real rf1 = vel[1] + (W + kap) * l1, rf2 = vel[2] + (W + kap) * l2;
       Real wgt = hw / (hw + W);
@@ -757,7 +754,7 @@ __device__ Real evaluate(const DevScene& sc, WS<Real>& w, const Real* u, const R
       Jr[6] = sr.lin_c.x; Jr[7] = sr.lin_c.y; Jr[8] = sr.lin_c.z; Jr[9] = ac_.x; Jr[10] = ac_.y; Jr[11] = ac_.z;
       Real v = Real(0);
       for (int q = 0; q < 6; ++q) v += Jr[q] * u[6 * bp + q] + Jr[6 + q] * u[6 * bc + q];
-      const Real alpha = Real(servo_alpha(sc, j, h));
+      const Real alpha = sc.alpha[j];
       const Real r = v + alpha * lam[i] + w.sbc[k];
       w.r2[i] = r; w.rhat[i] = r; w.C[i] = alpha;
     }
@@ -780,7 +777,7 @@ __device__ Real evaluate(const DevScene& sc, WS<Real>& w, const Real* u, const R
         rd.add_prod(w.J[12 * i + side + k], -hR * lam[i]);
       }
       if (k < 3) {
-        const Real m_ = Real(sc.mass[b]);
+        const Real m_ = sc.mass[b];
         rd.add_prod(m_, u[6 * b + k]);
         rd.add_prod(-m_, w.um[6 * b + k]);
       } else {
@@ -797,7 +794,7 @@ __device__ Real evaluate(const DevScene& sc, WS<Real>& w, const Real* u, const R
   Real part = Real(0);
   for (int b = tid; b < nb && dyn; b += nth) {
     const Real* rv = w.rdyn + 6 * b;
-    Real mi = Real(1) / Real(sc.mass[b]);
+    Real mi = sc.minv[b];
     vec3<Real> iw = mat3<Real>(w.Iwi + 9 * b, v3(rv[3], rv[4], rv[5]));
     Real mr[6] = {rv[0] * mi, rv[1] * mi, rv[2] * mi, iw.x, iw.y, iw.z};
     for (int k = 0; k < 6; ++k) { w.mr[6 * b + k] = mr[k]; part += mr[k] * mr[k]; }
@@ -814,7 +811,7 @@ __device__ Real evaluate(const DevScene& sc, WS<Real>& w, const Real* u, const R
     dpart += hR * (rowdot(Ji, 0, Yi, 0) + rowdot(Ji, 6, Yi, 6));
   }
   block_sum2(w, part, dpart);
-  if (tid == 0) w.scal[2] = m > 0 ? Real(sc.delta_rel) * dpart / Real(m) : Real(0);
+  if (tid == 0) w.scal[2] = m > 0 ? sc.delta_rel * dpart / Real(m) : Real(0);
   __syncthreads();                         // scal[2] is read by the assembly that follows
   return part;
 }
@@ -824,10 +821,10 @@ __device__ Real evaluate(const DevScene& sc, WS<Real>& w, const Real* u, const R
 // ---------------------------------------------------------------------------
 
 
-template <class Real> __device__ void assemble(const DevScene& sc, WS<Real>& w, double h) {
+template <class Real> __device__ void assemble(const KScene<Real>& sc, WS<Real>& w, const StepH<Real>& h) {
   const int tid = threadIdx.x, nth = blockDim.x;
   const int m = w.ints[0], mc = w.ints[1], gstr = tri_size(sc.pg), ss = sc.ss, ldg = sc.ldg;
-  const Real hR = Real(h);
+  const Real hR = h.h;
   // delta = delta_rel * mean diag(h J M^-1 J^T), formed by the evaluation at this iterate
   const Real delta = w.scal[2];
   // group blocks (full, symmetric) and their coupling rows E_g: a thread per contact row
@@ -1108,9 +1105,9 @@ template <class Real> __device__ __forceinline__ Real dot2col(const Real* T, int
 //   F_g = E_g L_g^-T (coupled separator rows; stored in H),
 //   Lsi = L_s^-1 with L_s L_s^T = S - sum_g F_g F_g^T, the reduced separator (stored in S,
 //   packed).
-template <class Real> __device__ void factor(const DevScene& sc, WS<Real>& w, double h) {
+template <class Real> __device__ void factor(const KScene<Real>& sc, WS<Real>& w, const StepH<Real>& h) {
   const int tid = threadIdx.x, nth = blockDim.x, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
-  const Real hR = Real(h);
+  const Real hR = h.h;
   const int pg = sc.pg, ss = sc.ss, ldg = sc.ldg, cm = sc.cmax, gstr = tri_size(pg);
   const int rb = pg > ss ? pg : ss;
   // Li_g in place: up to four teams (half-warps for CTAs of up to 64 threads, else warps)
@@ -1154,7 +1151,7 @@ template <class Real> __device__ void factor(const DevScene& sc, WS<Real>& w, do
 }
 
 // v <- A^-1 v with the inverse-form block-arrowhead factor (row-parallel phases)
-template <class Real> __device__ void arrow_solve(const DevScene& sc, WS<Real>& w, Real* v) {
+template <class Real> __device__ void arrow_solve(const KScene<Real>& sc, WS<Real>& w, Real* v) {
   const int tid = threadIdx.x, nth = blockDim.x;
   const int gstr = tri_size(sc.pg), ss = sc.ss, ldg = sc.ldg, cm = sc.cmax, mc = w.ints[1];
   Real* y = w.tmp;
@@ -1205,7 +1202,7 @@ template <class Real> __device__ void arrow_solve(const DevScene& sc, WS<Real>& 
 }
 
 // out_b = sum over rows touching body b of J_row,b^T x_row  (6 per body)
-template <class Real> __device__ void jt_apply(const DevScene& sc, WS<Real>& w, const Real* x, Real* out) {
+template <class Real> __device__ void jt_apply(const KScene<Real>& sc, WS<Real>& w, const Real* x, Real* out) {
   const int ssd = sc.ss > 0 ? sc.ss : 1;
   for (int b = threadIdx.x; b < sc.nb; b += blockDim.x) {
     Real jt[6] = {0, 0, 0, 0, 0, 0};
@@ -1223,7 +1220,7 @@ template <class Real> __device__ void jt_apply(const DevScene& sc, WS<Real>& w, 
 }
 
 // compensated variant of jt_apply (exact products, exact partial sums)
-template <class Real> __device__ void jt_apply_acc(const DevScene& sc, WS<Real>& w, const Real* x, Real* out) {
+template <class Real> __device__ void jt_apply_acc(const KScene<Real>& sc, WS<Real>& w, const Real* x, Real* out) {
   const int ssd = sc.ss > 0 ? sc.ss : 1;
   for (int b = threadIdx.x; b < sc.nb; b += blockDim.x) {
     acc2<Real> jt[6];
@@ -1241,9 +1238,9 @@ template <class Real> __device__ void jt_apply_acc(const DevScene& sc, WS<Real>&
 }
 
 // M^-1 v per body (6 per body)
-template <class Real> __device__ __forceinline__ void minv6(const DevScene& sc, const WS<Real>& w, int b, const Real* v,
+template <class Real> __device__ __forceinline__ void minv6(const KScene<Real>& sc, const WS<Real>& w, int b, const Real* v,
                                                             Real* o) {
-  Real mi = Real(1) / Real(sc.mass[b]);
+  Real mi = sc.minv[b];
   o[0] = v[0] * mi; o[1] = v[1] * mi; o[2] = v[2] * mi;
   vec3<Real> a = mat3<Real>(w.Iwi + 9 * b, v3(v[3], v[4], v[5]));
   o[3] = a.x; o[4] = a.y; o[5] = a.z;
@@ -1254,10 +1251,10 @@ template <class Real> __device__ __forceinline__ void minv6(const DevScene& sc, 
 // (+ the radial friction blocks) is formed matrix-free from J.  b is kept in `b`,
 // the solution is returned in `x`; t6 (6 per body) and r (rows) are scratch.
 template <class Real>
-__device__ void schur_solve(const DevScene& sc, WS<Real>& w, const Real* b, Real* x, Real* t6, Real* r, double h,
+__device__ void schur_solve(const KScene<Real>& sc, WS<Real>& w, const Real* b, Real* x, Real* t6, Real* r, const StepH<Real>& h,
                             int sweeps, Real stop_rel = Real(0)) {
   const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0];
-  const Real hR = Real(h);
+  const Real hR = h.h;
   // pass -1 solves for x itself (its correction from x = 0 is A^-1 b), so that one inlined
   // copy of the arrowhead solve serves the first solve and the sweeps
   for (int i = tid; i < m; i += nth) { x[i] = Real(0); r[i] = b[i]; }
@@ -1319,7 +1316,7 @@ __device__ void schur_solve(const DevScene& sc, WS<Real>& w, const Real* b, Real
 // products and compensated sums throughout (the adjoint's solve).  Returns this thread's
 // part of v . out; the caller reduces it (the rows are written by their owning threads).
 template <class Real, bool ACC>
-__device__ Real schur_apply(const DevScene& sc, WS<Real>& w, const Real* v, Real* out, Real* t6, double h) {
+__device__ Real schur_apply(const KScene<Real>& sc, WS<Real>& w, const Real* v, Real* out, Real* t6, const StepH<Real>& h) {
   const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0];
   const int ssd = sc.ss > 0 ? sc.ss : 1;
   for (int task = tid; task < 6 * sc.nb; task += nth) {
@@ -1341,7 +1338,7 @@ __device__ Real schur_apply(const DevScene& sc, WS<Real>& w, const Real* v, Real
     t6[task] = ACC ? ca.value() : acc;
   }
   __syncthreads();
-  const Real hR = Real(h), delta = w.scal[2];
+  const Real hR = h.h, delta = w.scal[2];
   Real part = Real(0);
   for (int i = tid; i < m; i += nth) {
     const Real* Ji = w.J + 12 * i;
@@ -1384,9 +1381,9 @@ __device__ Real schur_apply(const DevScene& sc, WS<Real>& w, const Real* v, Real
 }
 
 // Jacobi preconditioner: the inverse diagonal of A, stored per row by the row's thread
-template <class Real> __device__ void pcr_jacobi(const DevScene& sc, WS<Real>& w, double h) {
+template <class Real> __device__ void pcr_jacobi(const KScene<Real>& sc, WS<Real>& w, const StepH<Real>& h) {
   const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0];
-  const Real hR = Real(h), delta = w.scal[2];
+  const Real hR = h.h, delta = w.scal[2];
   Real* pd = w.pcr + 6 * sc.m_max;
   for (int i = tid; i < m; i += nth) {
     const Real* Ji = w.J + 12 * i;
@@ -1400,7 +1397,7 @@ template <class Real> __device__ void pcr_jacobi(const DevScene& sc, WS<Real>& w
 
 // Block-Jacobi preconditioner: each contact group's block and the (unreduced) separator
 // block of A, as assembled, factored in place to their inverse Cholesky factors (G, S)
-template <class Real> __device__ void factor_blocks(const DevScene& sc, WS<Real>& w) {
+template <class Real> __device__ void factor_blocks(const KScene<Real>& sc, WS<Real>& w) {
   const int tid = threadIdx.x, nth = blockDim.x, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
   const int pg = sc.pg, ss = sc.ss, gstr = tri_size(pg), rb = pg > ss ? pg : ss;
   if (nth <= 64) {
@@ -1417,7 +1414,7 @@ template <class Real> __device__ void factor_blocks(const DevScene& sc, WS<Real>
 // out = P v.  Jacobi: per row, by the row's thread (no synchronisation).  Block Jacobi:
 // L^-T L^-1 v per block (reads other rows of v: synchronises on entry and between the two
 // triangular products); out is written by the rows' threads.
-template <class Real> __device__ void pcr_precond(const DevScene& sc, WS<Real>& w, const Real* v, Real* out) {
+template <class Real> __device__ void pcr_precond(const KScene<Real>& sc, WS<Real>& w, const Real* v, Real* out) {
   const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0], mc = w.ints[1];
   if (sc.pc == PC_JACOBI) {
     const Real* pd = w.pcr + 6 * sc.m_max;
@@ -1466,8 +1463,8 @@ template <class Real> __device__ void pcr_precond(const DevScene& sc, WS<Real>& 
 // decision is taken on block-reduced values, so all threads leave together.  t6: 6 nb
 // scratch.  Returns the iterations taken.
 template <class Real, bool ACC>
-__device__ int pcr_solve(const DevScene& sc, WS<Real>& w, const Real* b, Real* x, int iters, Real rtol, Real* t6,
-                         double h, int* conv) {
+__device__ int pcr_solve(const KScene<Real>& sc, WS<Real>& w, const Real* b, Real* x, int iters, Real rtol, Real* t6,
+                         const StepH<Real>& h, int* conv) {
   const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0], M = sc.m_max;
   Real *r = w.pcr, *z = r + M, *p = z + M, *Ap = p + M, *Az = Ap + M, *q = Az + M;
   Real bb = Real(0);
@@ -1518,8 +1515,8 @@ __device__ int pcr_solve(const DevScene& sc, WS<Real>& w, const Real* b, Real* x
 // reaches.  dx, rt: m-row scratch.  Returns the PCR iterations; *conv = 1 when either
 // stopping test was met.
 template <class Real>
-__device__ int pcr_solve_refined(const DevScene& sc, WS<Real>& w, const Real* b, Real* x, int iters, Real rtol,
-                                 Real* t6, Real* dx, Real* rt, double h, int* conv) {
+__device__ int pcr_solve_refined(const KScene<Real>& sc, WS<Real>& w, const Real* b, Real* x, int iters, Real rtol,
+                                 Real* t6, Real* dx, Real* rt, const StepH<Real>& h, int* conv) {
   const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0];
   const Real floor = sizeof(Real) == 4 ? Real(1e-4) : Real(0);
   const Real ulp = sizeof(Real) == 4 ? Real(1.1920929e-7) : Real(2.220446049250313e-16);
@@ -1565,20 +1562,52 @@ __device__ int pcr_solve_refined(const DevScene& sc, WS<Real>& w, const Real* b,
 // ---------------------------------------------------------------------------
 // forward step kernel
 // ---------------------------------------------------------------------------
-// The scene lives in shared memory during a launch: kernels index its per-body and
-// per-row tables with thread-dependent indices, which the constant (parameter) cache
-// would serialise across a warp.
-__device__ __forceinline__ void scene_to_shared(const DevScene& src, DevScene& dst) {
-  const int* s = reinterpret_cast<const int*>(&src);
-  int* d = reinterpret_cast<int*>(&dst);
-  for (int i = threadIdx.x; i < (int)(sizeof(DevScene) / sizeof(int)); i += blockDim.x) d[i] = s[i];
+// The scene lives in shared memory during a launch, in working precision: kernels index its
+// per-body and per-row tables with thread-dependent indices, which the constant (parameter)
+// cache would serialise across a warp.
+template <class Real> __device__ __forceinline__ void scene_to_shared(const DevScene& src, double h, KScene<Real>& dst) {
+  const SceneLayout& sl = src;
+  SceneLayout& dl = dst;
+  const int* s = reinterpret_cast<const int*>(&sl);
+  int* d = reinterpret_cast<int*>(&dl);
+  const int tid = threadIdx.x, nth = blockDim.x;
+  for (int i = tid; i < (int)(sizeof(SceneLayout) / sizeof(int)); i += nth) d[i] = s[i];
+  for (int b = tid; b < src.nb; b += nth) {
+    dst.mass[b] = Real(src.mass[b]);
+    dst.minv[b] = Real(1) / dst.mass[b];
+    dst.radius[b] = Real(src.radius[b]);
+    dst.hw[b] = Real(src.hw[b]);
+    for (int k = 0; k < 3; ++k) {
+      dst.inertia[b][k] = Real(src.inertia[b][k]);
+      dst.iinv[b][k] = Real(1) / dst.inertia[b][k];
+      dst.half[b][k] = Real(src.half[b][k]);
+    }
+  }
+  for (int j = nth - 1 - tid; j < src.nj; j += nth) {   // from the last thread, beside the bodies
+    for (int k = 0; k < 3; ++k) {
+      dst.ap[j][k] = Real(src.ap[j][k]); dst.ac[j][k] = Real(src.ac[j][k]);
+      dst.axp[j][k] = Real(src.axp[j][k]); dst.axc[j][k] = Real(src.axc[j][k]);
+      dst.p1[j][k] = Real(src.p1[j][k]); dst.p2[j][k] = Real(src.p2[j][k]);
+    }
+    // servo compliance alpha of Eq. (8): 1/kp (velocity target), 1/(kd + h kp) (position)
+    dst.alpha[j] = Real(src.smode[j] == SERVO_POSITION ? 1.0 / (src.kd[j] + h * src.kp[j]) : 1.0 / src.kp[j]);
+  }
+  if (tid == 0) {
+    dst.mu = Real(src.mu); dst.g = Real(src.g);
+    for (int i = 0; i < 5; ++i) dst.box[i] = Real(src.box[i]);
+    dst.hsp = Real(src.hsp); dst.hox = Real(src.hox); dst.hoy = Real(src.hoy);
+    dst.tol = Real(src.tol); dst.delta_rel = Real(src.delta_rel); dst.kappa = Real(src.kappa);
+    dst.eps = Real(src.eps); dst.margin = Real(src.margin); dst.pcr_rtol_adj = Real(src.pcr_rtol_adj);
+    dst.hs.h = Real(h); dst.hs.hh = Real(0.5 * h);
+    dst.heights = src.heights;
+  }
   __syncthreads();
 }
 
 // One world's step; `item` is the launch's work index (the CTA index of a one-CTA-per-
 // world launch, or the index a persistent CTA took from the queue).
 template <class Real>
-__device__ __forceinline__ void step_world(const DevScene& sc, WS<Real>& w, const StepArgs& a, int item) {
+__device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, const StepArgs& a, int item) {
   const int tid = threadIdx.x, nth = blockDim.x;
   const int world = a.list ? a.list[item] : a.world0 + item;
   if (world < 0 || world >= a.n_worlds) return;
@@ -1592,7 +1621,7 @@ __device__ __forceinline__ void step_world(const DevScene& sc, WS<Real>& w, cons
   const int ld = a.ld, nb = sc.nb;
   const Real* sin = reinterpret_cast<const Real*>(a.state_in);
   const Real* ctl = reinterpret_cast<const Real*>(a.controls);
-  const double h = a.h;
+  const StepH<Real> h = sc.hs;
   // this world's inputs (structure of arrays, world index fastest)
   Src<Real> sq = {sin + world, (size_t)ld}, su = {sin + (size_t)7 * nb * ld + world, (size_t)ld};
   Src<Real> sb = {ctl ? ctl + world : sin, ctl ? (size_t)ld : (size_t)0};
@@ -1609,7 +1638,7 @@ __device__ __forceinline__ void step_world(const DevScene& sc, WS<Real>& w, cons
   Real merit = Real(0);
   Real best = Real(INFINITY);
   int best_k = -1, k = 0, conv = 0;
-  const Real tol2 = Real(sc.tol) * Real(sc.tol);
+  const Real tol2 = sc.tol * sc.tol;
   const int n_alpha = sc.ls ? 4 : 1;
   // phase 0: the warm start; 1: a Newton trial; 2: the returned iterate when it is not the
   // last one evaluated (the best iterate from k_min on, or the NaN iterate)
@@ -1714,7 +1743,7 @@ __device__ __forceinline__ void step_world(const DevScene& sc, WS<Real>& w, cons
     __syncthreads();
     for (int b = tid; b < nb; b += nth) {
       Real t[6];
-      for (int q = 0; q < 6; ++q) t[q] = Real(h) * w.du[6 * b + q] - w.rdyn[6 * b + q];
+      for (int q = 0; q < 6; ++q) t[q] = h.h * w.du[6 * b + q] - w.rdyn[6 * b + q];
       minv6(sc, w, b, t, w.du + 6 * b);
     }
     __syncthreads();
@@ -1765,7 +1794,7 @@ __device__ __forceinline__ void step_world(const DevScene& sc, WS<Real>& w, cons
   for (int i = tid; i < m; i += nth) {
     int li = w.meta[4 * i + 3];
     so[(size_t)(13 * nb + li) * ld + world] = w.lk[i];
-    if (imp) imp[(size_t)li * ld + world] = Real(h) * w.lk[i];
+    if (imp) imp[(size_t)li * ld + world] = h.h * w.lk[i];
   }
   if (a.ids)
     for (int sl = tid; sl < sc.n_slots; sl += nth) a.ids[(size_t)sl * ld + world] = w.sact[sl] ? w.sid[sl] : -1;
@@ -1784,8 +1813,8 @@ __device__ __forceinline__ void step_world(const DevScene& sc, WS<Real>& w, cons
 template <class Real>
 __global__ void __launch_bounds__(128, 3) step_kernel(const DevScene scp, const StepArgs a) {
   extern __shared__ __align__(16) char smem[];
-  __shared__ __align__(16) DevScene ssc;
-  scene_to_shared(scp, ssc);
+  __shared__ __align__(16) KScene<Real> ssc;
+  scene_to_shared(scp, a.h, ssc);
   WS<Real> w = ws_carve<Real>(smem, ssc);
   if (!a.queue) {
     step_world<Real>(ssc, w, a, blockIdx.x);
@@ -1833,7 +1862,7 @@ static __global__ void lpt_order_kernel(const int32_t* cost, int n, int32_t* ord
 // ---------------------------------------------------------------------------
 // Body part of Psi: g_q . q+(q-) + w_u . (M(q-)(u* - u-) - h f(q-, u-)), along (b, dc).
 template <class Real>
-__device__ Real body_vjp(const DevScene& sc, const WS<Real>& w, int b, int dc, const Real* gq, const Real* wu, double h) {
+__device__ Real body_vjp(const KScene<Real>& sc, const WS<Real>& w, int b, int dc, const Real* gq, const Real* wu, const StepH<Real>& h) {
   typedef dual<Real> D;
   D qm[7], qp[7];
   for (int c = 0; c < 7; ++c) qm[c] = D(w.qm[7 * b + c], c == dc ? Real(1) : Real(0));
@@ -1848,12 +1877,12 @@ __device__ Real body_vjp(const DevScene& sc, const WS<Real>& w, int b, int dc, c
     // R^T v via rotating by the conjugate quaternion
     D qc[4] = {qm[3], D(Real(0)) - qm[4], D(Real(0)) - qm[5], D(Real(0)) - qm[6]};
     vb = qrot(qc, v);
-    vb = v3(vb.x * D(Real(sc.inertia[b][0])), vb.y * D(Real(sc.inertia[b][1])), vb.z * D(Real(sc.inertia[b][2])));
+    vb = v3(vb.x * D(sc.inertia[b][0]), vb.y * D(sc.inertia[b][1]), vb.z * D(sc.inertia[b][2]));
     return qrot(qm + 3, vb);
   };
   vec3<D> Idw = Iw_apply(dw);
   vec3<D> gy = cross3(om, Iw_apply(om));        // f_ang = -gy
-  vec3<D> ra = Idw + scale(gy, D(Real(h)));     // angular r_dyn minus the lambda terms
+  vec3<D> ra = Idw + scale(gy, D(h.h));     // angular r_dyn minus the lambda terms
   acc = acc + D(wu[6 * b + 3]) * ra.x + D(wu[6 * b + 4]) * ra.y + D(wu[6 * b + 5]) * ra.z;
   return acc.d;
 }
@@ -1866,22 +1895,22 @@ namespace ost {
 template <class Real, int MODE>
 __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, const AdjArgs a) {
   extern __shared__ __align__(16) char smem[];
-  __shared__ __align__(16) DevScene ssc;
+  __shared__ __align__(16) KScene<Real> ssc;
   __shared__ int bgl[NB_CAP * GROUPS_PER_BODY], bgn[NB_CAP], item0[NB_CAP + 1];
   __shared__ int ncon[NB_CAP], jpre[NB_CAP + 1], cpre[NB_CAP + 1];
-  scene_to_shared(scp, ssc);
-  const DevScene& sc = ssc;
+  scene_to_shared(scp, a.h, ssc);
+  const KScene<Real>& sc = ssc;
   WS<Real> w = ws_carve<Real>(smem, sc);
   ExWS<Real> ex = {};
-  if (MODE == ADJ_EXACT) ex = ex_carve<Real>(smem + ws_bytes<Real>(sc), sc);
+  if (MODE == ADJ_EXACT) ex = ex_carve<Real>(smem + ws_layout_bytes<Real>(sc), sc);
   const int tid = threadIdx.x, nth = blockDim.x;
   const int world = a.list ? a.list[blockIdx.x] : a.world0 + blockIdx.x;
   if (world < 0 || world >= a.n_worlds) return;
   const int slot = a.list ? (a.list_slot ? a.list_slot[blockIdx.x] : -1) : 0;
   if (slot < 0 || (a.list && slot >= a.tape_slots)) return;
   const int ld = a.ld, nb = sc.nb;
-  const double h = a.h;
-  const Real hR = Real(h);
+  const StepH<Real> h = sc.hs;
+  const Real hR = h.h;
   const TapeLayout tl = tape_layout(sc);
   const Real* tp = reinterpret_cast<const Real*>(a.tape) + ((size_t)slot * a.n_worlds + world) * tl.total;
   if (sc.lin == LIN_DIRECT) {
@@ -1981,7 +2010,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
     } else {
       // a single PCR solve with the forward pass's operator and preconditioner (Sec. III-D)
       int pconv = 0;
-      const int its = pcr_solve_refined<Real>(sc, w, w.rhs, wl, sc.pcr_iters_adj, Real(sc.pcr_rtol_adj), w.f, w.lt,
+      const int its = pcr_solve_refined<Real>(sc, w, w.rhs, wl, sc.pcr_iters_adj, sc.pcr_rtol_adj, w.f, w.lt,
                                               w.tmp2, h, &pconv);
       if (tid == 0 && a.krylov) a.krylov[world] = its | (pconv ? 0 : (1 << 16));
     }
@@ -2005,7 +2034,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
     for (int i = tid; i < m; i += nth) ex.r[6 * nb + i] = Real(0);
     __syncthreads();
     Real msum = Real(0);
-    for (int b = 0; b < nb; ++b) msum += Real(sc.mass[b]);
+    for (int b = 0; b < nb; ++b) msum += sc.mass[b];
     const Real sigma = msum / (Real(nb) * hR);
     int conv = 0;
     const int its = exact_gmres(sc, w, ex, h, sigma, Real(sizeof(Real) == 4 ? 1e-6 : 1e-13), &conv);
@@ -2027,7 +2056,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
     for (int i = mc + 5 * sc.nj + tid; i < m; i += nth) {
       // d alpha / d k_p: -1/k_p^2 (velocity target), -h/(k_d + h k_p)^2 (position target)
       const int j = w.ref[i];
-      const Real al = Real(servo_alpha(sc, j, h));
+      const Real al = sc.alpha[j];
       const Real dal = sc.smode[j] == SERVO_POSITION ? -hR * al * al : -al * al;
       dkp[(size_t)(i - mc - 5 * sc.nj) * ld + world] = wl[i] * w.lk[i] * dal;
     }
@@ -2037,7 +2066,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
     for (int b = tid; b < nb; b += nth) {
       Real acc = 0;
       for (int k = 0; k < 3; ++k) acc += wu[6 * b + k] * (w.uk[6 * b + k] - w.um[6 * b + k]);
-      acc += wu[6 * b + 2] * (-hR * Real(sc.g));
+      acc += wu[6 * b + 2] * (-hR * sc.g);
       dm[(size_t)b * ld + world] = acc;
     }
   }
@@ -2069,7 +2098,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
         contact_group<Real, Real>(sc, w, sl, b, w.qm + 7 * b, w.uk + 6 * b, h, g);
         D rf[2];
         friction_rows<D, Real>(sc, D(g.vel[1]), D(g.vel[2]), D(w.lk[i]), w.lk[i + 1], w.lk[i + 2],
-                               hR * w.swhat[sl], D(Real(sc.mu), Real(1)), rf);
+                               hR * w.swhat[sl], D(sc.mu, Real(1)), rf);
         part += wl[i + 1] * rf[0].d + wl[i + 2] * rf[1].d;
       }
     }
@@ -2079,7 +2108,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
   // dL/du- = -M w_u - h (df/du-)^T w_u ;  dL/dubar = -w_lambda of the servo rows
   Real* dout = reinterpret_cast<Real*>(a.dL_dstate);
   for (int b = tid; b < nb; b += nth) {
-    Real mb = Real(sc.mass[b]);
+    Real mb = sc.mass[b];
     for (int c = 0; c < 3; ++c) dout[(size_t)(7 * nb + 6 * b + c) * ld + world] = -mb * wu[6 * b + c];
     vec3<Real> wa = v3(wu[6 * b + 3], wu[6 * b + 4], wu[6 * b + 5]);
     vec3<Real> om = v3(w.um[6 * b + 3], w.um[6 * b + 4], w.um[6 * b + 5]);

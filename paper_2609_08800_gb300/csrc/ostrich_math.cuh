@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
+#include "ostrich_scene.h"
 
 namespace ost {
 
@@ -41,6 +42,13 @@ template <class T> __device__ __forceinline__ dual<T> ssqrt(dual<T> a) {
 // correctly rounded square root and quotient in FP64
 __device__ __forceinline__ float pivot_rsqrt(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double pivot_rsqrt(double x) { return 1.0 / sqrt(x); }
+// x < 0.9 and x <= 1e-12, the bounds being the real numbers: in FP32 0.9 rounds down to its
+// nearest float below, so x < 0.9 holds for the floats up to that one; likewise 1e-12
+__device__ __forceinline__ bool below_09(float x) { return x <= 0.9f; }
+__device__ __forceinline__ bool below_09(double x) { return x < 0.9; }
+static_assert((double)0.9f < 0.9 && (double)1e-12f < 1e-12, "the float bounds round down");
+__device__ __forceinline__ bool upto_1em12(float x) { return x <= 1e-12f; }
+__device__ __forceinline__ bool upto_1em12(double x) { return x <= 1e-12; }
 __device__ __forceinline__ float sval(float x) { return x; }
 __device__ __forceinline__ double sval(double x) { return x; }
 template <class T> __device__ __forceinline__ T sval(dual<T> x) { return x.v; }
@@ -92,11 +100,11 @@ template <class S, class M> __device__ __forceinline__ vec3<S> mat3T(const M* R,
 }
 
 // Backward-Euler position update of one body, Eq. (1): p + h v, quat + h/2 (0, w) (x) quat.
-template <class S, class U> __device__ __forceinline__ void kin_body(const S* qm, const U* u, double h, S* qp) {
-  qp[0] = qm[0] + S(h) * u[0];
-  qp[1] = qm[1] + S(h) * u[1];
-  qp[2] = qm[2] + S(h) * u[2];
-  S hh = S(0.5 * h);
+template <class S, class U, class R> __device__ __forceinline__ void kin_body(const S* qm, const U* u, const StepH<R>& h, S* qp) {
+  qp[0] = qm[0] + S(h.h) * u[0];
+  qp[1] = qm[1] + S(h.h) * u[1];
+  qp[2] = qm[2] + S(h.h) * u[2];
+  S hh = S(h.hh);
   S wx = S(u[3]), wy = S(u[4]), wz = S(u[5]);
   S qw = qm[3], qx = qm[4], qy = qm[5], qz = qm[6];
   qp[3] = qw - hh * (wx * qx + wy * qy + wz * qz);
@@ -112,8 +120,8 @@ template <class S, class U> __device__ __forceinline__ void kin_body(const S* qm
 template <class T> struct MapE {
   vec3<T> wk;
   T hh, inv;
-  __device__ __forceinline__ MapE(vec3<T> w, double h) : wk(w) {
-    hh = T(0.5 * h);
+  template <class R> __device__ __forceinline__ MapE(vec3<T> w, const StepH<R>& h) : wk(w) {
+    hh = T(h.hh);
     const T den = T(1) + hh * hh * (wk.x * wk.x + wk.y * wk.y + wk.z * wk.z);
     inv = T(1) / den;
   }
@@ -127,7 +135,7 @@ template <class T> struct MapE {
     return v3((v.x + c.x * hh) * inv, (v.y + c.y * hh) * inv, (v.z + c.z * hh) * inv);
   }
 };
-template <class S, class T> __device__ __forceinline__ vec3<S> map_Et(vec3<S> a, vec3<T> wk, double h) {
+template <class S, class T, class R> __device__ __forceinline__ vec3<S> map_Et(vec3<S> a, vec3<T> wk, const StepH<R>& h) {
   return MapE<T>(wk, h)(a);
 }
 

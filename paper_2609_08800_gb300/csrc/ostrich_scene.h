@@ -18,34 +18,25 @@ enum { SERVO_VELOCITY = 0, SERVO_POSITION = 1 };
 enum { LIN_DIRECT = 0, LIN_PCR = 1 };     // Schur solve: block-arrowhead factor / PCR
 enum { PC_JACOBI = 0, PC_BLOCK = 1 };     // PCR preconditioner
 
-// Everything a kernel needs to know about the scene and the solver settings.
-// Passed by value as a kernel parameter.
-struct DevScene {
+// Integer part of a scene: counts, tables and the layout derived from them.
+struct SceneLayout {
   int nb, nj, n_servo, n_slots, m_max, n_state, env, nf;
-  double mu, g;
-  double box[5];                 // x0, x1, y0, y1, H
-  int hn; double hsp, hox, hoy;  // heightmap grid
-  const float* heights;          // device pointer, hn*hn, or null
+  int hn;                        // heightmap grid points per side
   // bodies
-  double mass[NB_CAP], inertia[NB_CAP][3], half[NB_CAP][3], radius[NB_CAP], hw[NB_CAP];
   int shape[NB_CAP], slot_base[NB_CAP], slot_count[NB_CAP];
   unsigned char slot_body[SLOT_CAP];
   // joints
   int jp[NJ_CAP], jc[NJ_CAP], servo_of[NJ_CAP];
-  double ap[NJ_CAP][3], ac[NJ_CAP][3], axp[NJ_CAP][3], axc[NJ_CAP][3], p1[NJ_CAP][3], p2[NJ_CAP][3], kp[NJ_CAP];
-  double kd[NJ_CAP];
   int jtype[NJ_CAP];   // JOINT_REVOLUTE / JOINT_PRISMATIC
   int smode[NJ_CAP];   // SERVO_VELOCITY / SERVO_POSITION
   // solver settings
   int budget, kmin, ls, pullback;
-  double tol, delta_rel, kappa, eps, margin;
   int refine;     // iterative-refinement sweeps after each forward (Newton-step) Schur solve
   int refine_adj; // iterative-refinement sweeps after the adjoint's Schur solve
   // linear solver of Eq. (12): LIN_DIRECT, or LIN_PCR (matrix-free preconditioned conjugate
   // residual with preconditioner pc; pcr_iters iterations per Newton step; the adjoint's
   // solve stops at |r| <= pcr_rtol_adj |b| or after pcr_iters_adj iterations)
   int lin, pc, pcr_iters, pcr_iters_adj;
-  double pcr_rtol_adj;
   // layout caps derived from the scene
   int n_groups;   // bodies that carry contact slots (leaf blocks of the Schur matrix)
   int pg;         // largest leaf block (3 x slots of one body)
@@ -60,6 +51,38 @@ struct DevScene {
   unsigned char sep_n[SEP_CAP], sep_g[SEP_CAP][2], sep_k[SEP_CAP][2];
 };
 
+// Everything a kernel needs to know about the scene and the solver settings, passed by
+// value as a kernel parameter.  The physical values are doubles here; a launch turns them
+// once into its own precision (KScene).
+struct DevScene : SceneLayout {
+  double mu, g;
+  double box[5];                 // x0, x1, y0, y1, H
+  double hsp, hox, hoy;          // heightmap grid
+  const float* heights;          // device pointer, hn*hn, or null
+  double mass[NB_CAP], inertia[NB_CAP][3], half[NB_CAP][3], radius[NB_CAP], hw[NB_CAP];
+  double ap[NJ_CAP][3], ac[NJ_CAP][3], axp[NJ_CAP][3], axc[NJ_CAP][3], p1[NJ_CAP][3], p2[NJ_CAP][3], kp[NJ_CAP];
+  double kd[NJ_CAP];
+  double tol, delta_rel, kappa, eps, margin;
+  double pcr_rtol_adj;
+};
+
+// The time step and half of it in working precision.
+template <class Real> struct StepH { Real h, hh; };
+
+// The scene of one launch in working precision, in shared memory: the layout, the physical
+// values rounded to Real, and the quotients that the kernels would otherwise form again for
+// every row (1/m, 1/I, the servo compliance).  On this chip a double-precision operation or
+// conversion costs tens of cycles, so none is left on the FP32 kernels' path.
+template <class Real> struct KScene : SceneLayout {
+  Real mu, g, box[5], hsp, hox, hoy;
+  Real mass[NB_CAP], minv[NB_CAP], inertia[NB_CAP][3], iinv[NB_CAP][3], half[NB_CAP][3], radius[NB_CAP], hw[NB_CAP];
+  Real ap[NJ_CAP][3], ac[NJ_CAP][3], axp[NJ_CAP][3], axc[NJ_CAP][3], p1[NJ_CAP][3], p2[NJ_CAP][3];
+  Real alpha[NJ_CAP];            // servo compliance of Eq. (8)
+  Real tol, delta_rel, kappa, eps, margin, pcr_rtol_adj;
+  StepH<Real> hs;
+  const float* heights;
+};
+
 // Packed lower-triangular storage of the symmetric Schur blocks and their inverse
 // factors: element (i, j), j <= i, of an n x n block sits at tri(i, j); a block takes
 // tri_size(n) entries and its row i is contiguous.
@@ -67,7 +90,7 @@ __host__ __device__ inline int tri(int i, int j) { return ((i * (i + 1)) >> 1) +
 __host__ __device__ inline int tri_size(int n) { return (n * (n + 1)) >> 1; }
 
 // Derived layout of a filled scene: groups, block sizes, the static coupling lists.
-inline void finish_scene(DevScene& s) {
+inline void finish_scene(SceneLayout& s) {
   s.n_groups = 0; s.pg = 0;
   for (int b = 0; b < s.nb; ++b)
     if (s.slot_count[b] > 0) {
@@ -141,7 +164,7 @@ struct TapeLayout {
 };
 constexpr int CT_PER_SLOT = 9;   // active, id, feature type (bit-exact), normal (3), offset, edge (2)
 
-inline __host__ __device__ TapeLayout tape_layout(const DevScene& s) {
+inline __host__ __device__ TapeLayout tape_layout(const SceneLayout& s) {
   TapeLayout t;
   int o = 0;
   t.off_qm = o; o += 7 * s.nb;
