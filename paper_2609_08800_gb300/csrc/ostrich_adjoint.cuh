@@ -177,9 +177,9 @@ template <class Real> struct ExWS {
 
 template <class Real> __host__ __device__ inline int ex_n(const SceneLayout& s) { return 6 * s.nb + s.m_max; }
 
-template <class Real> __host__ __device__ ExWS<Real> ex_carve(char* base, const SceneLayout& s) {
+template <class Real> __host__ __device__ __forceinline__ ExWS<Real> ex_carve(char* base, const SceneLayout& s, size_t* bytes = nullptr) {
   ExWS<Real> e;
-  char* p = base;
+  Carver p = {base, 0};
   const int nb = s.nb, n = ex_n<Real>(s), ns = s.n_slots > 0 ? s.n_slots : 1;
   e.K = carve<Real>(p, nb * nb * 36);
   e.G = carve<Real>(p, 12 * s.m_max);
@@ -193,13 +193,14 @@ template <class Real> __host__ __device__ ExWS<Real> ex_carve(char* base, const 
   e.t6 = carve<Real>(p, 6 * nb);
   e.wred = carve<Real>(p, 4 * (KRYLOV + 2));
   e.scal = carve<Real>(p, 8);
+  if (bytes) *bytes = p.off;
   return e;
 }
 
-template <class Real> __host__ __device__ size_t ex_bytes(const DevScene& s) {
-  char* base = reinterpret_cast<char*>(uintptr_t(16));
-  ExWS<Real> e = ex_carve<Real>(base, s);
-  return (size_t)(reinterpret_cast<char*>(e.scal + 8) - base);
+template <class Real> size_t ex_bytes(const DevScene& s) {
+  size_t used = 0;
+  ex_carve<Real>(nullptr, s, &used);
+  return used;
 }
 
 // Shared memory of one world in the adjoint kernel of a mode.

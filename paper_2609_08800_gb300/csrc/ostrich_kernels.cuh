@@ -56,18 +56,23 @@ template <class Real> struct WS {
   Real *pcr;      // PCR mode: r, z, p, A p, A z, P A p and the Jacobi diagonal, m_max each
 };
 
-template <class T> __host__ __device__ __forceinline__ T* carve(char*& p, int n) {
-  size_t a = alignof(T) < 8 ? 8 : alignof(T);
-  uintptr_t q = (reinterpret_cast<uintptr_t>(p) + a - 1) & ~(uintptr_t)(a - 1);
-  T* r = reinterpret_cast<T*>(q);
-  p = reinterpret_cast<char*>(q + sizeof(T) * (size_t)(n > 0 ? n : 1));
-  return r;
+// Takes n elements of T from the workspace at base: off is the byte offset of the first
+// free byte.  Pointers stay base + offset (no integer round trip), so that the compiler
+// sees that they point into shared memory and uses its loads, stores and 32-bit addresses.
+struct Carver {
+  char* base;
+  size_t off;
+};
+template <class T> __host__ __device__ __forceinline__ T* carve(Carver& p, int n, size_t align = 8) {
+  const size_t a = alignof(T) < align ? align : alignof(T);
+  const size_t q = (p.off + a - 1) & ~(a - 1);
+  p.off = q + sizeof(T) * (size_t)(n > 0 ? n : 1);
+  return reinterpret_cast<T*>(p.base + q);
 }
 
-
-template <class Real> __host__ __device__ WS<Real> ws_carve(char* base, const SceneLayout& s) {
+template <class Real> __host__ __device__ __forceinline__ WS<Real> ws_carve(char* base, const SceneLayout& s, size_t* bytes = nullptr) {
   WS<Real> w;
-  char* p = base;
+  Carver p = {base, 0};
   int nb = s.nb, m = s.m_max, ns = s.n_slots > 0 ? s.n_slots : 1, ng = s.n_groups > 0 ? s.n_groups : 1;
   int ss = s.ss > 0 ? s.ss : 1, pg = s.pg > 0 ? s.pg : 1;
   w.qm = carve<Real>(p, 7 * nb); w.um = carve<Real>(p, 6 * nb); w.ubar = carve<Real>(p, s.n_servo + 1);
@@ -97,19 +102,17 @@ template <class Real> __host__ __device__ WS<Real> ws_carve(char* base, const Sc
   w.tmp = carve<Real>(p, m); w.tmp2 = carve<Real>(p, m);
   w.red = carve<Real>(p, 64); w.ints = carve<int>(p, 16); w.scal = carve<Real>(p, 8);
   w.pcr = s.lin == LIN_PCR ? carve<Real>(p, 7 * m) : nullptr;
+  if (bytes) *bytes = p.off;
   return w;
 }
 
-// Dynamic shared memory of one world: the carve itself, run from a 16-byte aligned base
-// (the dynamic shared-memory base is 16-byte aligned and carve aligns to 8), rounded up
-// to 16 bytes.
-template <class Real> __host__ __device__ size_t ws_layout_bytes(const SceneLayout& s) {
-  char* base = reinterpret_cast<char*>(uintptr_t(16));
-  WS<Real> w = ws_carve<Real>(base, s);
-  size_t used = (size_t)(reinterpret_cast<char*>(w.pcr ? w.pcr + 7 * s.m_max : w.scal + 8) - base);
+// Dynamic shared memory of one world: what the carve takes from a 16-byte aligned base (the
+// dynamic shared-memory base is), rounded up to 16 bytes.
+template <class Real> __host__ __device__ __forceinline__ size_t ws_layout_bytes(const SceneLayout& s) {
+  size_t used = 0;
+  ws_carve<Real>(nullptr, s, &used);
   return (used + 15) & ~(size_t)15;
 }
-
 template <class Real> size_t ws_bytes(const DevScene& s) { return ws_layout_bytes<Real>(s); }
 
 // deterministic block reduction (fixed tree); result broadcast through w.red[0]
@@ -2238,10 +2241,9 @@ cudaError_t launch_adjoint(const DevScene& sc, const AdjArgs& a, int threads, cu
 // Bytes the carve of one world actually consumes from a 16-byte aligned base; the
 // context refuses a scene for which this exceeds ws_bytes (checked on the host).
 template <class Real> size_t ws_used(const DevScene& s) {
-  alignas(16) static char probe[16];
-  char* base = probe;
-  WS<Real> w = ws_carve<Real>(base, s);
-  return (size_t)(reinterpret_cast<char*>(w.pcr ? w.pcr + 7 * s.m_max : w.scal + 8) - base);
+  size_t used = 0;
+  ws_carve<Real>(nullptr, s, &used);
+  return used;
 }
 
 template cudaError_t launch_step<OST_REAL>(const DevScene&, const StepArgs&, int, cudaStream_t);
