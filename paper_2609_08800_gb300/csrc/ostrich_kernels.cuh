@@ -98,7 +98,10 @@ template <class Real> __host__ __device__ __forceinline__ WS<Real> ws_carve(char
   if (gsz + rest < 14 * m) gsz = 14 * m - rest;
   w.G = carve<Real>(p, gsz); w.E = carve<Real>(p, esz); w.H = carve<Real>(p, ng * cm * ldg);
   w.S = carve<Real>(p, tri_size(ss));
-  w.prow = carve<Real>(p, 4 * (pg > ss ? pg : ss));
+  // exchange rows of the register factors (64 values per warp, at most four warps), or four
+  // columns of a separator beyond 32 rows
+  w.prow = carve<Real>(p, 4 * 64, 16);
+  static_assert(SEP_CAP <= 64, "four columns of a separator fit the exchange buffer");
   w.tmp = carve<Real>(p, m); w.tmp2 = carve<Real>(p, m);
   w.red = carve<Real>(p, 64); w.ints = carve<int>(p, 16); w.scal = carve<Real>(p, 8);
   w.pcr = s.lin == LIN_PCR ? carve<Real>(p, 7 * m) : nullptr;
@@ -889,8 +892,7 @@ template <class Real> __device__ void assemble(const KScene<Real>& sc, WS<Real>&
   __syncthreads();
 }
 
-// L^-1 of an n x n symmetric positive definite block, in place, by a team of threads:
-// one warp (TEAM = 0, __syncwarp) or the whole CTA (TEAM = 1, __syncthreads).  A (packed
+// L^-1 of an n x n symmetric positive definite block, in place, by one warp.  A (packed
 // lower triangle, tri()) holds the block on entry and L^-1 on return, L L^T = A; colbuf
 // holds n values.  Right-looking, one pivot k at a time:
 //   pass 1: column k of L below the pivot goes to colbuf; row k of L^-1 is finished,
@@ -901,38 +903,28 @@ template <class Real> __device__ void assemble(const KScene<Real>& sc, WS<Real>&
 //           read again, to Xt[i][k].
 // Each element of L and of L^-1 receives the same operations in the same order as the
 // sequential column-by-column factor and forward substitution (k, resp. l,
-// ascending), so the result does not depend on the team size.
-template <int TEAM, class Real> __device__ void chol_inv_inplace(Real* A, int n, Real* colbuf) {
-  // TEAM 0: one warp; 1: the whole CTA; 2: one half-warp (16 lanes)
-  const int t = TEAM == 1 ? (int)threadIdx.x : (TEAM == 2 ? (int)(threadIdx.x & 15) : (int)(threadIdx.x & 31));
-  const int T = TEAM == 1 ? (int)blockDim.x : (TEAM == 2 ? 16 : 32);
-  const int cw = TEAM == 2 ? 16 : 32;                         // columns per pass
-  const unsigned half = 0xffffu << (16 * ((threadIdx.x >> 4) & 1));
-  auto team_sync = [&]() {
-    if (TEAM == 1) __syncthreads();
-    else if (TEAM == 2) __syncwarp(half);
-    else __syncwarp();
-  };
+// ascending), so the result does not depend on how the rows are shared out.
+template <class Real> __device__ void chol_inv_inplace(Real* A, int n, Real* colbuf) {
+  const int t = threadIdx.x & 31;
   for (int k = 0; k < n; ++k) {
     const Real akk = A[tri(k, k)];
     const Real inv = pivot_rsqrt(akk > Real(0) ? akk : Real(1e-30));
     const Real xkk = inv;                   // X[k][k], known to every thread
-    for (int e = t; e < n; e += T) {        // the pivot entry itself is left for pass 2
+    for (int e = t; e < n; e += 32) {        // the pivot entry itself is left for pass 2
       if (e > k) colbuf[e] = A[tri(e, k)] * inv;
       else if (e < k) A[tri(k, e)] *= inv;
     }
-    team_sync();
+    __syncwarp();
     if (t == 0) A[tri(k, k)] = xkk;
-    // lanes own columns (j = lane, lane + cw, ...), groups of cw lanes take every nw-th row
-    const int nw = T / cw, lane = t % cw;
-    for (int j = lane; j < n; j += cw) {
+    // lanes own columns (j = t, t + 32, ...)
+    for (int j = t; j < n; j += 32) {
       // per column: the multiplier of l_ik (X[k][j], X[k][k] or l_jk) and whether the
       // entry keeps its value (no branch inside the row loop)
       const Real coef = j < k ? A[tri(k, j)] : (j == k ? xkk : colbuf[j]);
       const bool keep = j != k;
-      int i = (k + 1 > j ? k + 1 : j) + t / cw;
-      for (; i + 3 * nw < n; i += 4 * nw) {             // four independent rows per pass
-        const int i1 = i + nw, i2 = i1 + nw, i3 = i2 + nw;
+      int i = k + 1 > j ? k + 1 : j;
+      for (; i + 3 < n; i += 4) {             // four independent rows per pass
+        const int i1 = i + 1, i2 = i + 2, i3 = i + 3;
         const Real l0 = colbuf[i], l1 = colbuf[i1], l2 = colbuf[i2], l3 = colbuf[i3];
         Real* a0 = A + tri(i, j);
         Real* a1 = A + tri(i1, j);
@@ -942,14 +934,109 @@ template <int TEAM, class Real> __device__ void chol_inv_inplace(Real* A, int n,
         const Real o2 = keep ? *a2 : Real(0), o3 = keep ? *a3 : Real(0);
         *a0 = o0 - l0 * coef; *a1 = o1 - l1 * coef; *a2 = o2 - l2 * coef; *a3 = o3 - l3 * coef;
       }
-      for (; i < n; i += nw) {
+      for (; i < n; ++i) {
         const Real lik = colbuf[i];
         Real* aij = A + tri(i, j);
         const Real old = keep ? *aij : Real(0);
         *aij = old - lik * coef;
       }
     }
-    team_sync();
+    __syncwarp();
+  }
+}
+
+// Rows of a register block updated per uniform test of how many are left
+constexpr int REG_CHUNK = 8;
+
+__device__ __forceinline__ void load_chunk(const float* b, float* v) {
+  const float4 x = reinterpret_cast<const float4*>(b)[0], y = reinterpret_cast<const float4*>(b)[1];
+  v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w; v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+}
+__device__ __forceinline__ void load_chunk(const double* b, double* v) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const double2 x = reinterpret_cast<const double2*>(b)[q];
+    v[2 * q] = x.x; v[2 * q + 1] = x.y;
+  }
+}
+
+// L^-1 of an n x n symmetric positive definite block in place, as chol_inv_inplace, by TW
+// lanes of a warp (32, or 16 with two blocks per warp) with the block in registers:
+// n <= NR <= TW; nmax is the largest n in the warp (its lanes leave the loop together).
+// Lane j holds column j of the symmetric block, later of L^-1: rows k .. n-1 at the k-th
+// pivot, the pivot row always in a[0] (the rows move up by one as they are updated, so
+// that one loop body serves every pivot).  A pivot takes one broadcast of the diagonal,
+// the reciprocal root, one exchange of the pivot row through `buf` (column k of L is row k
+// of the symmetric block times 1/L[k][k], so every lane supplies its own entry) and one
+// fused multiply-add per row; row k of L^-1 is then final and goes to A.  Every entry
+// receives the operations of chol_inv_inplace in the same order.  buf: 2 TW values,
+// 16-byte aligned, the team's own (two halves in turn: one warp barrier per pivot).
+// What bounds it is the pivot's chain (shuffle, reciprocal root, exchange: about 130
+// cycles), not the row updates; the block through shared memory took about 600 cycles
+// per pivot.
+template <int NR, int TW, class Real>
+__device__ __forceinline__ void chol_inv_regs(Real* A, int n, int nmax, Real* buf) {
+  const int lane = threadIdx.x & (TW - 1);
+  Real a[NR];
+#pragma unroll
+  for (int r = 0; r < NR; ++r)
+    a[r] = r < n && lane < n ? A[r >= lane ? tri(r, 0) + lane : tri(lane, 0) + r] : Real(0);
+  Real* row = A;
+  for (int k = 0; k < nmax; ++k) {
+    const Real akk = __shfl_sync(0xffffffffu, a[0], k, TW);
+    const Real inv = pivot_rsqrt(akk > Real(0) ? akk : Real(1e-30));
+    const bool piv = lane == k;
+    const Real c = piv ? inv : a[0] * inv;
+    Real* bk = buf + (k & 1 ? TW : 0);
+    if (lane > k) bk[lane - k - 1] = c;
+    if (lane <= k && k < n) row[lane] = c;
+    row += k + 1;
+    __syncwarp();
+    const int left = nmax - 1 - k;
+#pragma unroll
+    for (int q = 0; q < NR; q += REG_CHUNK)
+      if (q < left) {
+        Real l[REG_CHUNK];
+        load_chunk(bk + q, l);
+#pragma unroll
+        for (int r = 0; r < REG_CHUNK; ++r)
+          if (q + r + 1 < NR) a[q + r] = rn_fma(-l[r], c, piv ? Real(0) : a[q + r + 1]);
+      }
+  }
+}
+
+// The same for a block of any n the whole warp can hold (n <= 32).
+template <class Real> __device__ __forceinline__ void chol_inv_warp(Real* A, int n, Real* buf) {
+  if (n <= 8) chol_inv_regs<8, 32>(A, n, n, buf);
+  else if (n <= 16) chol_inv_regs<16, 32>(A, n, n, buf);
+  else if (n <= 24) chol_inv_regs<24, 32>(A, n, n, buf);
+  else chol_inv_regs<32, 32>(A, n, n, buf);
+}
+
+// The inverse factors of the contact groups' blocks.  Blocks of up to 16 rows (five of a
+// wheel's slots active; a robot on flat ground has 6 rows per wheel) go two to a warp, larger
+// ones one to a warp, and blocks beyond 32 rows through shared memory.
+template <class Real> __device__ __forceinline__ void factor_groups(const KScene<Real>& sc, WS<Real>& w) {
+  const int tid = threadIdx.x, wid = tid >> 5, nw = blockDim.x >> 5;
+  const int ng = sc.n_groups, gstr = tri_size(sc.pg);
+  int big = 0;
+  for (int g = 0; g < ng; ++g) big = w.gn[g] > big ? w.gn[g] : big;
+  if (big <= 16) {
+    const int half = (tid >> 4) & 1;
+    Real* buf = w.prow + 64 * wid + 32 * half;
+    for (int g0 = 2 * wid; g0 < ng; g0 += 2 * nw) {
+      const int g = g0 + half, n = g < ng ? w.gn[g] : 0;
+      const int na = w.gn[g0], nb = g0 + 1 < ng ? w.gn[g0 + 1] : 0, nmax = na > nb ? na : nb;
+      Real* A = w.G + (g < ng ? g : g0) * gstr;
+      if (nmax <= 8) chol_inv_regs<8, 16>(A, n, nmax, buf);
+      else chol_inv_regs<16, 16>(A, n, nmax, buf);
+    }
+  } else {
+    for (int g = wid; g < ng; g += nw) {
+      const int n = w.gn[g];
+      if (n <= 32) chol_inv_warp(w.G + g * gstr, n, w.prow + 64 * wid);
+      else chol_inv_inplace(w.G + g * gstr, n, w.prow + 64 * wid);
+    }
   }
 }
 
@@ -1080,6 +1167,17 @@ template <class Real> __device__ void chol_inv_inplace4(Real* A, int n, Real* co
   if (k < n) chol_round<1>(A, n, k, colbuf);
 }
 
+// L_s^-1 of the separator block in place over S: in one warp's registers up to 32 rows, else
+// by the whole CTA through shared memory.
+template <class Real> __device__ __forceinline__ void factor_separator(const KScene<Real>& sc, WS<Real>& w) {
+  if (sc.ss > 32) {
+    chol_inv_inplace4(w.S, sc.ss, w.prow);
+  } else {
+    if (threadIdx.x < 32) chol_inv_warp(w.S, sc.ss, w.prow);
+    __syncthreads();
+  }
+}
+
 // Two-accumulator dot products (even and odd terms apart, halving the dependent chain):
 // a contiguous one, and one down a column of a packed triangle (element (l, c), l = c0 ..
 // n-1, at tri(l, c), the offset growing by l + 1 per row).
@@ -1109,19 +1207,9 @@ template <class Real> __device__ __forceinline__ Real dot2col(const Real* T, int
 //   Lsi = L_s^-1 with L_s L_s^T = S - sum_g F_g F_g^T, the reduced separator (stored in S,
 //   packed).
 template <class Real> __device__ void factor(const KScene<Real>& sc, WS<Real>& w, const StepH<Real>& h) {
-  const int tid = threadIdx.x, nth = blockDim.x, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
-  const Real hR = h.h;
-  const int pg = sc.pg, ss = sc.ss, ldg = sc.ldg, cm = sc.cmax, gstr = tri_size(pg);
-  const int rb = pg > ss ? pg : ss;
-  // Li_g in place: up to four teams (half-warps for CTAs of up to 64 threads, else warps)
-  // each take their groups
-  if (nth <= 64) {
-    const int team = tid >> 4, nteams = nth >> 4;
-    for (int g = team; g < sc.n_groups; g += nteams)
-      chol_inv_inplace<2>(w.G + g * gstr, w.gn[g], w.prow + team * rb);
-  } else {
-    for (int g = wid; g < sc.n_groups; g += nw) chol_inv_inplace<0>(w.G + g * gstr, w.gn[g], w.prow + (wid & 3) * rb);
-  }
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int ldg = sc.ldg, cm = sc.cmax, gstr = tri_size(sc.pg);
+  factor_groups(sc, w);
   __syncthreads();
   // F_g[k][j] = sum_{l <= j} E_g[k][l] Li_g[j][l]
   for (int g = 0; g < sc.n_groups; ++g) {
@@ -1149,8 +1237,7 @@ template <class Real> __device__ void factor(const KScene<Real>& sc, WS<Real>& w
     }
     __syncthreads();
   }
-  // Lsi = L_s^-1 in place over S, the whole CTA
-  if (ss > 0) chol_inv_inplace4(w.S, ss, w.prow);
+  factor_separator(sc, w);
 }
 
 // v <- A^-1 v with the inverse-form block-arrowhead factor (row-parallel phases)
@@ -1401,17 +1488,9 @@ template <class Real> __device__ void pcr_jacobi(const KScene<Real>& sc, WS<Real
 // Block-Jacobi preconditioner: each contact group's block and the (unreduced) separator
 // block of A, as assembled, factored in place to their inverse Cholesky factors (G, S)
 template <class Real> __device__ void factor_blocks(const KScene<Real>& sc, WS<Real>& w) {
-  const int tid = threadIdx.x, nth = blockDim.x, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
-  const int pg = sc.pg, ss = sc.ss, gstr = tri_size(pg), rb = pg > ss ? pg : ss;
-  if (nth <= 64) {
-    const int team = tid >> 4, nteams = nth >> 4;
-    for (int g = team; g < sc.n_groups; g += nteams)
-      chol_inv_inplace<2>(w.G + g * gstr, w.gn[g], w.prow + team * rb);
-  } else {
-    for (int g = wid; g < sc.n_groups; g += nw) chol_inv_inplace<0>(w.G + g * gstr, w.gn[g], w.prow + (wid & 3) * rb);
-  }
+  factor_groups(sc, w);
   __syncthreads();
-  if (ss > 0) chol_inv_inplace4(w.S, ss, w.prow);
+  factor_separator(sc, w);
 }
 
 // out = P v.  Jacobi: per row, by the row's thread (no synchronisation).  Block Jacobi:
