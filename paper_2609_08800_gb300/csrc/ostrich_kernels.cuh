@@ -34,7 +34,9 @@ template <class Real> struct WS {
   Real *qm, *um, *ubar, *uk, *ut, *ub, *du, *f, *rdyn, *mr, *Iw, *Iwi, *R, *qp;
   Real *sbc;      // per servo: the bias b_c of Eq. (8) (-target, or (x(q-) - target)/h)
   // rows
-  Real *J, *C, *rhat, *r2, *lk, *lt, *lb, *dl, *rhs;
+  // J: 12 per row, both bodies' parts; a contact row touches one body, and the second half
+  // of its row holds Y = M^-1 J^T.  ys: Y of the separator rows, 12 per row.
+  Real *J, *ys, *C, *rhat, *r2, *lk, *lt, *lb, *dl, *rhs;
   int16_t *meta;  // 4 per row: type | sub << 4, b0, b1 (or -1), lam index (state lambda block)
   int16_t *ref;   // slot or joint of the row
   // slots
@@ -82,7 +84,7 @@ template <class Real> __host__ __device__ __forceinline__ WS<Real> ws_carve(char
   w.Iw = carve<Real>(p, 9 * nb); w.Iwi = carve<Real>(p, 9 * nb); w.R = carve<Real>(p, 9 * nb);
   w.qp = carve<Real>(p, 7 * nb);
   w.sbc = carve<Real>(p, s.n_servo + 1);
-  w.J = carve<Real>(p, 12 * m);
+  w.J = carve<Real>(p, 12 * m, 16); w.ys = carve<Real>(p, 12 * ss, 16);
   w.C = carve<Real>(p, m); w.rhat = carve<Real>(p, m); w.r2 = carve<Real>(p, m); w.lk = carve<Real>(p, m);
   w.lt = carve<Real>(p, m); w.lb = carve<Real>(p, m); w.dl = carve<Real>(p, m); w.rhs = carve<Real>(p, m);
   w.meta = carve<int16_t>(p, 4 * m); w.ref = carve<int16_t>(p, m);
@@ -624,20 +626,47 @@ template <class Real> __device__ __forceinline__ Real rowdot(const Real* Ja, int
          Ja[sa + 4] * Yb[sb + 4] + Ja[sa + 5] * Yb[sb + 5];
 }
 
-// y = M^-1 J_i^T for both body blocks of row i: (J_lin / m, Iw^-1 J_ang) per side (zero
-// for a side without a body); the same values Eq. (2)'s M~^-1 gives the row.
-template <class Real> __device__ __forceinline__ void minv_row(const KScene<Real>& sc, const WS<Real>& w, int i, Real* y) {
-  const Real* Jr = w.J + 12 * i;
-  for (int side = 0; side < 2; ++side) {
-    const int b = w.meta[4 * i + 1 + side];
-    Real* ys = y + 6 * side;
-    if (b < 0) { for (int q = 0; q < 6; ++q) ys[q] = Real(0); continue; }
-    const Real* Js = Jr + 6 * side;
-    const Real mi = sc.minv[b];
-    ys[0] = Js[0] * mi; ys[1] = Js[1] * mi; ys[2] = Js[2] * mi;
-    const vec3<Real> ia = mat3<Real>(w.Iwi + 9 * b, v3(Js[3], Js[4], Js[5]));
-    ys[3] = ia.x; ys[4] = ia.y; ys[5] = ia.z;
+// Six consecutive values of a row (rows are 16-byte aligned and 48 or 96 bytes long), two at
+// a time.
+__device__ __forceinline__ void load6(const float* p, float* v) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const float2 x = reinterpret_cast<const float2*>(p)[q];
+    v[2 * q] = x.x; v[2 * q + 1] = x.y;
   }
+}
+__device__ __forceinline__ void load6(const double* p, double* v) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const double2 x = reinterpret_cast<const double2*>(p)[q];
+    v[2 * q] = x.x; v[2 * q + 1] = x.y;
+  }
+}
+__device__ __forceinline__ void store6(float* p, const float* v) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) reinterpret_cast<float2*>(p)[q] = make_float2(v[2 * q], v[2 * q + 1]);
+}
+__device__ __forceinline__ void store6(double* p, const double* v) {
+#pragma unroll
+  for (int q = 0; q < 3; ++q) reinterpret_cast<double2*>(p)[q] = make_double2(v[2 * q], v[2 * q + 1]);
+}
+
+// J part . Y part, both six values in shared memory
+template <class Real> __device__ __forceinline__ Real rowdot6(const Real* J, const Real* Y) {
+  Real a[6], b[6];
+  load6(J, a);
+  load6(Y, b);
+  return rowdot(a, 0, b, 0);
+}
+
+// y = M^-1 J^T of one body's part of a row: (J_lin / m, Iw^-1 J_ang); the values Eq. (2)'s
+// M~^-1 gives the row.
+template <class Real>
+__device__ __forceinline__ void minv_row6(const KScene<Real>& sc, const WS<Real>& w, int b, const Real* Js, Real* ys) {
+  const Real mi = sc.minv[b];
+  ys[0] = Js[0] * mi; ys[1] = Js[1] * mi; ys[2] = Js[2] * mi;
+  const vec3<Real> ia = mat3<Real>(w.Iwi + 9 * b, v3(Js[3], Js[4], Js[5]));
+  ys[3] = ia.x; ys[4] = ia.y; ys[5] = ia.z;
 }
 
 // ---------------------------------------------------------------------------
@@ -678,7 +707,6 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
         vec3<Real> ang = Ek(cross3(lev, dirs[k]));
         Real* Jr = w.J + 12 * (i + k);
         Jr[0] = dirs[k].x; Jr[1] = dirs[k].y; Jr[2] = dirs[k].z; Jr[3] = ang.x; Jr[4] = ang.y; Jr[5] = ang.z;
-        for (int q = 6; q < 12; ++q) Jr[q] = 0;
         vel[k] = dirs[k].x * u[6 * b] + dirs[k].y * u[6 * b + 1] + dirs[k].z * u[6 * b + 2] + ang.x * u[6 * b + 3] +
                  ang.y * u[6 * b + 4] + ang.z * u[6 * b + 5];
       }
@@ -805,16 +833,27 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
     Real mr[6] = {rv[0] * mi, rv[1] * mi, rv[2] * mi, iw.x, iw.y, iw.z};
     for (int k = 0; k < 6; ++k) { w.mr[6 * b + k] = mr[k]; part += mr[k] * mr[k]; }
   }
-  if (dyn)
-    for (int i = tid; i < m; i += nth) part += w.r2[i] * w.r2[i];
-  // with the merit: delta = delta_rel * mean diag(h J M^-1 J^T) of these rows, for the
-  // assembly at this iterate (scal[2])
+  // with the merit: Y = M^-1 J^T of every row and delta = delta_rel * mean diag(h J Y) of
+  // these rows, for the assembly at this iterate (scal[2])
   Real dpart = 0;
   for (int i = tid; i < m; i += nth) {
-    const Real* Ji = w.J + 12 * i;
-    Real Yi[12];
-    minv_row(sc, w, i, Yi);
-    dpart += hR * (rowdot(Ji, 0, Yi, 0) + rowdot(Ji, 6, Yi, 6));
+    if (dyn) part += w.r2[i] * w.r2[i];
+    Real* Ji = w.J + 12 * i;
+    Real Yi[6], Jv[6];
+    load6(Ji, Jv);
+    minv_row6(sc, w, w.meta[4 * i + 1], Jv, Yi);
+    Real d = rowdot(Jv, 0, Yi, 0);
+    if (i < mc) {
+      store6(Ji + 6, Yi);
+    } else {
+      Real* Ys = w.ys + 12 * (i - mc);
+      store6(Ys, Yi);
+      load6(Ji + 6, Jv);
+      minv_row6(sc, w, w.meta[4 * i + 2], Jv, Yi);
+      store6(Ys + 6, Yi);
+      d = d + rowdot(Jv, 0, Yi, 0);
+    }
+    dpart += hR * d;
   }
   block_sum2(w, part, dpart);
   if (tid == 0) w.scal[2] = m > 0 ? sc.delta_rel * dpart / Real(m) : Real(0);
@@ -827,67 +866,69 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
 // ---------------------------------------------------------------------------
 
 
+// Row of the packed lower triangle that entry e lies in.  (8 e + 1 is the square of 2 a + 1
+// at a row's first entry and below the next odd square in it, and below 2^24 here, so the
+// rounded root's integer part is exact.)
+__device__ __forceinline__ int tri_row(int e) { return (int)(0.5f * (sqrtf((float)(8 * e + 1)) - 1.0f)); }
+
+// The group blocks A_g and their coupling rows E_g (two threads per contact row, taking its
+// columns in turn) and the separator block (an entry per thread and turn: its rows are too
+// few and too uneven for a thread each), all from J and Y = M^-1 J^T as the evaluation left
+// them.  Latency is what counts here, one world keeping two warps: with a thread per row,
+// its own Y and all columns after one another this took 9.9 k cycles per Newton iteration of
+// a robot.
 template <class Real> __device__ void assemble(const KScene<Real>& sc, WS<Real>& w, const StepH<Real>& h) {
   const int tid = threadIdx.x, nth = blockDim.x;
-  const int m = w.ints[0], mc = w.ints[1], gstr = tri_size(sc.pg), ss = sc.ss, ldg = sc.ldg;
+  const int mc = w.ints[1], gstr = tri_size(sc.pg), ss = sc.ss, ldg = sc.ldg;
   const Real hR = h.h;
   // delta = delta_rel * mean diag(h J M^-1 J^T), formed by the evaluation at this iterate
   const Real delta = w.scal[2];
-  // group blocks (full, symmetric) and their coupling rows E_g: a thread per contact row
-  for (int r = tid; r < mc; r += nth) {
+  const int par = tid & 1;
+  for (int r = tid >> 1; r < mc; r += nth >> 1) {
     const int g = w.rgrp[r], r0 = w.g0[g], i = r - r0, bg = sc.group_body[g];
-    Real* Gb = w.G + g * gstr;
     const int ti = w.meta[4 * r] & 15, si = w.meta[4 * r] >> 4;
-    Real Yr[12];
-    minv_row(sc, w, r, Yr);
-    // row i of the group block: h J M^-1 J^T for every column, then the diagonal and the
-    // radial terms of the row's own contact (friction rows of one slot are adjacent)
-    Real* Gi = Gb + tri(i, 0);
-    int jj = r0;
-    for (; jj + 1 <= r; jj += 2) {
-      const Real v0 = hR * rowdot(w.J + 12 * jj, 0, Yr, 0);
-      const Real v1 = hR * rowdot(w.J + 12 * (jj + 1), 0, Yr, 0);
-      Gi[jj - r0] = v0;
-      Gi[jj + 1 - r0] = v1;
-    }
-    if (jj <= r) Gi[jj - r0] = hR * rowdot(w.J + 12 * jj, 0, Yr, 0);
-    Real dg = Gi[i] + (w.C[r] + delta);
-    if (ti == ROW_FRIC) {
-      const Real* rd = w.srad + 3 * w.ref[r];
-      if (si == 1) {
-        dg += rd[0];
-      } else {
-        dg += rd[2];
-        Gi[i - 1] += rd[1];
+    Real Yr[6], Jv[6];
+    load6(w.J + 12 * r + 6, Yr);
+    // row i of the group block: h J M^-1 J^T, with the diagonal and the radial terms of the
+    // row's own contact (friction rows of one slot are adjacent)
+    Real* Gi = w.G + g * gstr + tri(i, 0);
+#pragma unroll 2
+    for (int j = par; j <= i; j += 2) {
+      load6(w.J + 12 * (r0 + j), Jv);
+      Real v = rn_mul(hR, rowdot(Jv, 0, Yr, 0));
+      if (j + 1 >= i && (j == i || (ti == ROW_FRIC && si == 2))) {
+        const Real* rd = w.srad + 3 * w.ref[r];
+        if (j == i) {
+          v = rn_add(v, rn_add(w.C[r], delta));
+          if (ti == ROW_FRIC) v = rn_add(v, si == 1 ? rd[0] : rd[2]);
+        } else {
+          v = rn_add(v, rd[1]);
+        }
       }
+      Gi[j] = v;
     }
-    Gi[i] = dg;
-    Real* Eb = w.E + g * sc.cmax * ldg;
-    for (int k = 0; k < sc.cpl_n[g]; ++k) {
-      const int row = mc + sc.cpl_row[g][k];
-      const int side = w.meta[4 * row + 1] == bg ? 0 : 6;
-      Eb[k * ldg + i] = hR * rowdot(w.J + 12 * row, side, Yr, 0);
+    Real* Eb = w.E + g * sc.cmax * ldg + i;
+    const int nc = sc.cpl_n[g];
+#pragma unroll 2
+    for (int k = par; k < nc; k += 2) {
+      const int a = sc.cpl_row[g][k];
+      load6(w.J + 12 * (mc + a) + (sc.sep_b[a][0] == bg ? 0 : 6), Jv);
+      Eb[k * ldg] = hR * rowdot(Jv, 0, Yr, 0);
     }
   }
-  // separator block: a thread per separator row, counted from the last thread so that it
-  // runs beside the contact rows (counted from the first) rather than after them
-  for (int a = nth - 1 - tid; a >= 0 && a < ss; a += nth) {
-    const int i = mc + a;
-    const int ia0 = w.meta[4 * i + 1], ia1 = w.meta[4 * i + 2];
-    Real Yi[12];
-    minv_row(sc, w, i, Yi);
-    for (int b = 0; b <= a; ++b) {
-      const int j = mc + b;
-      const int jb0 = w.meta[4 * j + 1], jb1 = w.meta[4 * j + 2];
-      Real v = 0;
-      if (ia0 == jb0) v += rowdot(w.J + 12 * j, 0, Yi, 0);
-      if (ia0 == jb1) v += rowdot(w.J + 12 * j, 6, Yi, 0);
-      if (ia1 >= 0 && ia1 == jb0) v += rowdot(w.J + 12 * j, 0, Yi, 6);
-      if (ia1 >= 0 && ia1 == jb1) v += rowdot(w.J + 12 * j, 6, Yi, 6);
-      v *= hR;
-      if (a == b) v += w.C[i] + delta;
-      w.S[tri(a, b)] = v;
-    }
+  for (int e = tid; e < tri_size(ss); e += nth) {
+    const int a = tri_row(e), b = e - tri(a, 0);
+    const int ia0 = sc.sep_b[a][0], ia1 = sc.sep_b[a][1], jb0 = sc.sep_b[b][0], jb1 = sc.sep_b[b][1];
+    const Real* Ya = w.ys + 12 * a;
+    const Real* Jb = w.J + 12 * (mc + b);
+    Real v = 0;
+    if (ia0 == jb0) v += rowdot6(Jb, Ya);
+    if (ia0 == jb1) v += rowdot6(Jb + 6, Ya);
+    if (ia1 == jb0) v += rowdot6(Jb, Ya + 6);
+    if (ia1 == jb1) v += rowdot6(Jb + 6, Ya + 6);
+    v = rn_mul(v, hR);
+    if (a == b) v = rn_add(v, rn_add(w.C[mc + a], delta));
+    w.S[e] = v;
   }
   __syncthreads();
 }
@@ -1211,32 +1252,30 @@ template <class Real> __device__ void factor(const KScene<Real>& sc, WS<Real>& w
   const int ldg = sc.ldg, cm = sc.cmax, gstr = tri_size(sc.pg);
   factor_groups(sc, w);
   __syncthreads();
-  // F_g[k][j] = sum_{l <= j} E_g[k][l] Li_g[j][l]
-  for (int g = 0; g < sc.n_groups; ++g) {
-    const int n = w.gn[g], cnt = sc.cpl_n[g] * n;
-    const Real* Lb = w.G + g * gstr;
-    const Real* Eb = w.E + g * cm * ldg;
-    Real* Fb = w.H + g * cm * ldg;
-    for (int e = tid; e < cnt; e += nth) {
-      const int k = e / n, j = e - k * n;
-      Fb[k * ldg + j] = dot2c(Eb + k * ldg, Lb + tri(j, 0), j + 1);
+  // F_g[k][j] = sum_{l <= j} E_g[k][l] Li_g[j][l], two threads per contact row
+  const int mc = w.ints[1];
+  for (int r = tid >> 1; r < mc; r += nth >> 1) {
+    const int g = w.rgrp[r], j = r - w.g0[g], nc = sc.cpl_n[g];
+    const Real* Lj = w.G + g * gstr + tri(j, 0);
+    for (int k = tid & 1; k < nc; k += 2)
+      w.H[(g * cm + k) * ldg + j] = dot2c(w.E + (g * cm + k) * ldg, Lj, j + 1);
+  }
+  __syncthreads();
+  // S' = S - sum_g F_g F_g^T, an entry per thread and turn (the pairs of rows that share a
+  // group; two bodies of one joint may both carry one, then in group order)
+  for (int e = tid; e < tri_size(sc.ss); e += nth) {
+    const int a = tri_row(e), b = e - tri(a, 0), na = sc.sep_n[a], nb2 = sc.sep_n[b];
+    for (int t = 0; t < na; ++t) {
+      // the groups of row a, ascending
+      int pa = t;
+      if (na == 2) pa = (sc.sep_g[a][0] < sc.sep_g[a][1]) == (t == 0) ? 0 : 1;
+      const int g = sc.sep_g[a][pa];
+      for (int pb = 0; pb < nb2; ++pb)
+        if (sc.sep_g[b][pb] == g)
+          w.S[e] -= dot2c(w.H + (g * cm + sc.sep_k[a][pa]) * ldg, w.H + (g * cm + sc.sep_k[b][pb]) * ldg, w.gn[g]);
     }
   }
   __syncthreads();
-  // S' = S - sum_g F_g F_g^T: group by group (a separator row may couple to two groups),
-  // one coupled row pair (k1 >= k2 of the group's coupling list) per thread
-  for (int g = 0; g < sc.n_groups; ++g) {
-    const int nc = sc.cpl_n[g], n = w.gn[g];
-    if (n == 0) continue;                    // no active contact rows: F_g is empty
-    const Real* Fb = w.H + g * cm * ldg;
-    for (int e = tid; e < nc * nc; e += nth) {
-      const int k1 = e / nc, k2 = e - k1 * nc;
-      if (k2 > k1) continue;
-      const int a = sc.cpl_row[g][k1], b = sc.cpl_row[g][k2];
-      w.S[a >= b ? tri(a, b) : tri(b, a)] -= dot2c(Fb + k1 * ldg, Fb + k2 * ldg, n);
-    }
-    __syncthreads();
-  }
   factor_separator(sc, w);
 }
 
@@ -1472,14 +1511,14 @@ __device__ Real schur_apply(const KScene<Real>& sc, WS<Real>& w, const Real* v, 
 
 // Jacobi preconditioner: the inverse diagonal of A, stored per row by the row's thread
 template <class Real> __device__ void pcr_jacobi(const KScene<Real>& sc, WS<Real>& w, const StepH<Real>& h) {
-  const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0];
+  const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0], mc = w.ints[1];
   const Real hR = h.h, delta = w.scal[2];
   Real* pd = w.pcr + 6 * sc.m_max;
   for (int i = tid; i < m; i += nth) {
     const Real* Ji = w.J + 12 * i;
-    Real Yi[12];
-    minv_row(sc, w, i, Yi);
-    Real d = hR * (rowdot(Ji, 0, Yi, 0) + rowdot(Ji, 6, Yi, 6)) + w.C[i] + delta;
+    const Real* Ys = w.ys + 12 * (i - mc);
+    const Real jy = i < mc ? rowdot6(Ji, Ji + 6) : rowdot6(Ji, Ys) + rowdot6(Ji + 6, Ys + 6);
+    Real d = hR * jy + w.C[i] + delta;
     if ((w.meta[4 * i] & 15) == ROW_FRIC) d += w.srad[3 * w.ref[i] + ((w.meta[4 * i] >> 4) == 1 ? 0 : 2)];
     pd[i] = Real(1) / d;
   }

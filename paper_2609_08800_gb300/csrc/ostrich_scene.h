@@ -49,6 +49,7 @@ struct SceneLayout {
   int cpl_n[NB_CAP];
   unsigned char cpl_row[NB_CAP][SEP_CAP];
   unsigned char sep_n[SEP_CAP], sep_g[SEP_CAP][2], sep_k[SEP_CAP][2];
+  unsigned char sep_b[SEP_CAP][2];       // parent and child body of a separator row
 };
 
 // Everything a kernel needs to know about the scene and the solver settings, passed by
@@ -111,6 +112,8 @@ inline void finish_scene(SceneLayout& s) {
     }
     s.sep_n[a] = 0;
     int bodies[2] = {s.jp[j], s.jc[j]};
+    s.sep_b[a][0] = (unsigned char)bodies[0];
+    s.sep_b[a][1] = (unsigned char)bodies[1];
     for (int t = 0; t < 2; ++t) {
       int g = gof[bodies[t]];
       if (g < 0) continue;
