@@ -441,7 +441,6 @@ __device__ void exact_apply(const KScene<Real>& sc, const WS<Real>& w, const ExW
   const Real hR = h.h;
   const Real* vu = v;
   const Real* vl = v + 6 * nb;
-  const int ssd = sc.ss > 0 ? sc.ss : 1;
   for (int task = tid; task < 6 * nb; task += nth) {
     const int b = task / 6, k = task - 6 * b;
     acc2<Real> a;
@@ -452,14 +451,7 @@ __device__ void exact_apply(const KScene<Real>& sc, const WS<Real>& w, const ExW
     for (int bb = 0; bb < nb; ++bb)
       for (int r = 0; r < 6; ++r) a.add_prod(ex.K[(bb * nb + b) * 36 + r * 6 + k], vu[6 * bb + r]);
     // G^T v_lambda over the rows touching body b
-    const int g = w.bgrp[b];
-    if (g >= 0)
-      for (int i = w.g0[g]; i < w.g0[g] + w.gn[g]; ++i) a.add_prod(ex.G[12 * i + k], vl[i]);
-    for (int t = 0; t < w.bsepn[b]; ++t) {
-      const int i = w.bsep[b * ssd + t];
-      const int side = w.meta[4 * i + 1] == b ? 0 : 6;
-      a.add_prod(ex.G[12 * i + side + k], vl[i]);
-    }
+    body_rows(sc, w, b, [&](int off, int i) { a.add_prod(ex.G[off + k], vl[i]); });
     out[task] = a.value();
   }
   for (int i = tid; i < m; i += nth) {
@@ -510,7 +502,7 @@ __device__ void exact_precond(const KScene<Real>& sc, WS<Real>& w, const ExWS<Re
   }
   __syncthreads();
   arrow_solve(sc, w, z + 6 * nb);
-  jt_apply_acc(sc, w, z + 6 * nb, ex.t6);
+  jt_apply<true>(sc, w, z + 6 * nb, ex.t6);
   __syncthreads();
   for (int b = tid; b < nb; b += nth) {
     Real t[6];

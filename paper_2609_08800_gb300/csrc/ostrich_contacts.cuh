@@ -169,9 +169,12 @@ __device__ __forceinline__ bool activate_rim_hm(const KScene<Real>& s, int b, in
   hm_cell(s, rrim_deepest(c, a, r, n0), i, j);
   int k = 0;
   bool over = false;
+#pragma unroll 1
   for (int ii = i - 1; ii <= i + 1; ++ii)
+#pragma unroll 1
     for (int jj = j - 1; jj <= j + 1; ++jj) {
       if (ii < 0 || jj < 0 || ii > s.hn - 2 || jj > s.hn - 2) continue;
+#pragma unroll 1
       for (int tt = 0; tt < 2; ++tt) {
         f3 n; float d;
         hm_face(s, ii, jj, tt, n, d);

@@ -43,7 +43,7 @@ template <class Real> struct WS {
   Real *sn, *sd, *st1, *st2, *swhat, *srad, *sedge;
   int *sact, *srow, *sid, *sftype;
   // per-body row lists
-  int *bgrp, *bsepn, *bsep;
+  int *bgrp, *bsepn, *bsep;   // bsep: offset of the body's part in J << 8 | row
   // groups
   int *g0, *gn;
   int16_t *rgrp;  // group of a contact row
@@ -146,14 +146,10 @@ template <class Real> __device__ void block_sum2(WS<Real>& w, Real& a, Real& b) 
   __syncthreads();
   if (lane == 0) { w.red[wid] = a; w.red[16 + wid] = b; }
   __syncthreads();
-  if (tid == 0) {
-    Real sa = Real(0), sb = Real(0);
-    for (int i = 0; i < nw; ++i) { sa += w.red[i]; sb += w.red[16 + i]; }
-    w.red[32] = sa; w.red[48] = sb;
-  }
-  __syncthreads();
-  a = w.red[32];
-  b = w.red[48];
+  Real sa = Real(0), sb = Real(0);
+  for (int i = 0; i < nw; ++i) { sa += w.red[i]; sb += w.red[16 + i]; }
+  a = sa;
+  b = sb;
 }
 
 // block maximum (every thread gets it), through w.red[33..]
@@ -413,65 +409,64 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
   for (int i = tid; i < 6 * nb; i += nth) w.um[i] = umv.p[i * umv.stride];
   for (int i = tid; i < sc.n_servo; i += nth) w.ubar[i] = ubarv.p[i * ubarv.stride];
   __syncthreads();
-  // contact activation (FP32 predicate) and slot frames in working precision
-  auto store_slot = [&](int sl, int b, int local, const SlotAct& a) {
-    w.sact[sl] = a.active; w.sid[sl] = a.id; w.sftype[sl] = a.ftype;
-    w.sedge[2 * sl] = (Real)a.ex; w.sedge[2 * sl + 1] = (Real)a.ez;
-    vec3<Real> n; Real d;
-    Real ns[3] = {(Real)a.n[0], (Real)a.n[1], (Real)a.n[2]};
-    slot_frame2<Real, Real>(sc, b, local, a.ftype, w.qm + 7 * b, ns, (Real)a.d, w.sedge + 2 * sl, n, d);
-    vec3<Real> t1, t2;
-    tangent_basis(n, t1, t2);
-    w.sn[3 * sl] = n.x; w.sn[3 * sl + 1] = n.y; w.sn[3 * sl + 2] = n.z; w.sd[sl] = d;
-    w.st1[3 * sl] = t1.x; w.st1[3 * sl + 1] = t1.y; w.st1[3 * sl + 2] = t1.z;
-    w.st2[3 * sl] = t2.x; w.st2[3 * sl + 1] = t2.y; w.st2[3 * sl + 2] = t2.z;
-    if (ct_out) {
-      Real* c = ct_out + CT_PER_SLOT * sl;
-      c[0] = tape_from_int(a.active, Real(0)); c[1] = tape_from_int(a.id, Real(0)); c[2] = tape_from_int(a.ftype, Real(0));
-      c[3] = Real(a.n[0]); c[4] = Real(a.n[1]); c[5] = Real(a.n[2]); c[6] = Real(a.d);
-      c[7] = Real(a.ex); c[8] = Real(a.ez);
-    }
-  };
+  // contact activation (FP32 predicate) and slot frames in working precision; an item is one
+  // slot, or on a heightmap one wheel rim, whose candidate faces fill its nf slots in order.
+  // (Rare or long pieces stay loops and single call sites: their code is read once per step
+  // and only pushes the Newton loop's out of the instruction cache.)
   if (tid == 0) w.ints[7] = 0;
   __syncthreads();
-  if (ct_in) {
-    for (int sl = tid; sl < sc.n_slots; sl += nth) {
+  const bool hm = sc.env == ENV_HEIGHTMAP && !ct_in;
+  const int n_rims = hm ? 2 * nb : 0;
+#pragma unroll 1
+  for (int e = tid; e < n_rims + sc.n_slots; e += nth) {
+    SlotAct acts[8];
+    int sl, b, local, cnt = 1;
+    if (e < n_rims) {
+      b = e >> 1;
+      if (sc.shape[b] != SHAPE_WHEEL) continue;
+      local = (e & 1) * sc.nf; cnt = sc.nf;
+      sl = sc.slot_base[b] + local;
+    } else {
+      sl = e - n_rims;
+      b = sc.slot_body[sl];
+      if (hm && sc.shape[b] == SHAPE_WHEEL) continue;
+      local = sl - sc.slot_base[b];
+    }
+    if (ct_in) {
       const Real* c = ct_in + CT_PER_SLOT * sl;
-      SlotAct a;
+      SlotAct& a = acts[0];
       a.active = tape_to_int(c[0]); a.id = tape_to_int(c[1]); a.ftype = tape_to_int(c[2]);
       a.n[0] = (float)c[3]; a.n[1] = (float)c[4]; a.n[2] = (float)c[5]; a.d = (float)c[6];
       a.ex = (float)c[7]; a.ez = (float)c[8];
-      const int b = sc.slot_body[sl];
-      store_slot(sl, b, sl - sc.slot_base[b], a);
-    }
-  } else if (sc.env == ENV_HEIGHTMAP) {
-    // one thread per wheel rim: the rim's candidate faces fill its nf slots in order
-    for (int e = tid; e < 2 * nb; e += nth) {
-      const int b = e >> 1, rim = e & 1;
-      if (sc.shape[b] != SHAPE_WHEEL) continue;
+    } else {
       float q7[7], u6[6];
       for (int k = 0; k < 7; ++k) q7[k] = (float)w.qm[7 * b + k];
       for (int k = 0; k < 6; ++k) u6[k] = (float)w.um[6 * b + k];
-      SlotAct acts[8];
-      if (activate_rim_hm(sc, b, rim, q7, u6, acts)) atomicOr(&w.ints[7], 4);
-      for (int f = 0; f < sc.nf; ++f) store_slot(sc.slot_base[b] + rim * sc.nf + f, b, rim * sc.nf + f, acts[f]);
-    }
-    for (int sl = tid; sl < sc.n_slots; sl += nth)      // box corners (no wheel rim)
-      if (sc.shape[sc.slot_body[sl]] != SHAPE_WHEEL) {
-        int b = sc.slot_body[sl];
-        float q7[7], u6[6];
-        for (int k = 0; k < 7; ++k) q7[k] = (float)w.qm[7 * b + k];
-        for (int k = 0; k < 6; ++k) u6[k] = (float)w.um[6 * b + k];
-        store_slot(sl, b, sl - sc.slot_base[b], activate_slot(sc, b, sl - sc.slot_base[b], q7, u6));
+      if (e < n_rims) {
+        if (activate_rim_hm(sc, b, e & 1, q7, u6, acts)) atomicOr(&w.ints[7], 4);
+      } else {
+        acts[0] = activate_slot(sc, b, local, q7, u6);
       }
-  } else {
-    for (int sl = tid; sl < sc.n_slots; sl += nth) {
-      int b = sc.slot_body[sl];
-      int local = sl - sc.slot_base[b];
-      float q7[7], u6[6];
-      for (int k = 0; k < 7; ++k) q7[k] = (float)w.qm[7 * b + k];
-      for (int k = 0; k < 6; ++k) u6[k] = (float)w.um[6 * b + k];
-      store_slot(sl, b, local, activate_slot(sc, b, local, q7, u6));
+    }
+#pragma unroll 1
+    for (int f = 0; f < cnt; ++f, ++sl, ++local) {
+      const SlotAct a = acts[f];
+      w.sact[sl] = a.active; w.sid[sl] = a.id; w.sftype[sl] = a.ftype;
+      w.sedge[2 * sl] = (Real)a.ex; w.sedge[2 * sl + 1] = (Real)a.ez;
+      vec3<Real> n; Real d;
+      Real ns[3] = {(Real)a.n[0], (Real)a.n[1], (Real)a.n[2]};
+      slot_frame2<Real, Real>(sc, b, local, a.ftype, w.qm + 7 * b, ns, (Real)a.d, w.sedge + 2 * sl, n, d);
+      vec3<Real> t1, t2;
+      tangent_basis(n, t1, t2);
+      w.sn[3 * sl] = n.x; w.sn[3 * sl + 1] = n.y; w.sn[3 * sl + 2] = n.z; w.sd[sl] = d;
+      w.st1[3 * sl] = t1.x; w.st1[3 * sl + 1] = t1.y; w.st1[3 * sl + 2] = t1.z;
+      w.st2[3 * sl] = t2.x; w.st2[3 * sl + 1] = t2.y; w.st2[3 * sl + 2] = t2.z;
+      if (ct_out) {
+        Real* c = ct_out + CT_PER_SLOT * sl;
+        c[0] = tape_from_int(a.active, Real(0)); c[1] = tape_from_int(a.id, Real(0)); c[2] = tape_from_int(a.ftype, Real(0));
+        c[3] = Real(a.n[0]); c[4] = Real(a.n[1]); c[5] = Real(a.n[2]); c[6] = Real(a.d);
+        c[7] = Real(a.ex); c[8] = Real(a.ez);
+      }
     }
   }
   // bodies: world inertia at q-, external force, warm-start velocity
@@ -497,7 +492,7 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
     vec3<Real> dw = mat3<Real>(w.Iwi + 9 * b, v3(w.f[6 * b + 3], w.f[6 * b + 4], w.f[6 * b + 5]));
     w.uk[6 * b] = w.um[6 * b];
     w.uk[6 * b + 1] = w.um[6 * b + 1];
-    w.uk[6 * b + 2] = w.um[6 * b + 2] + h.h * sc.g;
+    w.uk[6 * b + 2] = rn_fma(h.h, sc.g, w.um[6 * b + 2]);
     w.uk[6 * b + 3] = w.um[6 * b + 3] + h.h * dw.x;
     w.uk[6 * b + 4] = w.um[6 * b + 4] + h.h * dw.y;
     w.uk[6 * b + 5] = w.um[6 * b + 5] + h.h * dw.z;
@@ -586,7 +581,8 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
       int cnt = 0;
       for (int a2 = 0; a2 < sc.ss; ++a2) {
         const int j = a2 < 5 * sc.nj ? a2 / 5 : servo_joint(sc, a2 - 5 * sc.nj);
-        if (sc.jp[j] == bb || sc.jc[j] == bb) w.bsep[bb * ssd + cnt++] = mc + a2;
+        if (sc.jp[j] == bb || sc.jc[j] == bb)
+          w.bsep[bb * ssd + cnt++] = (12 * (mc + a2) + (sc.jp[j] == bb ? 0 : 6)) << 8 | (mc + a2);
       }
       w.bsepn[bb] = cnt;
     }
@@ -607,18 +603,18 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
   __syncthreads();
 }
 
-template <class Real> __device__ __forceinline__ void clamp_cone(const KScene<Real>& sc, WS<Real>& w, Real* lam) {
-  // first safeguard of Sec. III-B: |lambda_f| <= mu lambda_n
-  for (int sl = threadIdx.x; sl < sc.n_slots; sl += blockDim.x) {
-    if (!w.sact[sl]) continue;
-    int i = w.srow[sl];
-    Real rad = sc.mu * (lam[i] > Real(0) ? lam[i] : Real(0));
-    Real nn = ssqrt(lam[i + 1] * lam[i + 1] + lam[i + 2] * lam[i + 2]);
-    if (nn > rad) {
-      Real f = nn > Real(0) ? rad / nn : Real(0);
-      lam[i + 1] *= f; lam[i + 2] *= f;
-    }
+// first safeguard of Sec. III-B: |lambda_f| <= mu lambda_n (l: a slot's three multipliers)
+template <class Real> __device__ __forceinline__ void clamp_slot(const KScene<Real>& sc, Real* l) {
+  Real rad = sc.mu * (l[0] > Real(0) ? l[0] : Real(0));
+  Real nn = ssqrt(l[1] * l[1] + l[2] * l[2]);
+  if (nn > rad) {
+    Real f = nn > Real(0) ? rad / nn : Real(0);
+    l[1] *= f; l[2] *= f;
   }
+}
+template <class Real> __device__ __forceinline__ void clamp_cone(const KScene<Real>& sc, WS<Real>& w, Real* lam) {
+  for (int sl = threadIdx.x; sl < sc.n_slots; sl += blockDim.x)
+    if (w.sact[sl]) clamp_slot(sc, lam + w.srow[sl]);
 }
 
 template <class Real> __device__ __forceinline__ Real rowdot(const Real* Ja, int sa, const Real* Yb, int sb) {
@@ -669,6 +665,92 @@ __device__ __forceinline__ void minv_row6(const KScene<Real>& sc, const WS<Real>
   ys[3] = ia.x; ys[4] = ia.y; ys[5] = ia.z;
 }
 
+// The rows touching body b, in row order: its contact group's, then the separator rows of its
+// joints.  f(offset of the body's part of the row in J, row).
+template <class Real, class F>
+__device__ __forceinline__ void body_rows(const KScene<Real>& sc, const WS<Real>& w, int b, F&& f) {
+  const int g = w.bgrp[b], r0 = g >= 0 ? w.g0[g] : 0, n = g >= 0 ? w.gn[g] : 0, tot = n + w.bsepn[b];
+  const int* bs = w.bsep + b * (sc.ss > 0 ? sc.ss : 1) - n;
+#pragma unroll 4
+  for (int t = 0; t < tot; ++t) {
+    const int e = t < n ? (12 * (r0 + t)) << 8 | (r0 + t) : bs[t];
+    f(e >> 8, e & 255);
+  }
+}
+
+// Separator row a at the iterate (u, lam): one of a joint's five position rows (Eq. (3), as
+// joint_rows_each forms them) or a servo row (Eq. (8), as servo_row_geom).  A thread per row:
+// all five by one thread are five copies of the row's code and five times its latency.
+template <class Real>
+__device__ __forceinline__ void sep_row(const KScene<Real>& sc, WS<Real>& w, const Real* u, const Real* lam,
+                                        const StepH<Real>& h, int a, int mc) {
+  const int i = mc + a, j = w.ref[i], bp = sc.sep_b[a][0], bc = sc.sep_b[a][1];
+  const int k = a < 5 * sc.nj ? a - 5 * j : 5;           // row of the joint; 5: its servo
+  const bool rev = sc.jtype[j] == JOINT_REVOLUTE;
+  const vec3<Real> pp = v3(w.qp[7 * bp], w.qp[7 * bp + 1], w.qp[7 * bp + 2]);
+  const vec3<Real> pc = v3(w.qp[7 * bc], w.qp[7 * bc + 1], w.qp[7 * bc + 2]);
+  const MatRot<Real> rotp{w.R + 9 * bp}, rotc{w.R + 9 * bc};
+  const vec3<Real> z = v3(Real(0), Real(0), Real(0));
+  vec3<Real> lp = z, ap, lc = z, ac;       // the child's angular part is -ac where neg
+  Real c = Real(0);
+  const bool neg = k < 5 && (rev || k >= 2);
+  if (k < 5 && k >= (rev ? 3 : 2)) {
+    // alignment (and a prismatic joint's twist lock): b . v
+    const bool first = k == (rev ? 3 : 2);
+    const vec3<Real> b = rotp(cvec<Real>(first ? sc.p1[j] : sc.p2[j]));
+    const vec3<Real> v = rotc(cvec<Real>(!rev && k == 4 ? sc.p1[j] : sc.axc[j]));
+    ap = cross3(b, v);
+    ac = ap;
+    c = dot3(b, v);
+  } else if (k == 5 && rev) {
+    // joint rate: the relative angular velocity about the parent axis
+    ac = rotp(cvec<Real>(sc.axp[j]));
+    ap = scale(ac, Real(-1));
+  } else {
+    const vec3<Real> rp = rotp(cvec<Real>(sc.ap[j])), rc = rotc(cvec<Real>(sc.ac[j]));
+    const vec3<Real> d = (pc + rc) - (pp + rp);
+    if (rev) {
+      // anchor rows by component
+      lp = v3(k == 0 ? Real(1) : Real(0), k == 1 ? Real(1) : Real(0), k == 2 ? Real(1) : Real(0));
+      ap = cross3(rp, lp);
+      lc = scale(lp, Real(-1));
+      ac = cross3(rc, lp);
+      c = Real(0) - (k == 0 ? d.x : k == 1 ? d.y : d.z);
+    } else {
+      // the anchor off the axis along a perpendicular, or the slide rate along the axis
+      const vec3<Real> b = rotp(cvec<Real>(k == 0 ? sc.p1[j] : k == 1 ? sc.p2[j] : sc.axp[j]));
+      lp = scale(b, Real(-1));
+      ap = cross3(b, d + rp);
+      lc = b;
+      ac = cross3(rc, b);
+      c = dot3(b, d);
+    }
+  }
+  const vec3<Real> wp = v3(u[6 * bp + 3], u[6 * bp + 4], u[6 * bp + 5]);
+  const vec3<Real> wc = v3(u[6 * bc + 3], u[6 * bc + 4], u[6 * bc + 5]);
+  const vec3<Real> ap_ = map_Et(ap, wp, h);
+  // E of -ac as (w x ac, -ac): the rounding of the row's other users (joint_rows_each)
+  const MapE<Real> Ec(wc, h);
+  const vec3<Real> x = cross3(neg ? wc : ac, neg ? ac : wc);
+  const vec3<Real> as = neg ? scale(ac, Real(-1)) : ac;
+  const vec3<Real> ac_ = v3((as.x + x.x * Ec.hh) * Ec.inv, (as.y + x.y * Ec.hh) * Ec.inv, (as.z + x.z * Ec.hh) * Ec.inv);
+  const Real Jr[12] = {lp.x, lp.y, lp.z, ap_.x, ap_.y, ap_.z, lc.x, lc.y, lc.z, ac_.x, ac_.y, ac_.z};
+  store6(w.J + 12 * i, Jr);
+  store6(w.J + 12 * i + 6, Jr + 6);
+  Real r, C = Real(0);
+  if (k < 5) {
+    r = c / h.h;
+  } else {
+    // J_c u + alpha lambda_c + b_c
+    Real v = Real(0);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) v = rn_add(v, rn_fma(Jr[q], u[6 * bp + q], rn_mul(Jr[6 + q], u[6 * bc + q])));
+    C = sc.alpha[j];
+    r = v + C * lam[i] + w.sbc[a - 5 * sc.nj];
+  }
+  w.r2[i] = r; w.rhat[i] = r; w.C[i] = C;
+}
+
 // ---------------------------------------------------------------------------
 // one residual / Jacobian evaluation at iterate (u, lam); returns the merit
 // ---------------------------------------------------------------------------
@@ -685,10 +767,9 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
     qmat(w.qp + 7 * b + 3, w.R + 9 * b);
   }
   __syncthreads();
-  const int n_items = sc.n_slots + sc.nj + sc.n_servo;
-  for (int it = tid; it < n_items; it += nth) {
-    if (it < sc.n_slots) {
-      int sl = it;
+  // contact slots from the first thread on, separator rows from the last: they run beside
+  // one another in different warps
+  for (int sl = tid; sl < sc.n_slots; sl += nth) {
       if (!w.sact[sl]) continue;
       int i = w.srow[sl];
       int b = w.meta[4 * i + 1];
@@ -754,62 +835,17 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
       }
       Real e1 = l1 / lfn, e2 = l2 / lfn;
       w.srad[3 * sl] = rho * e1 * e1; w.srad[3 * sl + 1] = rho * e1 * e2; w.srad[3 * sl + 2] = rho * e2 * e2;
-    } else if (it < sc.n_slots + sc.nj) {
-      const int j = it - sc.n_slots;
-      const int i0 = mc + 5 * j;
-      const int bp = sc.jp[j], bc = sc.jc[j];
-      const vec3<Real> wp = v3(u[6 * bp + 3], u[6 * bp + 4], u[6 * bp + 5]);
-      const vec3<Real> wc = v3(u[6 * bc + 3], u[6 * bc + 4], u[6 * bc + 5]);
-      const MapE<Real> Ep(wp, h), Ec(wc, h);
-      joint_rows_each<Real>(sc, j, v3(w.qp[7 * bp], w.qp[7 * bp + 1], w.qp[7 * bp + 2]), MatRot<Real>{w.R + 9 * bp},
-                            v3(w.qp[7 * bc], w.qp[7 * bc + 1], w.qp[7 * bc + 2]), MatRot<Real>{w.R + 9 * bc},
-                            [&](int k, vec3<Real> lp, vec3<Real> ap, vec3<Real> lc, vec3<Real> ac, Real c) {
-        const vec3<Real> ap_ = Ep(ap), ac_ = Ec(ac);
-        const int i = i0 + k;
-        Real* Jr = w.J + 12 * i;
-        Jr[0] = lp.x; Jr[1] = lp.y; Jr[2] = lp.z; Jr[3] = ap_.x; Jr[4] = ap_.y; Jr[5] = ap_.z;
-        Jr[6] = lc.x; Jr[7] = lc.y; Jr[8] = lc.z; Jr[9] = ac_.x; Jr[10] = ac_.y; Jr[11] = ac_.z;
-        w.r2[i] = c / hR; w.rhat[i] = c / hR; w.C[i] = Real(0);
-      });
-    } else {
-      // k-th servo, Eq. (8): J_c u + alpha lambda_c + b_c
-      const int k = it - sc.n_slots - sc.nj;
-      const int j = servo_joint(sc, k);
-      const int i = mc + 5 * sc.nj + k;
-      const int bp = sc.jp[j], bc = sc.jc[j];
-      SRow<Real> sr;
-      servo_row_geom<Real>(sc, j, v3(w.qp[7 * bp], w.qp[7 * bp + 1], w.qp[7 * bp + 2]), MatRot<Real>{w.R + 9 * bp},
-                           v3(w.qp[7 * bc], w.qp[7 * bc + 1], w.qp[7 * bc + 2]), MatRot<Real>{w.R + 9 * bc}, sr);
-      const vec3<Real> wp = v3(u[6 * bp + 3], u[6 * bp + 4], u[6 * bp + 5]);
-      const vec3<Real> wc = v3(u[6 * bc + 3], u[6 * bc + 4], u[6 * bc + 5]);
-      const vec3<Real> ap_ = map_Et(sr.ang_p, wp, h), ac_ = map_Et(sr.ang_c, wc, h);
-      Real* Jr = w.J + 12 * i;
-      Jr[0] = sr.lin_p.x; Jr[1] = sr.lin_p.y; Jr[2] = sr.lin_p.z; Jr[3] = ap_.x; Jr[4] = ap_.y; Jr[5] = ap_.z;
-      Jr[6] = sr.lin_c.x; Jr[7] = sr.lin_c.y; Jr[8] = sr.lin_c.z; Jr[9] = ac_.x; Jr[10] = ac_.y; Jr[11] = ac_.z;
-      Real v = Real(0);
-      for (int q = 0; q < 6; ++q) v += Jr[q] * u[6 * bp + q] + Jr[6 + q] * u[6 * bc + q];
-      const Real alpha = sc.alpha[j];
-      const Real r = v + alpha * lam[i] + w.sbc[k];
-      w.r2[i] = r; w.rhat[i] = r; w.C[i] = alpha;
-    }
   }
+  for (int a = nth - 1 - tid; a < sc.ss; a += nth) sep_row(sc, w, u, lam, h, a, mc);
   __syncthreads();
   if (dyn) {
     // Eq. (10): r_dyn = M (u - u-) - h f - h J^T lambda, per body; merit part |M^-1 r_dyn|^2.
     // The inertia and constraint terms nearly cancel at convergence, so the sum is
     // accumulated with exact products and exact partial sums (acc2).
-    const int ssd = sc.ss > 0 ? sc.ss : 1;
     for (int task = tid; task < 6 * nb; task += nth) {
       const int b = task / 6, k = task - 6 * (task / 6);
       acc2<Real> rd;
-      int g = w.bgrp[b];
-      if (g >= 0)
-        for (int i = w.g0[g]; i < w.g0[g] + w.gn[g]; ++i) rd.add_prod(w.J[12 * i + k], -hR * lam[i]);
-      for (int t = 0; t < w.bsepn[b]; ++t) {
-        int i = w.bsep[b * ssd + t];
-        int side = w.meta[4 * i + 1] == b ? 0 : 6;
-        rd.add_prod(w.J[12 * i + side + k], -hR * lam[i]);
-      }
+      body_rows(sc, w, b, [&](int off, int i) { rd.add_prod(w.J[off + k], -hR * lam[i]); });
       if (k < 3) {
         const Real m_ = sc.mass[b];
         rd.add_prod(m_, u[6 * b + k]);
@@ -1208,38 +1244,56 @@ template <class Real> __device__ void chol_inv_inplace4(Real* A, int n, Real* co
   if (k < n) chol_round<1>(A, n, k, colbuf);
 }
 
-// L_s^-1 of the separator block in place over S: in one warp's registers up to 32 rows, else
-// by the whole CTA through shared memory.
+// L_s^-1 of the separator block in place over S: in one warp's registers up to 32 rows (the
+// CTA's other warps do not join), else by the whole CTA through shared memory.  The caller
+// synchronises.
 template <class Real> __device__ __forceinline__ void factor_separator(const KScene<Real>& sc, WS<Real>& w) {
-  if (sc.ss > 32) {
-    chol_inv_inplace4(w.S, sc.ss, w.prow);
-  } else {
-    if (threadIdx.x < 32) chol_inv_warp(w.S, sc.ss, w.prow);
-    __syncthreads();
-  }
+  if (sc.ss > 32) chol_inv_inplace4(w.S, sc.ss, w.prow);
+  else if (threadIdx.x < 32) chol_inv_warp(w.S, sc.ss, w.prow);
 }
 
 // Two-accumulator dot products (even and odd terms apart, halving the dependent chain):
-// a contiguous one, and one down a column of a packed triangle (element (l, c), l = c0 ..
-// n-1, at tri(l, c), the offset growing by l + 1 per row).
+// a contiguous one, and one down a column of a packed triangle (element (l, c), l = c ..
+// n-1, at tri(l, c)).  Eight terms at a time, the loads of all eight in flight together,
+// terms past the end zero: the vectors are short (6 to 24), and a plain loop waits for
+// shared memory once per pair while its unrolled copies and remainders fill the
+// instruction cache.
 template <class Real> __device__ __forceinline__ Real dot2c(const Real* a, const Real* b, int n) {
   Real s0 = Real(0), s1 = Real(0);
-  int l = 0;
-  for (; l + 1 < n; l += 2) { s0 += a[l] * b[l]; s1 += a[l + 1] * b[l + 1]; }
-  if (l < n) s0 += a[l] * b[l];
-  return s0 + s1;
-}
-template <class Real> __device__ __forceinline__ Real dot2col(const Real* T, int c, int c0, int n, const Real* b) {
-  Real s0 = Real(0), s1 = Real(0);
-  int l = c0, off = tri(c0, c);
-  for (; l + 1 < n; l += 2) {
-    s0 += T[off] * b[l];
-    off += l + 1;
-    s1 += T[off] * b[l + 1];
-    off += l + 2;
+#pragma unroll 1
+  for (int l = 0; l < n; l += 8) {
+    Real x[8], y[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      x[q] = l + q < n ? a[l + q] : Real(0);
+      y[q] = l + q < n ? b[l + q] : Real(0);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; q += 2) {
+      s0 = rn_fma(x[q], y[q], s0);
+      s1 = rn_fma(x[q + 1], y[q + 1], s1);
+    }
   }
-  if (l < n) s0 += T[off] * b[l];
-  return s0 + s1;
+  return rn_add(s0, s1);
+}
+template <class Real> __device__ __forceinline__ Real dot2col(const Real* T, int c, int n, const Real* b) {
+  Real s0 = Real(0), s1 = Real(0);
+#pragma unroll 1
+  for (int l = c; l < n; l += 8) {
+    const Real* Tl = T + tri(l, c);
+    Real x[8], y[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      x[q] = l + q < n ? Tl[q * l + ((q * (q + 1)) >> 1)] : Real(0);
+      y[q] = l + q < n ? b[l + q] : Real(0);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; q += 2) {
+      s0 = rn_fma(x[q], y[q], s0);
+      s1 = rn_fma(x[q + 1], y[q + 1], s1);
+    }
+  }
+  return rn_add(s0, s1);
 }
 
 // Block-arrowhead factorisation kept in inverse form for row-parallel solves:
@@ -1247,7 +1301,8 @@ template <class Real> __device__ __forceinline__ Real dot2col(const Real* T, int
 //   F_g = E_g L_g^-T (coupled separator rows; stored in H),
 //   Lsi = L_s^-1 with L_s L_s^T = S - sum_g F_g F_g^T, the reduced separator (stored in S,
 //   packed).
-template <class Real> __device__ void factor(const KScene<Real>& sc, WS<Real>& w, const StepH<Real>& h) {
+// Here all but the last; factor_separator follows.
+template <class Real> __device__ __forceinline__ void factor_eliminate(const KScene<Real>& sc, WS<Real>& w) {
   const int tid = threadIdx.x, nth = blockDim.x;
   const int ldg = sc.ldg, cm = sc.cmax, gstr = tri_size(sc.pg);
   factor_groups(sc, w);
@@ -1276,93 +1331,96 @@ template <class Real> __device__ void factor(const KScene<Real>& sc, WS<Real>& w
     }
   }
   __syncthreads();
-  factor_separator(sc, w);
 }
 
-// v <- A^-1 v with the inverse-form block-arrowhead factor (row-parallel phases)
-template <class Real> __device__ void arrow_solve(const KScene<Real>& sc, WS<Real>& w, Real* v) {
-  const int tid = threadIdx.x, nth = blockDim.x;
-  const int gstr = tri_size(sc.pg), ss = sc.ss, ldg = sc.ldg, cm = sc.cmax, mc = w.ints[1];
+// v <- A^-1 v with the inverse-form block-arrowhead factor, in three parts.
+// Groups, forward: y_g = Li_g b_g, then the separator's right-hand side
+// b_s' = b_s - sum_g F_g y_g, by the T threads t = 0 .. T-1 that sync() joins (needs no S).
+template <class Real, class Sync>
+__device__ __forceinline__ void arrow_forward(const KScene<Real>& sc, WS<Real>& w, const Real* v, int t, int T,
+                                              Sync&& sync) {
+  const int gstr = tri_size(sc.pg), ldg = sc.ldg, cm = sc.cmax, mc = w.ints[1];
   Real* y = w.tmp;
   Real* z = w.tmp2;
-  // y_g = Li_g b_g
-  for (int r = tid; r < mc; r += nth) {
+  for (int r = t; r < mc; r += T) {
     const int g = w.rgrp[r], r0 = w.g0[g], i = r - r0;
     y[r] = dot2c(w.G + g * gstr + tri(i, 0), v + r0, i + 1);
   }
-  __syncthreads();
-  // b_s' = b_s - sum_g F_g y_g
-  for (int a = tid; a < ss; a += nth) {
+  sync();
+  for (int a = t; a < sc.ss; a += T) {
     Real acc = v[mc + a];
     for (int pa = 0; pa < sc.sep_n[a]; ++pa) {
       const int g = sc.sep_g[a][pa];
-      acc -= dot2c(w.H + g * cm * ldg + sc.sep_k[a][pa] * ldg, y + w.g0[g], w.gn[g]);
+      acc -= dot2c(w.H + (g * cm + sc.sep_k[a][pa]) * ldg, y + w.g0[g], w.gn[g]);
     }
     z[a] = acc;
   }
-  __syncthreads();
-  // y_s = Lsi b_s'
-  for (int a = tid; a < ss; a += nth) y[mc + a] = dot2c(w.S + tri(a, 0), z, a + 1);
-  __syncthreads();
-  // x_s = Lsi^T y_s
-  for (int a = tid; a < ss; a += nth) v[mc + a] = dot2col(w.S, a, a, ss, y + mc);
-  __syncthreads();
-  // r_g = y_g - F_g^T x_s
+}
+
+// Separator, by one warp: y_s = Lsi b_s', x_s = Lsi^T y_s into v.
+template <class Real> __device__ __forceinline__ void arrow_separator(const KScene<Real>& sc, WS<Real>& w, Real* v) {
+  const int lane = threadIdx.x & 31, ss = sc.ss, mc = w.ints[1];
+  Real* y = w.tmp + mc;
+  for (int a = lane; a < ss; a += 32) y[a] = dot2c(w.S + tri(a, 0), w.tmp2, a + 1);
+  __syncwarp();
+  for (int a = lane; a < ss; a += 32) v[mc + a] = dot2col(w.S, a, ss, y);
+}
+
+// Groups, backward, by the whole CTA: x_g = Li_g^T (y_g - F_g^T x_s) into v.
+template <class Real> __device__ __forceinline__ void arrow_backward(const KScene<Real>& sc, WS<Real>& w, Real* v) {
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const int gstr = tri_size(sc.pg), ldg = sc.ldg, cm = sc.cmax, mc = w.ints[1];
+  const Real* y = w.tmp;
+  Real* z = w.tmp2;
   for (int r = tid; r < mc; r += nth) {
-    const int g = w.rgrp[r], i = r - w.g0[g];
-    const Real* Fb = w.H + g * cm * ldg;
+    const int g = w.rgrp[r], i = r - w.g0[g], nc = sc.cpl_n[g];
+    const Real* Fb = w.H + g * cm * ldg + i;
     Real s0 = y[r], s1 = Real(0);
-    const int nc = sc.cpl_n[g];
-    int k = 0;
-    for (; k + 1 < nc; k += 2) {
-      s0 -= Fb[k * ldg + i] * v[mc + sc.cpl_row[g][k]];
-      s1 -= Fb[(k + 1) * ldg + i] * v[mc + sc.cpl_row[g][k + 1]];
+#pragma unroll 1
+    for (int k = 0; k < nc; k += 8) {
+      Real x[8], f[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        x[q] = k + q < nc ? v[mc + sc.cpl_row[g][k + q]] : Real(0);
+        f[q] = k + q < nc ? Fb[(k + q) * ldg] : Real(0);
+      }
+#pragma unroll
+      for (int q = 0; q < 8; q += 2) {
+        s0 = rn_fma(-f[q], x[q], s0);
+        s1 = rn_fma(-f[q + 1], x[q + 1], s1);
+      }
     }
-    if (k < nc) s0 -= Fb[k * ldg + i] * v[mc + sc.cpl_row[g][k]];
-    z[r] = s0 + s1;
+    z[r] = rn_add(s0, s1);
   }
   __syncthreads();
-  // x_g = Li_g^T r_g
   for (int r = tid; r < mc; r += nth) {
-    const int g = w.rgrp[r], r0 = w.g0[g], i = r - r0, n = w.gn[g];
-    v[r] = dot2col(w.G + g * gstr, i, i, n, z + r0);
+    const int g = w.rgrp[r], r0 = w.g0[g], i = r - r0;
+    v[r] = dot2col(w.G + g * gstr, i, w.gn[g], z + r0);
   }
   __syncthreads();
 }
 
-// out_b = sum over rows touching body b of J_row,b^T x_row  (6 per body)
-template <class Real> __device__ void jt_apply(const KScene<Real>& sc, WS<Real>& w, const Real* x, Real* out) {
-  const int ssd = sc.ss > 0 ? sc.ss : 1;
-  for (int b = threadIdx.x; b < sc.nb; b += blockDim.x) {
-    Real jt[6] = {0, 0, 0, 0, 0, 0};
-    int g = w.bgrp[b];
-    if (g >= 0)
-      for (int i = w.g0[g]; i < w.g0[g] + w.gn[g]; ++i)
-        for (int k = 0; k < 6; ++k) jt[k] += w.J[12 * i + k] * x[i];
-    for (int t = 0; t < w.bsepn[b]; ++t) {
-      int i = w.bsep[b * ssd + t];
-      int side = w.meta[4 * i + 1] == b ? 0 : 6;
-      for (int k = 0; k < 6; ++k) jt[k] += w.J[12 * i + side + k] * x[i];
-    }
-    for (int k = 0; k < 6; ++k) out[6 * b + k] = jt[k];
-  }
+template <class Real> __device__ __forceinline__ void arrow_solve(const KScene<Real>& sc, WS<Real>& w, Real* v) {
+  arrow_forward(sc, w, v, threadIdx.x, blockDim.x, [] { __syncthreads(); });
+  __syncthreads();
+  if (threadIdx.x < 32) arrow_separator(sc, w, v);
+  __syncthreads();
+  arrow_backward(sc, w, v);
 }
 
-// compensated variant of jt_apply (exact products, exact partial sums)
-template <class Real> __device__ void jt_apply_acc(const KScene<Real>& sc, WS<Real>& w, const Real* x, Real* out) {
-  const int ssd = sc.ss > 0 ? sc.ss : 1;
-  for (int b = threadIdx.x; b < sc.nb; b += blockDim.x) {
-    acc2<Real> jt[6];
-    int g = w.bgrp[b];
-    if (g >= 0)
-      for (int i = w.g0[g]; i < w.g0[g] + w.gn[g]; ++i)
-        for (int k = 0; k < 6; ++k) jt[k].add_prod(w.J[12 * i + k], x[i]);
-    for (int t = 0; t < w.bsepn[b]; ++t) {
-      int i = w.bsep[b * ssd + t];
-      int side = w.meta[4 * i + 1] == b ? 0 : 6;
-      for (int k = 0; k < 6; ++k) jt[k].add_prod(w.J[12 * i + side + k], x[i]);
-    }
-    for (int k = 0; k < 6; ++k) out[6 * b + k] = jt[k].value();
+// out_b = sum over rows touching body b of J_row,b^T x_row (6 per body), a thread per
+// component; with ACC exact products and exact partial sums.
+template <bool ACC, class Real>
+__device__ __forceinline__ void jt_apply(const KScene<Real>& sc, WS<Real>& w, const Real* x, Real* out) {
+  for (int task = threadIdx.x; task < 6 * sc.nb; task += blockDim.x) {
+    const int b = task / 6, k = task - 6 * (task / 6);
+    acc2<Real> ca;
+    Real acc = Real(0);
+    body_rows(sc, w, b, [&](int off, int i) {
+      if (ACC) ca.add_prod(w.J[off + k], x[i]);
+      else acc += w.J[off + k] * x[i];
+    });
+    out[task] = ACC ? ca.value() : acc;
   }
 }
 
@@ -1391,7 +1449,7 @@ __device__ void schur_solve(const KScene<Real>& sc, WS<Real>& w, const Real* b, 
   const Real delta = w.scal[2];
   for (int sweep = -1; sweep < sweeps; ++sweep) {
     if (sweep >= 0) {
-      jt_apply(sc, w, x, t6);
+      jt_apply<false>(sc, w, x, t6);
       __syncthreads();
       for (int bb = tid; bb < sc.nb; bb += nth) {
         Real o[6];
@@ -1447,25 +1505,7 @@ __device__ void schur_solve(const KScene<Real>& sc, WS<Real>& w, const Real* b, 
 template <class Real, bool ACC>
 __device__ Real schur_apply(const KScene<Real>& sc, WS<Real>& w, const Real* v, Real* out, Real* t6, const StepH<Real>& h) {
   const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0];
-  const int ssd = sc.ss > 0 ? sc.ss : 1;
-  for (int task = tid; task < 6 * sc.nb; task += nth) {
-    const int b = task / 6, k = task - 6 * (task / 6);
-    acc2<Real> ca;
-    Real acc = Real(0);
-    const int g = w.bgrp[b];
-    if (g >= 0)
-      for (int i = w.g0[g]; i < w.g0[g] + w.gn[g]; ++i) {
-        if (ACC) ca.add_prod(w.J[12 * i + k], v[i]);
-        else acc += w.J[12 * i + k] * v[i];
-      }
-    for (int t = 0; t < w.bsepn[b]; ++t) {
-      const int i = w.bsep[b * ssd + t];
-      const Real jv = w.J[12 * i + (w.meta[4 * i + 1] == b ? 0 : 6) + k];
-      if (ACC) ca.add_prod(jv, v[i]);
-      else acc += jv * v[i];
-    }
-    t6[task] = ACC ? ca.value() : acc;
-  }
+  jt_apply<ACC>(sc, w, v, t6);
   __syncthreads();
   const Real hR = h.h, delta = w.scal[2];
   Real part = Real(0);
@@ -1526,10 +1566,11 @@ template <class Real> __device__ void pcr_jacobi(const KScene<Real>& sc, WS<Real
 
 // Block-Jacobi preconditioner: each contact group's block and the (unreduced) separator
 // block of A, as assembled, factored in place to their inverse Cholesky factors (G, S)
-template <class Real> __device__ void factor_blocks(const KScene<Real>& sc, WS<Real>& w) {
+template <class Real> __device__ __forceinline__ void factor_blocks(const KScene<Real>& sc, WS<Real>& w) {
   factor_groups(sc, w);
   __syncthreads();
   factor_separator(sc, w);
+  __syncthreads();
 }
 
 // out = P v.  Jacobi: per row, by the row's thread (no synchronisation).  Block Jacobi:
@@ -1747,7 +1788,7 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
   Src<Real> sq = {sin + world, (size_t)ld}, su = {sin + (size_t)7 * nb * ld + world, (size_t)ld};
   Src<Real> sb = {ctl ? ctl + world : sin, ctl ? (size_t)ld : (size_t)0};
   world_setup<Real>(sc, w, sq, su, sb, h, tpw ? tpw + tl.off_ct : nullptr);
-  const int m = w.ints[0];
+  const int m = w.ints[0], mc = w.ints[1];
   // warm start: lambda from the previous step on the active rows, into the trial buffers;
   // the loop's evaluation takes it as its first trial
   for (int i = tid; i < 6 * nb; i += nth) w.ut[i] = w.uk[i];
@@ -1830,51 +1871,83 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
     if (fin && !(tpw && sc.lin == LIN_DIRECT)) break;
     // Schur step, Eq. (12): (h J M^-1 J^T + C + delta) dl = J M^-1 r_dyn - rhat, by the
     // block-arrowhead factor or by PCR (the preconditioner formed at this iterate)
-    if (sc.lin == LIN_DIRECT) {
+    const bool direct = sc.lin == LIN_DIRECT;
+    if (direct || sc.pc == PC_BLOCK) {
       assemble(sc, w, h);
-      factor(sc, w, h);
-      if (fin) break;
-    } else if (sc.pc == PC_BLOCK) {
-      assemble(sc, w, h);
-      factor_blocks(sc, w);
+      if (direct) {
+        factor_eliminate(sc, w);
+        if (fin) {
+          factor_separator(sc, w);
+          break;
+        }
+      } else {
+        factor_blocks(sc, w);
+      }
     } else {
       pcr_jacobi(sc, w, h);
     }
-    for (int i = tid; i < m; i += nth) {
-      const Real* Ji = w.J + 12 * i;
-      int b0 = w.meta[4 * i + 1], b1 = w.meta[4 * i + 2];
-      acc2<Real> jm;
-      for (int q = 0; q < 6; ++q) jm.add_prod(Ji[q], w.mr[6 * b0 + q]);
-      if (b1 >= 0) for (int q = 0; q < 6; ++q) jm.add_prod(Ji[6 + q], w.mr[6 * b1 + q]);
-      jm.add(-w.rhat[i]);
-      // unrefined direct solve: the right-hand side goes straight to dl, solved in place
-      if (sc.lin == LIN_DIRECT && sc.refine == 0) w.dl[i] = jm.value();
-      else w.rhs[i] = jm.value();
+    // right-hand side J M^-1 r_dyn - rhat.  Direct: by the second warp, with the groups'
+    // forward pass, beside the first warp's factorisation of the separator (neither needs the
+    // other), straight into dl, solved in place.
+    const bool beside = direct && nth > 32 && sc.ss <= 32;
+    Real* rhs = direct ? w.dl : w.rhs;
+    const int t0 = beside ? tid - 32 : tid, T = beside ? 32 : nth;
+    if (beside && tid < 32) factor_separator(sc, w);
+    if (t0 >= 0 && t0 < T) {
+      for (int i = t0; i < m; i += T) {
+        const Real* Ji = w.J + 12 * i;
+        const int b0 = w.meta[4 * i + 1], b1 = w.meta[4 * i + 2];
+        acc2<Real> jm;
+        for (int q = 0; q < 6; ++q) jm.add_prod(Ji[q], w.mr[6 * b0 + q]);
+        if (b1 >= 0) for (int q = 0; q < 6; ++q) jm.add_prod(Ji[6 + q], w.mr[6 * b1 + q]);
+        jm.add(-w.rhat[i]);
+        rhs[i] = jm.value();
+      }
+      if (beside) {
+        __syncwarp();
+        arrow_forward(sc, w, w.dl, t0, T, [] { __syncwarp(); });
+      }
     }
     __syncthreads();
-    if (sc.lin == LIN_DIRECT) {
-      if (sc.refine == 0) arrow_solve(sc, w, w.dl);
-      else schur_solve(sc, w, w.rhs, w.dl, w.du, w.lt, h, sc.refine);
+    if (direct) {
+      if (!beside) {
+        arrow_forward(sc, w, w.dl, tid, nth, [] { __syncthreads(); });
+        factor_separator(sc, w);
+        __syncthreads();
+      }
+      if (tid < 32) arrow_separator(sc, w, w.dl);
+      __syncthreads();
+      arrow_backward(sc, w, w.dl);
     } else {
       int pconv;
       pcr_solve<Real, false>(sc, w, w.rhs, w.dl, sc.pcr_iters, Real(0), w.du, h, &pconv);
     }
-    // Eq. (13): du = M^-1 (h J^T dl - r_dyn)
-    jt_apply(sc, w, w.dl, w.du);
-    __syncthreads();
-    for (int b = tid; b < nb; b += nth) {
-      Real t[6];
-      for (int q = 0; q < 6; ++q) t[q] = h.h * w.du[6 * b + q] - w.rdyn[6 * b + q];
-      minv6(sc, w, b, t, w.du + 6 * b);
+    // Eq. (13): du = M^-1 (h J^T dl - r_dyn), and the full-step trial (mr is free once the
+    // right-hand side is formed)
+    for (int task = tid; task < 6 * nb; task += nth) {
+      const int b = task / 6, k = task - 6 * (task / 6);
+      Real jt = Real(0);
+      body_rows(sc, w, b, [&](int off, int i) { jt += w.J[off + k] * w.dl[i]; });
+      w.mr[task] = h.h * jt - w.rdyn[task];
     }
     __syncthreads();
-    // the full-step trial
     ai = 0;
     alpha = Real(1);
-    for (int i = tid; i < 6 * nb; i += nth) w.ut[i] = w.uk[i] + alpha * w.du[i];
-    for (int i = tid; i < m; i += nth) w.lt[i] = w.lk[i] + alpha * w.dl[i];
-    __syncthreads();
-    clamp_cone(sc, w, w.lt);
+    for (int task = tid; task < 6 * nb; task += nth) {
+      const int b = task / 6, k = task - 6 * (task / 6);
+      const Real* t = w.mr + 6 * b;
+      const Real* Iv = w.Iwi + 9 * b + 3 * (k - 3);
+      const Real d = k < 3 ? t[k] * sc.minv[b] : Iv[0] * t[3] + Iv[1] * t[4] + Iv[2] * t[5];
+      w.du[task] = d;
+      w.ut[task] = w.uk[task] + alpha * d;
+    }
+    for (int i = nth - 1 - tid; i < sc.ss; i += nth) w.lt[mc + i] = w.lk[mc + i] + alpha * w.dl[mc + i];
+    for (int sl = nth - 1 - tid; sl < sc.n_slots; sl += nth) {
+      if (!w.sact[sl]) continue;
+      const int i = w.srow[sl];
+      for (int q = 0; q < 3; ++q) w.lt[i + q] = w.lk[i + q] + alpha * w.dl[i + q];
+      clamp_slot(sc, w.lt + i);
+    }
     __syncthreads();
   }
   if (!(mret == mret) || !(fabs((double)mret) < 1e300)) status |= 2u;
@@ -1937,18 +2010,20 @@ __global__ void __launch_bounds__(128, 3) step_kernel(const DevScene scp, const 
   __shared__ __align__(16) KScene<Real> ssc;
   scene_to_shared(scp, a.h, ssc);
   WS<Real> w = ws_carve<Real>(smem, ssc);
-  if (!a.queue) {
-    step_world<Real>(ssc, w, a, blockIdx.x);
-    return;
-  }
-  // persistent: take work items until the queue is exhausted (no CTA waits on another)
+  // one CTA per world, or persistent: take work items until the queue is exhausted (no CTA
+  // waits on another).  One call site for both: a second inlined copy would double the code.
   for (;;) {
-    __syncthreads();
-    if (threadIdx.x == 0) w.ints[15] = atomicAdd(a.queue, 1);
-    __syncthreads();
-    const int it = w.ints[15];
-    if (it >= a.n_items) break;
-    step_world<Real>(ssc, w, a, a.order ? a.order[it] : it);
+    int it = blockIdx.x;
+    if (a.queue) {
+      __syncthreads();
+      if (threadIdx.x == 0) w.ints[15] = atomicAdd(a.queue, 1);
+      __syncthreads();
+      it = w.ints[15];
+      if (it >= a.n_items) break;
+      if (a.order) it = a.order[it];
+    }
+    step_world<Real>(ssc, w, a, it);
+    if (!a.queue) break;
   }
 }
 
@@ -2072,7 +2147,9 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
     // PCR mode tapes no factor: the exact mode's GMRES preconditioner is the direct factor,
     // formed here at the taped iterate
     assemble(sc, w, h);
-    factor(sc, w, h);
+    factor_eliminate(sc, w);
+    factor_separator(sc, w);
+    __syncthreads();
   } else if (sc.pc == PC_BLOCK) {
     // the PCR operator and preconditioner of the forward pass, at the taped iterate
     assemble(sc, w, h);
@@ -2136,7 +2213,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
       if (tid == 0 && a.krylov) a.krylov[world] = its | (pconv ? 0 : (1 << 16));
     }
     // Eq. (19): w_u = -M^-1 (g + J^T w_lambda)
-    jt_apply_acc(sc, w, wl, w.f);     // f is free now
+    jt_apply<true>(sc, w, wl, w.f);     // f is free now
     __syncthreads();
     for (int b = tid; b < nb; b += nth) {
       Real t[6], o[6];
