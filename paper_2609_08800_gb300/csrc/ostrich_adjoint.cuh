@@ -216,7 +216,7 @@ template <class Real> __device__ void body_groups(const KScene<Real>& sc, const 
   for (int b = 0; b < sc.nb; ++b) {
     int k = 0;
     for (int sl = sc.slot_base[b]; sl < sc.slot_base[b] + sc.slot_count[b]; ++sl)
-      if (w.sact[sl]) bgl[b * GROUPS_PER_BODY + k++] = sl;
+      if (w.srow[sl] >= 0) bgl[b * GROUPS_PER_BODY + k++] = sl;
     for (int j = 0; j < sc.nj; ++j)
       if (sc.jp[j] == b || sc.jc[j] == b) bgl[b * GROUPS_PER_BODY + k++] = sc.n_slots + j;
     bgn[b] = k;
@@ -405,7 +405,7 @@ template <class Real> __device__ void exact_slot_terms(const KScene<Real>& sc, c
   typedef dual<Real> D;
   const Real hR = h.h, eps = sc.eps, kap = sc.kappa;
   for (int sl = threadIdx.x; sl < sc.n_slots; sl += blockDim.x) {
-    if (!w.sact[sl]) continue;
+    if (w.srow[sl] < 0) continue;
     const int i = w.srow[sl], b = sc.slot_body[sl];
     Real u[6], qm[7];
     for (int q = 0; q < 6; ++q) u[q] = w.uk[6 * b + q];
@@ -456,23 +456,23 @@ __device__ void exact_apply(const KScene<Real>& sc, const WS<Real>& w, const ExW
   }
   for (int i = tid; i < m; i += nth) {
     const Real* Ji = w.J + 12 * i;
-    const int b0 = w.meta[4 * i + 1], b1 = w.meta[4 * i + 2];
+    const int b0 = row_b0(w.row[i]), b1 = row_b1(w.row[i]);
     acc2<Real> a;
     for (int q = 0; q < 6; ++q) a.add_prod(-hR * Ji[q], vu[6 * b0 + q]);
     if (b1 >= 0) for (int q = 0; q < 6; ++q) a.add_prod(-hR * Ji[6 + q], vu[6 * b1 + q]);
-    const int t = w.meta[4 * i] & 15, sub = w.meta[4 * i] >> 4;
+    const int t = row_type(w.row[i]), sub = row_sub(w.row[i]);
     // normal rows: d(phi/scl)/dlambda_n = (fa kappa + fb h what)/scl; evaluate() keeps
     // kappa + fb h what/scl, equal unless the scale is clamped (fa < 1e-12)
-    const Real cii = t == ROW_NORMAL ? w.C[i] + (ex.fsc[w.ref[i]] - Real(1)) * sc.kappa : w.C[i];
+    const Real cii = t == ROW_NORMAL ? w.C[i] + (ex.fsc[row_ref(w.row[i])] - Real(1)) * sc.kappa : w.C[i];
     a.add_prod(cii, vl[i]);
     if (t == ROW_FRIC) {
-      const Real* rd = w.srad + 3 * w.ref[i];
+      const Real* rd = w.srad + 3 * row_ref(w.row[i]);
       if (sub == 1) a.add_prod(rd[1], vl[i + 1]);
       else a.add_prod(rd[1], vl[i - 1]);
       a.add_prod(sub == 1 ? rd[0] : rd[2], vl[i]);
     } else if (t == ROW_NORMAL) {
       // column lambda_n of the two friction rows, transposed
-      const int sl = w.ref[i];
+      const int sl = row_ref(w.row[i]);
       a.add_prod(ex.cfn[2 * sl], vl[i + 1]);
       a.add_prod(ex.cfn[2 * sl + 1], vl[i + 2]);
     }
@@ -493,7 +493,7 @@ __device__ void exact_precond(const KScene<Real>& sc, WS<Real>& w, const ExWS<Re
   __syncthreads();
   for (int i = tid; i < m; i += nth) {
     const Real* Ji = w.J + 12 * i;
-    const int b0 = w.meta[4 * i + 1], b1 = w.meta[4 * i + 2];
+    const int b0 = row_b0(w.row[i]), b1 = row_b1(w.row[i]);
     acc2<Real> a;
     for (int q = 0; q < 6; ++q) a.add_prod(hR * Ji[q], w.mr[6 * b0 + q]);
     if (b1 >= 0) for (int q = 0; q < 6; ++q) a.add_prod(hR * Ji[6 + q], w.mr[6 * b1 + q]);

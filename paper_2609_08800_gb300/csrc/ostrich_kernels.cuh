@@ -37,16 +37,16 @@ template <class Real> struct WS {
   // J: 12 per row, both bodies' parts; a contact row touches one body, and the second half
   // of its row holds Y = M^-1 J^T.  ys: Y of the separator rows, 12 per row.
   Real *J, *ys, *C, *rhat, *r2, *lk, *lt, *lb, *dl, *rhs;
-  int16_t *meta;  // 4 per row: type | sub << 4, b0, b1 (or -1), lam index (state lambda block)
-  int16_t *ref;   // slot or joint of the row
+  uint32_t *row;  // what each row is: row_word()
   // slots
   Real *sn, *sd, *st1, *st2, *swhat, *srad, *sedge;
-  int *sact, *srow, *sid, *sftype;
+  int *srow;      // first row of an active slot, -1 of an inactive one
+  int *sid, *sftype;
   // per-body row lists
-  int *bgrp, *bsepn, *bsep;   // bsep: offset of the body's part in J << 8 | row
+  int *bgrp, *bsepn;
+  uint16_t *bsep;   // offsets in J of the body's parts of the separator rows touching it
   // groups
   int *g0, *gn;
-  int16_t *rgrp;  // group of a contact row
   // Schur storage (block-arrowhead, inverse form): G group blocks, E coupling rows,
   // H = E G, S reduced separator; prow a pivot-row buffer per warp
   Real *G, *E, *H, *S, *prow, *tmp, *tmp2;
@@ -72,6 +72,20 @@ template <class T> __host__ __device__ __forceinline__ T* carve(Carver& p, int n
   return reinterpret_cast<T*>(p.base + q);
 }
 
+// Word of a row: its index in the state's lambda block, its bodies (15: none), type, index among
+// its slot's or joint's rows, contact group, and slot or joint.
+__device__ __forceinline__ uint32_t row_word(int lam, int b0, int b1, int type, int sub, int grp, int ref) {
+  return (uint32_t)(lam | b0 << 8 | (b1 & 15) << 12 | type << 16 | sub << 18 | grp << 21 | ref << 24);
+}
+static_assert(5 * NJ_CAP + NJ_CAP + 3 * SLOT_CAP <= 256 && NB_CAP <= 8 && SLOT_CAP <= 256, "a row's word holds these");
+__device__ __forceinline__ int row_lam(uint32_t x) { return x & 255; }
+__device__ __forceinline__ int row_b0(uint32_t x) { return (x >> 8) & 15; }
+__device__ __forceinline__ int row_b1(uint32_t x) { const int b = (x >> 12) & 15; return b == 15 ? -1 : b; }
+__device__ __forceinline__ int row_type(uint32_t x) { return (x >> 16) & 3; }
+__device__ __forceinline__ int row_sub(uint32_t x) { return (x >> 18) & 7; }
+__device__ __forceinline__ int row_grp(uint32_t x) { return (x >> 21) & 7; }
+__device__ __forceinline__ int row_ref(uint32_t x) { return x >> 24; }
+
 template <class Real> __host__ __device__ __forceinline__ WS<Real> ws_carve(char* base, const SceneLayout& s, size_t* bytes = nullptr) {
   WS<Real> w;
   Carver p = {base, 0};
@@ -84,27 +98,36 @@ template <class Real> __host__ __device__ __forceinline__ WS<Real> ws_carve(char
   w.Iw = carve<Real>(p, 9 * nb); w.Iwi = carve<Real>(p, 9 * nb); w.R = carve<Real>(p, 9 * nb);
   w.qp = carve<Real>(p, 7 * nb);
   w.sbc = carve<Real>(p, s.n_servo + 1);
-  w.J = carve<Real>(p, 12 * m, 16); w.ys = carve<Real>(p, 12 * ss, 16);
-  w.C = carve<Real>(p, m); w.rhat = carve<Real>(p, m); w.r2 = carve<Real>(p, m); w.lk = carve<Real>(p, m);
-  w.lt = carve<Real>(p, m); w.lb = carve<Real>(p, m); w.dl = carve<Real>(p, m); w.rhs = carve<Real>(p, m);
-  w.meta = carve<int16_t>(p, 4 * m); w.ref = carve<int16_t>(p, m);
+  w.J = carve<Real>(p, 12 * m, 16);
+  w.C = carve<Real>(p, m); w.rhat = carve<Real>(p, m); w.lk = carve<Real>(p, m); w.lb = carve<Real>(p, m);
+  // r2 is done with once the merit is summed: its place then holds the exchange rows of the
+  // register factors (64 values per warp, at most four warps), or four columns of a
+  // separator beyond 32 rows
+  w.r2 = carve<Real>(p, m > 4 * 64 ? m : 4 * 64, 16);
+  w.prow = w.r2;
+  static_assert(SEP_CAP <= 64, "four columns of a separator fit the exchange buffer");
+  w.row = carve<uint32_t>(p, m);
   w.sn = carve<Real>(p, 3 * ns); w.st1 = carve<Real>(p, 3 * ns); w.st2 = carve<Real>(p, 3 * ns);
   w.srad = carve<Real>(p, 3 * ns); w.sd = carve<Real>(p, ns); w.swhat = carve<Real>(p, ns);
   w.sedge = carve<Real>(p, 2 * ns);
-  w.sact = carve<int>(p, ns); w.srow = carve<int>(p, ns); w.sid = carve<int>(p, ns); w.sftype = carve<int>(p, ns);
-  w.bgrp = carve<int>(p, nb); w.bsepn = carve<int>(p, nb); w.bsep = carve<int>(p, nb * ss);
-  w.g0 = carve<int>(p, ng); w.gn = carve<int>(p, ng); w.rgrp = carve<int16_t>(p, m);
-  int cm = s.cmax > 0 ? s.cmax : 1, ldg = s.ldg > 0 ? s.ldg : 1;
-  int esz = ng * cm * ldg;
-  int gsz = ng * tri_size(pg), rest = esz + ng * cm * ldg + tri_size(ss);
-  if (gsz + rest < 14 * m) gsz = 14 * m - rest;
-  w.G = carve<Real>(p, gsz); w.E = carve<Real>(p, esz); w.H = carve<Real>(p, ng * cm * ldg);
+  w.srow = carve<int>(p, ns); w.sid = carve<int>(p, ns); w.sftype = carve<int>(p, ns);
+  w.bgrp = carve<int>(p, nb); w.bsepn = carve<int>(p, nb); w.bsep = carve<uint16_t>(p, nb * ss);
+  w.g0 = carve<int>(p, ng); w.gn = carve<int>(p, ng);
+  const int cm = s.cmax > 0 ? s.cmax : 1, ldg = s.ldg > 0 ? s.ldg : 1, esz = ng * cm * ldg;
+  // The coupling rows E live from the assembly to F = E L^-T, when the trial multipliers, the
+  // step and the solve's scratch are free: one place for both
+  const size_t e0 = (p.off + 15) & ~(size_t)15;
+  w.lt = carve<Real>(p, m, 16);
+  w.dl = carve<Real>(p, m); w.rhs = carve<Real>(p, m); w.tmp = carve<Real>(p, m); w.tmp2 = carve<Real>(p, m);
+  w.E = w.lt;
+  if (p.off < e0 + sizeof(Real) * (size_t)esz) p.off = e0 + sizeof(Real) * (size_t)esz;
+  // G, H and S in one run (the adjoint keeps up to 14 m pull-back items there).  The separator
+  // rows' Y lives from the evaluation to the assembly, F from the elimination on: one place.
+  const int hsz = esz > 12 * ss ? esz : 12 * ss;
+  int gsz = ng * tri_size(pg);
+  if (gsz + hsz + tri_size(ss) < 14 * m) gsz = 14 * m - hsz - tri_size(ss);
+  w.G = carve<Real>(p, gsz); w.H = carve<Real>(p, hsz, 16); w.ys = w.H;
   w.S = carve<Real>(p, tri_size(ss));
-  // exchange rows of the register factors (64 values per warp, at most four warps), or four
-  // columns of a separator beyond 32 rows
-  w.prow = carve<Real>(p, 4 * 64, 16);
-  static_assert(SEP_CAP <= 64, "four columns of a separator fit the exchange buffer");
-  w.tmp = carve<Real>(p, m); w.tmp2 = carve<Real>(p, m);
   w.red = carve<Real>(p, 64); w.ints = carve<int>(p, 16); w.scal = carve<Real>(p, 8);
   w.pcr = s.lin == LIN_PCR ? carve<Real>(p, 7 * m) : nullptr;
   if (bytes) *bytes = p.off;
@@ -451,7 +474,7 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
 #pragma unroll 1
     for (int f = 0; f < cnt; ++f, ++sl, ++local) {
       const SlotAct a = acts[f];
-      w.sact[sl] = a.active; w.sid[sl] = a.id; w.sftype[sl] = a.ftype;
+      w.srow[sl] = a.active ? 0 : -1; w.sid[sl] = a.id; w.sftype[sl] = a.ftype;
       w.sedge[2 * sl] = (Real)a.ex; w.sedge[2 * sl + 1] = (Real)a.ez;
       vec3<Real> n; Real d;
       Real ns[3] = {(Real)a.n[0], (Real)a.n[1], (Real)a.n[2]};
@@ -517,8 +540,8 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
   // prefix counts, and each lane writes its own slot's rows.
   if (tid < 32) {
     const int lane = tid, ns = sc.n_slots;
-    const unsigned m0 = __ballot_sync(0xffffffffu, lane < ns && w.sact[lane]);
-    const unsigned m1 = __ballot_sync(0xffffffffu, 32 + lane < ns && w.sact[32 + lane]);
+    const unsigned m0 = __ballot_sync(0xffffffffu, lane < ns && w.srow[lane] >= 0);
+    const unsigned m1 = __ballot_sync(0xffffffffu, 32 + lane < ns && w.srow[32 + lane] >= 0);
     const int c0 = __popc(m0);
     for (int c = 0; c < 2; ++c) {
       const int sl = 32 * c + lane;
@@ -533,10 +556,7 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
       while (sc.group_body[gb] != bb) ++gb;
       for (int k = 0; k < 3; ++k) {
         const int r = r0 + k;
-        w.meta[4 * r] = (k == 0 ? ROW_NORMAL : ROW_FRIC) | (k << 4); w.meta[4 * r + 1] = bb; w.meta[4 * r + 2] = -1;
-        w.meta[4 * r + 3] = lam + k;
-        w.ref[r] = sl;
-        w.rgrp[r] = gb;
+        w.row[r] = row_word(lam + k, bb, -1, k == 0 ? ROW_NORMAL : ROW_FRIC, k, gb, sl);
       }
     }
     // groups: first row and row count of each body's slots
@@ -564,12 +584,10 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
       const int r = mc + a;
       if (a < 5 * sc.nj) {
         const int j = a / 5, k = a - 5 * j;
-        w.meta[4 * r] = ROW_JOINT | (k << 4); w.meta[4 * r + 1] = sc.jp[j]; w.meta[4 * r + 2] = sc.jc[j];
-        w.meta[4 * r + 3] = 5 * j + k; w.ref[r] = j;
+        w.row[r] = row_word(5 * j + k, sc.jp[j], sc.jc[j], ROW_JOINT, k, 0, j);
       } else {
         const int j = servo_joint(sc, a - 5 * sc.nj);
-        w.meta[4 * r] = ROW_SERVO; w.meta[4 * r + 1] = sc.jp[j]; w.meta[4 * r + 2] = sc.jc[j];
-        w.meta[4 * r + 3] = 5 * sc.nj + sc.servo_of[j]; w.ref[r] = j;
+        w.row[r] = row_word(5 * sc.nj + sc.servo_of[j], sc.jp[j], sc.jc[j], ROW_SERVO, 0, 0, j);
       }
     }
     // per-body lists: its group and the separator rows that touch it, in row order
@@ -582,7 +600,7 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
       for (int a2 = 0; a2 < sc.ss; ++a2) {
         const int j = a2 < 5 * sc.nj ? a2 / 5 : servo_joint(sc, a2 - 5 * sc.nj);
         if (sc.jp[j] == bb || sc.jc[j] == bb)
-          w.bsep[bb * ssd + cnt++] = (12 * (mc + a2) + (sc.jp[j] == bb ? 0 : 6)) << 8 | (mc + a2);
+          w.bsep[bb * ssd + cnt++] = (uint16_t)(12 * (mc + a2) + (sc.jp[j] == bb ? 0 : 6));
       }
       w.bsepn[bb] = cnt;
     }
@@ -590,8 +608,8 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
   __syncthreads();
   // normal-row scaling what = J_n M^-1 J_n^T at q- (geometric Jacobian, E = I)
   for (int sl = tid; sl < sc.n_slots; sl += nth) {
-    if (!w.sact[sl]) { w.swhat[sl] = 0; continue; }
-    int b = w.meta[4 * w.srow[sl] + 1];
+    if (w.srow[sl] < 0) { w.swhat[sl] = 0; continue; }
+    int b = sc.slot_body[sl];
     int local = sl - sc.slot_base[b];
     vec3<Real> n = v3(w.sn[3 * sl], w.sn[3 * sl + 1], w.sn[3 * sl + 2]);
     vec3<Real> p = v3(w.qm[7 * b], w.qm[7 * b + 1], w.qm[7 * b + 2]);
@@ -614,7 +632,7 @@ template <class Real> __device__ __forceinline__ void clamp_slot(const KScene<Re
 }
 template <class Real> __device__ __forceinline__ void clamp_cone(const KScene<Real>& sc, WS<Real>& w, Real* lam) {
   for (int sl = threadIdx.x; sl < sc.n_slots; sl += blockDim.x)
-    if (w.sact[sl]) clamp_slot(sc, lam + w.srow[sl]);
+    if (w.srow[sl] >= 0) clamp_slot(sc, lam + w.srow[sl]);
 }
 
 template <class Real> __device__ __forceinline__ Real rowdot(const Real* Ja, int sa, const Real* Yb, int sb) {
@@ -670,11 +688,11 @@ __device__ __forceinline__ void minv_row6(const KScene<Real>& sc, const WS<Real>
 template <class Real, class F>
 __device__ __forceinline__ void body_rows(const KScene<Real>& sc, const WS<Real>& w, int b, F&& f) {
   const int g = w.bgrp[b], r0 = g >= 0 ? w.g0[g] : 0, n = g >= 0 ? w.gn[g] : 0, tot = n + w.bsepn[b];
-  const int* bs = w.bsep + b * (sc.ss > 0 ? sc.ss : 1) - n;
+  const uint16_t* bs = w.bsep + b * (sc.ss > 0 ? sc.ss : 1) - n;
 #pragma unroll 4
   for (int t = 0; t < tot; ++t) {
-    const int e = t < n ? (12 * (r0 + t)) << 8 | (r0 + t) : bs[t];
-    f(e >> 8, e & 255);
+    const unsigned off = t < n ? 12 * (r0 + t) : bs[t];
+    f((int)off, (int)(off / 12u));
   }
 }
 
@@ -684,7 +702,7 @@ __device__ __forceinline__ void body_rows(const KScene<Real>& sc, const WS<Real>
 template <class Real>
 __device__ __forceinline__ void sep_row(const KScene<Real>& sc, WS<Real>& w, const Real* u, const Real* lam,
                                         const StepH<Real>& h, int a, int mc) {
-  const int i = mc + a, j = w.ref[i], bp = sc.sep_b[a][0], bc = sc.sep_b[a][1];
+  const int i = mc + a, j = row_ref(w.row[i]), bp = sc.sep_b[a][0], bc = sc.sep_b[a][1];
   const int k = a < 5 * sc.nj ? a - 5 * j : 5;           // row of the joint; 5: its servo
   const bool rev = sc.jtype[j] == JOINT_REVOLUTE;
   const vec3<Real> pp = v3(w.qp[7 * bp], w.qp[7 * bp + 1], w.qp[7 * bp + 2]);
@@ -770,9 +788,9 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
   // contact slots from the first thread on, separator rows from the last: they run beside
   // one another in different warps
   for (int sl = tid; sl < sc.n_slots; sl += nth) {
-      if (!w.sact[sl]) continue;
+      if (w.srow[sl] < 0) continue;
       int i = w.srow[sl];
-      int b = w.meta[4 * i + 1];
+      int b = sc.slot_body[sl];
       int local = sl - sc.slot_base[b];
       vec3<Real> p = v3(w.qp[7 * b], w.qp[7 * b + 1], w.qp[7 * b + 2]);
       vec3<Real> n = v3(w.sn[3 * sl], w.sn[3 * sl + 1], w.sn[3 * sl + 2]);
@@ -877,16 +895,18 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
     Real* Ji = w.J + 12 * i;
     Real Yi[6], Jv[6];
     load6(Ji, Jv);
-    minv_row6(sc, w, w.meta[4 * i + 1], Jv, Yi);
+    minv_row6(sc, w, row_b0(w.row[i]), Jv, Yi);
     Real d = rowdot(Jv, 0, Yi, 0);
     if (i < mc) {
       store6(Ji + 6, Yi);
     } else {
+      // (the direct adjoint, dyn = false, needs no Y, and its F is on its way to that place)
       Real* Ys = w.ys + 12 * (i - mc);
-      store6(Ys, Yi);
+      const bool keep = dyn || sc.lin == LIN_PCR;
+      if (keep) store6(Ys, Yi);
       load6(Ji + 6, Jv);
-      minv_row6(sc, w, w.meta[4 * i + 2], Jv, Yi);
-      store6(Ys + 6, Yi);
+      minv_row6(sc, w, row_b1(w.row[i]), Jv, Yi);
+      if (keep) store6(Ys + 6, Yi);
       d = d + rowdot(Jv, 0, Yi, 0);
     }
     dpart += hR * d;
@@ -907,64 +927,133 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
 // rounded root's integer part is exact.)
 __device__ __forceinline__ int tri_row(int e) { return (int)(0.5f * (sqrtf((float)(8 * e + 1)) - 1.0f)); }
 
-// The group blocks A_g and their coupling rows E_g (two threads per contact row, taking its
-// columns in turn) and the separator block (an entry per thread and turn: its rows are too
-// few and too uneven for a thread each), all from J and Y = M^-1 J^T as the evaluation left
-// them.  Latency is what counts here, one world keeping two warps: with a thread per row,
-// its own Y and all columns after one another this took 9.9 k cycles per Newton iteration of
-// a robot.
-template <class Real> __device__ void assemble(const KScene<Real>& sc, WS<Real>& w, const StepH<Real>& h) {
+// The group blocks A_g, their coupling rows E_g and the separator block, all from J and
+// Y = M^-1 J^T as the evaluation left them, in 3 x 3 (contact against contact, contact against
+// three coupled rows) and 2 x 3 tiles (separator), a tile per thread and turn: a tile reads
+// 6 rows for 9 products.  One thread per row, forming its own Y and taking its columns after
+// one another, took 9.9 k cycles per Newton iteration of a robot, two threads per row 5.8 k.
+template <class Real> __device__ __forceinline__ void assemble(const KScene<Real>& sc, WS<Real>& w, const StepH<Real>& h) {
   const int tid = threadIdx.x, nth = blockDim.x;
   const int mc = w.ints[1], gstr = tri_size(sc.pg), ss = sc.ss, ldg = sc.ldg;
   const Real hR = h.h;
   // delta = delta_rel * mean diag(h J M^-1 J^T), formed by the evaluation at this iterate
   const Real delta = w.scal[2];
-  const int par = tid & 1;
-  for (int r = tid >> 1; r < mc; r += nth >> 1) {
-    const int g = w.rgrp[r], r0 = w.g0[g], i = r - r0, bg = sc.group_body[g];
-    const int ti = w.meta[4 * r] & 15, si = w.meta[4 * r] >> 4;
-    Real Yr[6], Jv[6];
-    load6(w.J + 12 * r + 6, Yr);
-    // row i of the group block: h J M^-1 J^T, with the diagonal and the radial terms of the
-    // row's own contact (friction rows of one slot are adjacent)
-    Real* Gi = w.G + g * gstr + tri(i, 0);
-#pragma unroll 2
-    for (int j = par; j <= i; j += 2) {
-      load6(w.J + 12 * (r0 + j), Jv);
-      Real v = rn_mul(hR, rowdot(Jv, 0, Yr, 0));
-      if (j + 1 >= i && (j == i || (ti == ROW_FRIC && si == 2))) {
-        const Real* rd = w.srad + 3 * w.ref[r];
-        if (j == i) {
-          v = rn_add(v, rn_add(w.C[r], delta));
-          if (ti == ROW_FRIC) v = rn_add(v, si == 1 ? rd[0] : rd[2]);
-        } else {
-          v = rn_add(v, rd[1]);
-        }
-      }
-      Gi[j] = v;
+  // tiles of group g: its contact pairs, then its contacts by triples of coupled rows
+  int g = 0, base = 0;
+#pragma unroll 1
+  for (int t = tid; ; t += nth) {
+    int np = 0, nt = 0, nk = 0;
+    for (; g < sc.n_groups; ++g) {
+      const int nc = w.gn[g] / 3;
+      np = tri_size(nc);
+      nk = (sc.cpl_n[g] + 2) / 3;
+      nt = np + nc * nk;
+      if (t - base < nt) break;
+      base += nt;
     }
-    Real* Eb = w.E + g * sc.cmax * ldg + i;
-    const int nc = sc.cpl_n[g];
-#pragma unroll 2
-    for (int k = par; k < nc; k += 2) {
-      const int a = sc.cpl_row[g][k];
-      load6(w.J + 12 * (mc + a) + (sc.sep_b[a][0] == bg ? 0 : 6), Jv);
-      Eb[k * ldg] = hR * rowdot(Jv, 0, Yr, 0);
+    if (g >= sc.n_groups) break;
+    // three rows a of contact ca against three rows b: those of contact cb <= ca, or three of
+    // the group's coupled separator rows
+    const int e = t - base, r0 = w.g0[g];
+    const bool pair = e < np;
+    int ca, cb, ob[3];
+    if (pair) {
+      ca = tri_row(e);
+      cb = e - tri(ca, 0);
+#pragma unroll
+      for (int b = 0; b < 3; ++b) ob[b] = 12 * (r0 + 3 * cb + b);
+    } else {
+      ca = (e - np) / nk;
+      cb = e - np - ca * nk;
+      const int bg = sc.group_body[g], last = sc.cpl_n[g] - 1;
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const int a = sc.cpl_row[g][3 * cb + b < last ? 3 * cb + b : last];
+        ob[b] = 12 * (mc + a) + (sc.sep_b[a][0] == bg ? 0 : 6);
+      }
+    }
+    const int ra = r0 + 3 * ca;
+    Real v[3][3], y[3][6], x[6];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) load6(w.J + 12 * (ra + a) + 6, y[a]);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      load6(w.J + ob[b], x);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) v[a][b] = rn_mul(hR, rowdot(x, 0, y[a], 0));
+    }
+    if (pair) {
+      Real* Ga = w.G + g * gstr;
+      if (ca == cb) {
+        // a contact against itself: the diagonal and the radial friction terms
+        const Real* rd = w.srad + 3 * row_ref(w.row[ra]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) v[a][a] = rn_add(v[a][a], rn_add(w.C[ra + a], delta));
+        v[1][1] = rn_add(v[1][1], rd[0]); v[2][1] = rn_add(v[2][1], rd[1]); v[2][2] = rn_add(v[2][2], rd[2]);
+      }
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        Real* Gr = Ga + tri(3 * ca + a, 3 * cb);
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+          if (a >= b || ca != cb) Gr[b] = v[a][b];
+      }
+    } else {
+      Real* Eb = w.E + (g * sc.cmax + 3 * cb) * ldg + 3 * ca;
+#pragma unroll
+      for (int b = 0; b < 3; ++b)
+        if (3 * cb + b < sc.cpl_n[g])
+#pragma unroll
+          for (int a = 0; a < 3; ++a) Eb[b * ldg + a] = v[a][b];
     }
   }
-  for (int e = tid; e < tri_size(ss); e += nth) {
-    const int a = tri_row(e), b = e - tri(a, 0);
-    const int ia0 = sc.sep_b[a][0], ia1 = sc.sep_b[a][1], jb0 = sc.sep_b[b][0], jb1 = sc.sep_b[b][1];
-    const Real* Ya = w.ys + 12 * a;
-    const Real* Jb = w.J + 12 * (mc + b);
-    Real v = 0;
-    if (ia0 == jb0) v += rowdot6(Jb, Ya);
-    if (ia0 == jb1) v += rowdot6(Jb + 6, Ya);
-    if (ia1 == jb0) v += rowdot6(Jb, Ya + 6);
-    if (ia1 == jb1) v += rowdot6(Jb + 6, Ya + 6);
-    v = rn_mul(v, hR);
-    if (a == b) v = rn_add(v, rn_add(w.C[mc + a], delta));
-    w.S[e] = v;
+  // Separator, in blocks of 6 x 6 rows (a joint's five and its servo row, or so), six tiles each.
+  // Entry (a, b) is the sum of J_b . Y_a over the bodies the two rows share, parent parts of
+  // row a first; a part no entry of the tile shares is skipped.
+  const int nblk = tri_size((ss + 5) / 6);
+#pragma unroll 1
+  for (int t = nth - 1 - tid; t < 6 * nblk; t += nth) {
+    const int blk = t / 6, in = t - 6 * blk, I = tri_row(blk);
+    const int a0 = 6 * I + 2 * (in >> 1), b0 = 6 * (blk - tri(I, 0)) + 3 * (in & 1);
+    if (b0 > a0 + 1 || a0 >= ss || b0 >= ss) continue;
+    const int ar[2] = {a0, a0 + 1 < ss ? a0 + 1 : a0};
+    const int br[3] = {b0, b0 + 1 < ss ? b0 + 1 : b0, b0 + 2 < ss ? b0 + 2 : b0};
+    Real v[2][3] = {{Real(0), Real(0), Real(0)}, {Real(0), Real(0), Real(0)}};
+#pragma unroll 1
+    for (int part = 0; part < 4; ++part) {
+      const int pa = part >> 1, pb = part & 1;
+      bool on[2][3], any = false;
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          on[a][b] = sc.sep_b[ar[a]][pa] == sc.sep_b[br[b]][pb];
+          any = any || on[a][b];
+        }
+      if (!any) continue;
+      Real y[2][6], x[6];
+#pragma unroll
+      for (int a = 0; a < 2; ++a) load6(w.ys + 12 * ar[a] + 6 * pa, y[a]);
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        load6(w.J + 12 * (mc + br[b]) + 6 * pb, x);
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+          const Real d = rowdot(x, 0, y[a], 0);
+          if (on[a][b]) v[a][b] = rn_add(v[a][b], d);
+        }
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const int ra = a0 + a, cb = b0 + b;
+        if (ra >= ss || cb > ra) continue;
+        Real x = rn_mul(v[a][b], hR);
+        if (ra == cb) x = rn_add(x, rn_add(w.C[mc + ra], delta));
+        w.S[tri(ra, cb)] = x;
+      }
   }
   __syncthreads();
 }
@@ -1022,72 +1111,131 @@ template <class Real> __device__ void chol_inv_inplace(Real* A, int n, Real* col
   }
 }
 
-// Rows of a register block updated per uniform test of how many are left
-constexpr int REG_CHUNK = 8;
-
-__device__ __forceinline__ void load_chunk(const float* b, float* v) {
-  const float4 x = reinterpret_cast<const float4*>(b)[0], y = reinterpret_cast<const float4*>(b)[1];
-  v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w; v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+__device__ __forceinline__ void load4(const float* b, float* v) {
+  const float4 x = *reinterpret_cast<const float4*>(b);
+  v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
 }
-__device__ __forceinline__ void load_chunk(const double* b, double* v) {
+__device__ __forceinline__ void load4(const double* b, double* v) {
+  const double2 x = reinterpret_cast<const double2*>(b)[0], y = reinterpret_cast<const double2*>(b)[1];
+  v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
+}
+
+// Column `lane` of the symmetric n x n block whose packed lower triangle is A (zeros past its
+// end); the addresses are clamped rather than the loads predicated, so that all are in flight
+// together.
+template <int NR, class Real> __device__ __forceinline__ void load_column(const Real* A, int n, int lane, Real (&a)[NR]) {
+  const int last = n > 0 ? tri_size(n) - 1 : 0;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const double2 x = reinterpret_cast<const double2*>(b)[q];
-    v[2 * q] = x.x; v[2 * q + 1] = x.y;
+  for (int r = 0; r < NR; ++r) {
+    const int i = r >= lane ? tri(r, 0) + lane : tri(lane, 0) + r;
+    const Real v = A[i < last ? i : last];
+    a[r] = r < n && lane < n ? v : Real(0);
   }
 }
 
 // L^-1 of an n x n symmetric positive definite block in place, as chol_inv_inplace, by TW
 // lanes of a warp (32, or 16 with two blocks per warp) with the block in registers:
-// n <= NR <= TW; nmax is the largest n in the warp (its lanes leave the loop together).
+// 0 < n <= TW; nmax is the largest n in the warp (its lanes leave the loop together).
 // Lane j holds column j of the symmetric block, later of L^-1: rows k .. n-1 at the k-th
 // pivot, the pivot row always in a[0] (the rows move up by one as they are updated, so
-// that one loop body serves every pivot).  A pivot takes one broadcast of the diagonal,
-// the reciprocal root, one exchange of the pivot row through `buf` (column k of L is row k
-// of the symmetric block times 1/L[k][k], so every lane supplies its own entry) and one
-// fused multiply-add per row; row k of L^-1 is then final and goes to A.  Every entry
-// receives the operations of chol_inv_inplace in the same order.  buf: 2 TW values,
-// 16-byte aligned, the team's own (two halves in turn: one warp barrier per pivot).
-// What bounds it is the pivot's chain (shuffle, reciprocal root, exchange: about 130
-// cycles), not the row updates; the block through shared memory took about 600 cycles
-// per pivot.
-template <int NR, int TW, class Real>
-__device__ __forceinline__ void chol_inv_regs(Real* A, int n, int nmax, Real* buf) {
+// that one loop body serves every pivot).  Column k of L is row k of the symmetric block
+// times 1/L[k][k], so every lane supplies its own entry of it, exchanged through `buf` (2 TW
+// values, 16-byte aligned, the team's own; two halves in turn: one warp barrier per
+// pivot).  Row k of L^-1 is then final and goes to A.  Every entry receives the operations
+// of chol_inv_inplace in the same order.
+//
+// FP64: its multiply-adds bound it (two a clock per SM), so rows past the end are left out.
+template <int TW> __device__ __forceinline__ void chol_inv_regs(double* A, int n, int nmax, double* buf) {
   const int lane = threadIdx.x & (TW - 1);
-  Real a[NR];
-#pragma unroll
-  for (int r = 0; r < NR; ++r)
-    a[r] = r < n && lane < n ? A[r >= lane ? tri(r, 0) + lane : tri(lane, 0) + r] : Real(0);
-  Real* row = A;
+  double a[TW];
+  load_column(A, n, lane, a);
+  double* row = A + lane;
+#pragma unroll 1
   for (int k = 0; k < nmax; ++k) {
-    const Real akk = __shfl_sync(0xffffffffu, a[0], k, TW);
-    const Real inv = pivot_rsqrt(akk > Real(0) ? akk : Real(1e-30));
+    const double akk = __shfl_sync(0xffffffffu, a[0], k, TW);
+    const double inv = pivot_rsqrt(akk > 0.0 ? akk : 1e-30);
     const bool piv = lane == k;
-    const Real c = piv ? inv : a[0] * inv;
-    Real* bk = buf + (k & 1 ? TW : 0);
+    const double c = piv ? inv : a[0] * inv;
+    double* bk = buf + (k & 1 ? TW : 0);
     if (lane > k) bk[lane - k - 1] = c;
-    if (lane <= k && k < n) row[lane] = c;
+    if (lane <= k && k < n) *row = c;
     row += k + 1;
     __syncwarp();
-    const int left = nmax - 1 - k;
 #pragma unroll
-    for (int q = 0; q < NR; q += REG_CHUNK)
-      if (q < left) {
-        Real l[REG_CHUNK];
-        load_chunk(bk + q, l);
+    for (int q = 0; q < TW; q += 4)
+      if (q < nmax - 1 - k) {
+        double l[4];
+        load4(bk + q, l);
 #pragma unroll
-        for (int r = 0; r < REG_CHUNK; ++r)
-          if (q + r + 1 < NR) a[q + r] = rn_fma(-l[r], c, piv ? Real(0) : a[q + r + 1]);
+        for (int r = 0; r < 4; ++r)
+          if (q + r + 1 < TW) a[q + r] = rn_fma(-l[r], c, piv ? 0.0 : a[q + r + 1]);
       }
   }
 }
 
-// The same for a block of any n the whole warp can hold (n <= 32).
-template <class Real> __device__ __forceinline__ void chol_inv_warp(Real* A, int n, Real* buf) {
-  if (n <= 8) chol_inv_regs<8, 32>(A, n, n, buf);
-  else if (n <= 16) chol_inv_regs<16, 32>(A, n, n, buf);
-  else if (n <= 24) chol_inv_regs<24, 32>(A, n, n, buf);
-  else chol_inv_regs<32, 32>(A, n, n, buf);
+// FP32: what bounds a pivot is the chain from row to row -- multiply, exchange, update of the
+// next row -- and beside it the reciprocal root of the next diagonal, which lane k + 1 forms
+// from its own entries alone (a - c c).  The other rows' updates are put off by one pivot, into
+// the shadow of the next exchange, and the rows taken shrink from 32 or 16 by eights as the
+// block does.  A 24 x 24 block takes 2.8 k cycles of one warp (5.9 k with the updates in their
+// own pivot, tested eight rows at a time; two pivots per exchange with paired
+// multiply-adds 4.5 k), a 12 x 12 block 1.3 k (2.8 k).
+//
+// One pivot k.  On entry a[0] is row k, updated by all pivots before; the other rows still
+// lack the update of pivot k - 1, whose column is lp (lp[r]: row k + r) and whose multiplier
+// in this lane is cp (the lane's rows restart from 0 where its own column was that pivot).
+// Returns with the rows moved up by one, l the column of pivot k (l[r]: row k + 1 + r), c its
+// multiplier and inv 1 / L[k+1][k+1].  NS: rows taken.
+template <int NS, int TW>
+__device__ __forceinline__ void chol_pivot(float (&a)[TW], const float (&lp)[TW], float (&l)[TW], float cp, float& c,
+                                           float& inv, int k, int n, float* bk, float* row) {
+  const int lane = threadIdx.x & (TW - 1);
+  const bool piv = lane == k, kp = lane == k - 1;
+  c = piv ? inv : a[0] * inv;
+  if (lane > k) bk[lane - k - 1] = c;
+  if (lane <= k && k < n) row[lane] = c;
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < NS; q += 4) load4(bk + q, l + q);
+  a[0] = rn_fma(-lp[1], cp, kp ? 0.0f : a[1]);
+  const float d = rn_fma(-c, c, a[0]);
+  const float next = pivot_rsqrt(d > 0.0f ? d : 1e-30f);
+#pragma unroll
+  for (int r = 2; r < NS; ++r) a[r - 1] = rn_fma(-lp[r], cp, kp ? 0.0f : a[r]);
+  inv = __shfl_sync(0xffffffffu, next, k + 1, TW);
+  a[0] = rn_fma(-l[0], c, piv ? 0.0f : a[0]);
+}
+
+// The pivots at which NS rows, but not NS - 8, are needed; two per turn, so that the columns of
+// the last two pivots change places without moves.
+template <int NS, int TW>
+__device__ __forceinline__ void chol_stage(float (&a)[TW], float (&l0)[TW], float (&l1)[TW], float& c0, float& c1,
+                                           float& inv, int& k, int n, int nmax, float* buf, float*& row) {
+#pragma unroll 1
+  for (; k < nmax && (NS == 8 || nmax - k > NS - 8); k += 2) {
+    chol_pivot<NS, TW>(a, l1, l0, c1, c0, inv, k, n, buf, row);
+    row += k + 1;
+    chol_pivot<NS, TW>(a, l0, l1, c0, c1, inv, k + 1, n, buf + TW, row);
+    row += k + 2;
+  }
+}
+
+template <int TW> __device__ __forceinline__ void chol_inv_regs(float* A, int n, int nmax, float* buf) {
+  const int lane = threadIdx.x & (TW - 1);
+  float a[TW], l0[TW], l1[TW];
+  load_column(A, n, lane, a);
+#pragma unroll
+  for (int r = 0; r < TW; ++r) l1[r] = 0.0f;
+  const float a00 = __shfl_sync(0xffffffffu, a[0], 0, TW);
+  float inv = pivot_rsqrt(a00 > 0.0f ? a00 : 1e-30f), c0 = 0.0f, c1 = 0.0f;
+  float* row = A;
+  int k = 0;
+  if (TW == 32) {
+    chol_stage<TW, TW>(a, l0, l1, c0, c1, inv, k, n, nmax, buf, row);
+    chol_stage<TW - 8, TW>(a, l0, l1, c0, c1, inv, k, n, nmax, buf, row);
+  }
+  chol_stage<16, TW>(a, l0, l1, c0, c1, inv, k, n, nmax, buf, row);
+  chol_stage<8, TW>(a, l0, l1, c0, c1, inv, k, n, nmax, buf, row);
 }
 
 // The inverse factors of the contact groups' blocks.  Blocks of up to 16 rows (five of a
@@ -1104,14 +1252,12 @@ template <class Real> __device__ __forceinline__ void factor_groups(const KScene
     for (int g0 = 2 * wid; g0 < ng; g0 += 2 * nw) {
       const int g = g0 + half, n = g < ng ? w.gn[g] : 0;
       const int na = w.gn[g0], nb = g0 + 1 < ng ? w.gn[g0 + 1] : 0, nmax = na > nb ? na : nb;
-      Real* A = w.G + (g < ng ? g : g0) * gstr;
-      if (nmax <= 8) chol_inv_regs<8, 16>(A, n, nmax, buf);
-      else chol_inv_regs<16, 16>(A, n, nmax, buf);
+      if (nmax > 0) chol_inv_regs<16>(w.G + (g < ng ? g : g0) * gstr, n, nmax, buf);
     }
   } else {
     for (int g = wid; g < ng; g += nw) {
       const int n = w.gn[g];
-      if (n <= 32) chol_inv_warp(w.G + g * gstr, n, w.prow + 64 * wid);
+      if (n <= 32) chol_inv_regs<32>(w.G + g * gstr, n, n, w.prow + 64 * wid);
       else chol_inv_inplace(w.G + g * gstr, n, w.prow + 64 * wid);
     }
   }
@@ -1249,7 +1395,7 @@ template <class Real> __device__ void chol_inv_inplace4(Real* A, int n, Real* co
 // synchronises.
 template <class Real> __device__ __forceinline__ void factor_separator(const KScene<Real>& sc, WS<Real>& w) {
   if (sc.ss > 32) chol_inv_inplace4(w.S, sc.ss, w.prow);
-  else if (threadIdx.x < 32) chol_inv_warp(w.S, sc.ss, w.prow);
+  else if (threadIdx.x < 32 && sc.ss > 0) chol_inv_regs<32>(w.S, sc.ss, sc.ss, w.prow);
 }
 
 // Two-accumulator dot products (even and odd terms apart, halving the dependent chain):
@@ -1310,27 +1456,29 @@ template <class Real> __device__ __forceinline__ void factor_eliminate(const KSc
   // F_g[k][j] = sum_{l <= j} E_g[k][l] Li_g[j][l], two threads per contact row
   const int mc = w.ints[1];
   for (int r = tid >> 1; r < mc; r += nth >> 1) {
-    const int g = w.rgrp[r], j = r - w.g0[g], nc = sc.cpl_n[g];
+    const int g = row_grp(w.row[r]), j = r - w.g0[g], nc = sc.cpl_n[g];
     const Real* Lj = w.G + g * gstr + tri(j, 0);
     for (int k = tid & 1; k < nc; k += 2)
       w.H[(g * cm + k) * ldg + j] = dot2c(w.E + (g * cm + k) * ldg, Lj, j + 1);
   }
   __syncthreads();
-  // S' = S - sum_g F_g F_g^T, an entry per thread and turn (the pairs of rows that share a
-  // group; two bodies of one joint may both carry one, then in group order)
-  for (int e = tid; e < tri_size(sc.ss); e += nth) {
-    const int a = tri_row(e), b = e - tri(a, 0), na = sc.sep_n[a], nb2 = sc.sep_n[b];
-    for (int t = 0; t < na; ++t) {
-      // the groups of row a, ascending
-      int pa = t;
-      if (na == 2) pa = (sc.sep_g[a][0] < sc.sep_g[a][1]) == (t == 0) ? 0 : 1;
-      const int g = sc.sep_g[a][pa];
-      for (int pb = 0; pb < nb2; ++pb)
-        if (sc.sep_g[b][pb] == g)
-          w.S[e] -= dot2c(w.H + (g * cm + sc.sep_k[a][pa]) * ldg, w.H + (g * cm + sc.sep_k[b][pb]) * ldg, w.gn[g]);
+  // S' = S - sum_g F_g F_g^T: two threads per coupled row k1 of a group take its pairs k2 <= k1
+  // in turn.  All groups at once, or one after another where a joint's two bodies both
+  // carry one and an entry of its rows takes both groups' terms.
+  const int ng = sc.n_groups, ng_at_once = sc.sep_shared ? 1 : ng;
+  for (int g0 = 0; g0 < ng; g0 += ng_at_once) {
+    for (int e = tid >> 1; e < ng_at_once * cm; e += nth >> 1) {
+      int g = g0, k1 = e;
+      while (k1 >= cm) { k1 -= cm; ++g; }
+      const int n = w.gn[g];
+      if (n == 0 || k1 >= sc.cpl_n[g]) continue;
+      const Real* Fb = w.H + g * cm * ldg;
+      Real* Sa = w.S + tri(sc.cpl_row[g][k1], 0);
+      for (int k2 = tid & 1; k2 <= k1; k2 += 2) Sa[sc.cpl_row[g][k2]] -= dot2c(Fb + k1 * ldg, Fb + k2 * ldg, n);
     }
+    __syncthreads();
   }
-  __syncthreads();
+  if (ng == 0) __syncthreads();
 }
 
 // v <- A^-1 v with the inverse-form block-arrowhead factor, in three parts.
@@ -1343,7 +1491,7 @@ __device__ __forceinline__ void arrow_forward(const KScene<Real>& sc, WS<Real>& 
   Real* y = w.tmp;
   Real* z = w.tmp2;
   for (int r = t; r < mc; r += T) {
-    const int g = w.rgrp[r], r0 = w.g0[g], i = r - r0;
+    const int g = row_grp(w.row[r]), r0 = w.g0[g], i = r - r0;
     y[r] = dot2c(w.G + g * gstr + tri(i, 0), v + r0, i + 1);
   }
   sync();
@@ -1373,7 +1521,7 @@ template <class Real> __device__ __forceinline__ void arrow_backward(const KScen
   const Real* y = w.tmp;
   Real* z = w.tmp2;
   for (int r = tid; r < mc; r += nth) {
-    const int g = w.rgrp[r], i = r - w.g0[g], nc = sc.cpl_n[g];
+    const int g = row_grp(w.row[r]), i = r - w.g0[g], nc = sc.cpl_n[g];
     const Real* Fb = w.H + g * cm * ldg + i;
     Real s0 = y[r], s1 = Real(0);
 #pragma unroll 1
@@ -1394,7 +1542,7 @@ template <class Real> __device__ __forceinline__ void arrow_backward(const KScen
   }
   __syncthreads();
   for (int r = tid; r < mc; r += nth) {
-    const int g = w.rgrp[r], r0 = w.g0[g], i = r - r0;
+    const int g = row_grp(w.row[r]), r0 = w.g0[g], i = r - r0;
     v[r] = dot2col(w.G + g * gstr, i, w.gn[g], z + r0);
   }
   __syncthreads();
@@ -1459,7 +1607,7 @@ __device__ void schur_solve(const KScene<Real>& sc, WS<Real>& w, const Real* b, 
       __syncthreads();
       for (int i = tid; i < m; i += nth) {
         const Real* Ji = w.J + 12 * i;
-        int b0 = w.meta[4 * i + 1], b1 = w.meta[4 * i + 2];
+        int b0 = row_b0(w.row[i]), b1 = row_b1(w.row[i]);
         acc2<Real> ax;
         for (int k = 0; k < 6; ++k) ax.add_prod(Ji[k], t6[6 * b0 + k]);
         if (b1 >= 0) for (int k = 0; k < 6; ++k) ax.add_prod(Ji[6 + k], t6[6 * b1 + k]);
@@ -1468,9 +1616,9 @@ __device__ void schur_solve(const KScene<Real>& sc, WS<Real>& w, const Real* b, 
         res.add_prod(-hR, ax.s);
         res.add_prod(-hR, ax.c);
         res.add_prod(-(w.C[i] + delta), x[i]);
-        int t = w.meta[4 * i] & 15, sub = w.meta[4 * i] >> 4;
+        int t = row_type(w.row[i]), sub = row_sub(w.row[i]);
         if (t == ROW_FRIC) {
-          const Real* rd = w.srad + 3 * w.ref[i];
+          const Real* rd = w.srad + 3 * row_ref(w.row[i]);
           if (sub == 1) { res.add_prod(-rd[0], x[i]); res.add_prod(-rd[1], x[i + 1]); }
           else { res.add_prod(-rd[1], x[i - 1]); res.add_prod(-rd[2], x[i]); }
         }
@@ -1514,7 +1662,7 @@ __device__ Real schur_apply(const KScene<Real>& sc, WS<Real>& w, const Real* v, 
     acc2<Real> ca;
     Real ax = Real(0);
     for (int side = 0; side < 2; ++side) {
-      const int b = w.meta[4 * i + 1 + side];
+      const int b = (side ? row_b1(w.row[i]) : row_b0(w.row[i]));
       if (b < 0) continue;
       Real o[6];
       minv6(sc, w, b, t6 + 6 * b, o);
@@ -1524,14 +1672,14 @@ __device__ Real schur_apply(const KScene<Real>& sc, WS<Real>& w, const Real* v, 
       }
     }
     Real y;
-    const int t = w.meta[4 * i] & 15, sub = w.meta[4 * i] >> 4;
+    const int t = row_type(w.row[i]), sub = row_sub(w.row[i]);
     if (ACC) {
       acc2<Real> ya;
       ya.add_prod(hR, ca.s);
       ya.add_prod(hR, ca.c);
       ya.add_prod(w.C[i] + delta, v[i]);
       if (t == ROW_FRIC) {
-        const Real* rd = w.srad + 3 * w.ref[i];
+        const Real* rd = w.srad + 3 * row_ref(w.row[i]);
         if (sub == 1) { ya.add_prod(rd[0], v[i]); ya.add_prod(rd[1], v[i + 1]); }
         else { ya.add_prod(rd[1], v[i - 1]); ya.add_prod(rd[2], v[i]); }
       }
@@ -1539,7 +1687,7 @@ __device__ Real schur_apply(const KScene<Real>& sc, WS<Real>& w, const Real* v, 
     } else {
       y = hR * ax + (w.C[i] + delta) * v[i];
       if (t == ROW_FRIC) {
-        const Real* rd = w.srad + 3 * w.ref[i];
+        const Real* rd = w.srad + 3 * row_ref(w.row[i]);
         y += sub == 1 ? rd[0] * v[i] + rd[1] * v[i + 1] : rd[1] * v[i - 1] + rd[2] * v[i];
       }
     }
@@ -1559,7 +1707,7 @@ template <class Real> __device__ void pcr_jacobi(const KScene<Real>& sc, WS<Real
     const Real* Ys = w.ys + 12 * (i - mc);
     const Real jy = i < mc ? rowdot6(Ji, Ji + 6) : rowdot6(Ji, Ys) + rowdot6(Ji + 6, Ys + 6);
     Real d = hR * jy + w.C[i] + delta;
-    if ((w.meta[4 * i] & 15) == ROW_FRIC) d += w.srad[3 * w.ref[i] + ((w.meta[4 * i] >> 4) == 1 ? 0 : 2)];
+    if (row_type(w.row[i]) == ROW_FRIC) d += w.srad[3 * row_ref(w.row[i]) + (row_sub(w.row[i]) == 1 ? 0 : 2)];
     pd[i] = Real(1) / d;
   }
 }
@@ -1589,7 +1737,7 @@ template <class Real> __device__ void pcr_precond(const KScene<Real>& sc, WS<Rea
   for (int r = tid; r < m; r += nth) {
     Real acc = Real(0);
     if (r < mc) {
-      const int g = w.rgrp[r], r0 = w.g0[g], i = r - r0;
+      const int g = row_grp(w.row[r]), r0 = w.g0[g], i = r - r0;
       const Real* Li = w.G + g * gstr + tri(i, 0);
       for (int l = 0; l <= i; ++l) acc += Li[l] * v[r0 + l];
     } else {
@@ -1603,7 +1751,7 @@ template <class Real> __device__ void pcr_precond(const KScene<Real>& sc, WS<Rea
   for (int r = tid; r < m; r += nth) {
     Real acc = Real(0);
     if (r < mc) {
-      const int g = w.rgrp[r], r0 = w.g0[g], i = r - r0, n = w.gn[g];
+      const int g = row_grp(w.row[r]), r0 = w.g0[g], i = r - r0, n = w.gn[g];
       const Real* Lb = w.G + g * gstr;
       for (int l = i; l < n; ++l) acc += Lb[tri(l, i)] * y[r0 + l];
     } else {
@@ -1792,7 +1940,7 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
   // warm start: lambda from the previous step on the active rows, into the trial buffers;
   // the loop's evaluation takes it as its first trial
   for (int i = tid; i < 6 * nb; i += nth) w.ut[i] = w.uk[i];
-  for (int i = tid; i < m; i += nth) w.lt[i] = sin[(size_t)(13 * nb + w.meta[4 * i + 3]) * ld + world];
+  for (int i = tid; i < m; i += nth) w.lt[i] = sin[(size_t)(13 * nb + row_lam(w.row[i])) * ld + world];
   __syncthreads();
   clamp_cone(sc, w, w.lt);
   __syncthreads();
@@ -1896,7 +2044,7 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
     if (t0 >= 0 && t0 < T) {
       for (int i = t0; i < m; i += T) {
         const Real* Ji = w.J + 12 * i;
-        const int b0 = w.meta[4 * i + 1], b1 = w.meta[4 * i + 2];
+        const int b0 = row_b0(w.row[i]), b1 = row_b1(w.row[i]);
         acc2<Real> jm;
         for (int q = 0; q < 6; ++q) jm.add_prod(Ji[q], w.mr[6 * b0 + q]);
         if (b1 >= 0) for (int q = 0; q < 6; ++q) jm.add_prod(Ji[6 + q], w.mr[6 * b1 + q]);
@@ -1943,7 +2091,7 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
     }
     for (int i = nth - 1 - tid; i < sc.ss; i += nth) w.lt[mc + i] = w.lk[mc + i] + alpha * w.dl[mc + i];
     for (int sl = nth - 1 - tid; sl < sc.n_slots; sl += nth) {
-      if (!w.sact[sl]) continue;
+      if (w.srow[sl] < 0) continue;
       const int i = w.srow[sl];
       for (int q = 0; q < 3; ++q) w.lt[i + q] = w.lk[i + q] + alpha * w.dl[i + q];
       clamp_slot(sc, w.lt + i);
@@ -1962,7 +2110,7 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
     for (int i = tid; i < sc.n_servo; i += nth) tp[tl.off_ubar + i] = w.ubar[i];
     for (int i = tid; i < sc.m_max; i += nth) tp[tl.off_lam + i] = Real(0);
     __syncthreads();
-    for (int i = tid; i < m; i += nth) tp[tl.off_lam + w.meta[4 * i + 3]] = w.lk[i];
+    for (int i = tid; i < m; i += nth) tp[tl.off_lam + row_lam(w.row[i])] = w.lk[i];
     if (sc.lin == LIN_DIRECT) {
       for (int i = tid; i < sc.n_groups * tri_size(sc.pg); i += nth) tp[tl.off_G + i] = w.G[i];
       for (int i = tid; i < sc.n_groups * sc.cmax * sc.ldg; i += nth) tp[tl.off_H + i] = w.H[i];
@@ -1986,12 +2134,12 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
   }
   __syncthreads();
   for (int i = tid; i < m; i += nth) {
-    int li = w.meta[4 * i + 3];
+    int li = row_lam(w.row[i]);
     so[(size_t)(13 * nb + li) * ld + world] = w.lk[i];
     if (imp) imp[(size_t)li * ld + world] = h.h * w.lk[i];
   }
   if (a.ids)
-    for (int sl = tid; sl < sc.n_slots; sl += nth) a.ids[(size_t)sl * ld + world] = w.sact[sl] ? w.sid[sl] : -1;
+    for (int sl = tid; sl < sc.n_slots; sl += nth) a.ids[(size_t)sl * ld + world] = w.srow[sl] >= 0 ? w.sid[sl] : -1;
   if (tid == 0) {
     if (a.status) a.status[world] = status;
     if (a.cost) a.cost[world] = k;
@@ -1999,13 +2147,10 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
   }
 }
 
-// At most 128 threads per world, registers capped for 3 such CTAs per SM (164 in FP32,
-// no spills; 6 CTAs of 64 threads, the robot world's FP32 setting, fit as well).  A cap
-// for 7 CTAs of 64 threads (128 registers; the robot world's FP32 working set fits 7 per
-// SM) made the 8192-world step slower, 7.12 ms against 6.70 ms: the capped code spills
-// and instruction-fetch stalls grow with the extra CTA (1.5 -> 2.6 per issue).
+// At most 128 threads per world, registers capped at 128 in FP32: eight robot worlds of 64
+// threads per SM then, which their 24.9 KB of workspace allows too.
 template <class Real>
-__global__ void __launch_bounds__(128, 3) step_kernel(const DevScene scp, const StepArgs a) {
+__global__ void __launch_bounds__(128, sizeof(Real) == 4 ? 4 : 3) step_kernel(const DevScene scp, const StepArgs a) {
   extern __shared__ __align__(16) char smem[];
   __shared__ __align__(16) KScene<Real> ssc;
   scene_to_shared(scp, a.h, ssc);
@@ -2121,7 +2266,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
   world_setup<Real>(sc, w, sq, su, sb, h, (Real*)nullptr, tp + tl.off_ct);   // the step's contact set
   const int m = w.ints[0], mc = w.ints[1];
   for (int i = tid; i < 6 * nb; i += nth) w.uk[i] = tp[tl.off_u + i];
-  for (int i = tid; i < m; i += nth) w.lk[i] = tp[tl.off_lam + w.meta[4 * i + 3]];
+  for (int i = tid; i < m; i += nth) w.lk[i] = tp[tl.off_lam + row_lam(w.row[i])];
   __syncthreads();
   evaluate(sc, w, w.uk, w.lk, h, false);   // J (with E at u*), C, delta, poses at q+
   if (tid == 0) {
@@ -2194,7 +2339,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
     // reach the null space of J^T, where A's eigenvalue is only kappa
     for (int i = tid; i < m; i += nth) {
       const Real* Ji = w.J + 12 * i;
-      int b0 = w.meta[4 * i + 1], b1 = w.meta[4 * i + 2];
+      int b0 = row_b0(w.row[i]), b1 = row_b1(w.row[i]);
       acc2<Real> jm;
       for (int k = 0; k < 6; ++k) jm.add_prod(Ji[k], w.mr[6 * b0 + k]);
       if (b1 >= 0) for (int k = 0; k < 6; ++k) jm.add_prod(Ji[6 + k], w.mr[6 * b1 + k]);
@@ -2253,7 +2398,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
     Real* dkp = reinterpret_cast<Real*>(a.dL_dkp);
     for (int i = mc + 5 * sc.nj + tid; i < m; i += nth) {
       // d alpha / d k_p: -1/k_p^2 (velocity target), -h/(k_d + h k_p)^2 (position target)
-      const int j = w.ref[i];
+      const int j = row_ref(w.row[i]);
       const Real al = sc.alpha[j];
       const Real dal = sc.smode[j] == SERVO_POSITION ? -hR * al * al : -al * al;
       dkp[(size_t)(i - mc - 5 * sc.nj) * ld + world] = wl[i] * w.lk[i] * dal;
@@ -2290,7 +2435,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
     if (MODE == ADJ_EXACT) {
       typedef dual<Real> D;
       for (int sl = tid; sl < sc.n_slots; sl += nth) {
-        if (!w.sact[sl]) continue;
+        if (w.srow[sl] < 0) continue;
         const int i = w.srow[sl], b = sc.slot_body[sl];
         CGroup<Real> g;
         contact_group<Real, Real>(sc, w, sl, b, w.qm + 7 * b, w.uk + 6 * b, h, g);
@@ -2322,7 +2467,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
   Real* dctl = reinterpret_cast<Real*>(a.dL_dcontrols);
   if (dctl)   // d b_c / d target: -1 (velocity target), -1/h (position target)
     for (int i = mc + 5 * sc.nj + tid; i < m; i += nth)
-      dctl[(size_t)(i - mc - 5 * sc.nj) * ld + world] = sc.smode[w.ref[i]] == SERVO_POSITION ? -wl[i] / hR : -wl[i];
+      dctl[(size_t)(i - mc - 5 * sc.nj) * ld + world] = sc.smode[row_ref(w.row[i])] == SERVO_POSITION ? -wl[i] / hR : -wl[i];
   // dL/dq-: one work item per (body b, coordinate c of its q-, group touching b or the
   // body's own terms), each a dual-number evaluation along that coordinate; the items of a
   // coordinate are summed in a fixed order

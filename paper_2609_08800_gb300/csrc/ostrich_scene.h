@@ -50,6 +50,7 @@ struct SceneLayout {
   unsigned char cpl_row[NB_CAP][SEP_CAP];
   unsigned char sep_n[SEP_CAP], sep_g[SEP_CAP][2], sep_k[SEP_CAP][2];
   unsigned char sep_b[SEP_CAP][2];       // parent and child body of a separator row
+  int sep_shared;                        // a separator row lies in two groups' lists
 };
 
 // Everything a kernel needs to know about the scene and the solver settings, passed by
@@ -124,6 +125,8 @@ inline void finish_scene(SceneLayout& s) {
       s.sep_n[a]++;
     }
   }
+  s.sep_shared = 0;
+  for (int a = 0; a < s.ss; ++a) if (s.sep_n[a] > 1) s.sep_shared = 1;
   s.cmax = 0;
   for (int g = 0; g < s.n_groups; ++g) if (s.cpl_n[g] > s.cmax) s.cmax = s.cpl_n[g];
 }
