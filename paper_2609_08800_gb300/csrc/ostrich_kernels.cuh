@@ -30,6 +30,7 @@ namespace ost {
 // shared-memory layout of one world
 // ---------------------------------------------------------------------------
 template <class Real> struct WS {
+  int tid;        // this thread's number in the CTA's work (the kernels may turn the warps' order)
   // bodies
   Real *qm, *um, *ubar, *uk, *ut, *ub, *du, *f, *rdyn, *mr, *Iw, *Iwi, *R, *qp;
   Real *sbc;      // per servo: the bias b_c of Eq. (8) (-target, or (x(q-) - target)/h)
@@ -52,8 +53,8 @@ template <class Real> struct WS {
   Real *G, *E, *H, *S, *prow, *tmp, *tmp2;
   // scratch
   Real *red;
-  int *ints;      // [0] rows, [1] contact rows, [2] items, [3] converged, [4] best_k, [5] iters, [6] status,
-                  // [7] contact-generation status bits (4: candidates beyond the slots)
+  int *ints;      // [0] rows, [1] contact rows, [7] contact-generation status bits (4: candidates beyond
+                  // the slots), [8], [9] decisions of the exact adjoint, [14] turn of the warps, [15] work item
   Real *scal;     // [0] merit cur, [1] best merit, [2] delta, [3] merit trial
   Real *pcr;      // PCR mode: r, z, p, A p, A z, P A p and the Jacobi diagonal, m_max each
 };
@@ -145,7 +146,7 @@ template <class Real> size_t ws_bytes(const DevScene& s) { return ws_layout_byte
 
 // deterministic block reduction (fixed tree); result broadcast through w.red[0]
 template <class Real> __device__ Real block_sum(WS<Real>& w, Real v) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
+  const int tid = w.tid, lane = tid & 31, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   __syncthreads();
   if (lane == 0) w.red[wid] = v;
@@ -161,7 +162,7 @@ template <class Real> __device__ Real block_sum(WS<Real>& w, Real v) {
 
 // two deterministic block sums at once (fixed tree, as block_sum): results in a, b
 template <class Real> __device__ void block_sum2(WS<Real>& w, Real& a, Real& b) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
+  const int tid = w.tid, lane = tid & 31, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
   for (int o = 16; o > 0; o >>= 1) {
     a += __shfl_xor_sync(0xffffffffu, a, o);
     b += __shfl_xor_sync(0xffffffffu, b, o);
@@ -177,7 +178,7 @@ template <class Real> __device__ void block_sum2(WS<Real>& w, Real& a, Real& b) 
 
 // block maximum (every thread gets it), through w.red[33..]
 template <class Real> __device__ Real block_max(WS<Real>& w, Real v) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
+  const int tid = w.tid, lane = tid & 31, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
   for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
   __syncthreads();
   if (lane == 0) w.red[33 + wid] = v;
@@ -190,7 +191,7 @@ template <class Real> __device__ Real block_max(WS<Real>& w, Real v) {
 
 // two block maxima at once (every thread gets both), through w.red[40..] and w.red[56..]
 template <class Real> __device__ void block_max2(WS<Real>& w, Real& a, Real& b) {
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
+  const int tid = w.tid, lane = tid & 31, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
   for (int o = 16; o > 0; o >>= 1) {
     a = fmax(a, __shfl_xor_sync(0xffffffffu, a, o));
     b = fmax(b, __shfl_xor_sync(0xffffffffu, b, o));
@@ -426,7 +427,7 @@ __device__ __forceinline__ int tape_to_int(double v) { return (int)v; }
 template <class Real>
 __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, Src<Real> umv, Src<Real> ubarv,
                             const StepH<Real>& h, Real* ct_out = nullptr, const Real* ct_in = nullptr) {
-  const int tid = threadIdx.x, nth = blockDim.x;
+  const int tid = w.tid, nth = blockDim.x;
   const int nb = sc.nb;
   for (int i = tid; i < 7 * nb; i += nth) w.qm[i] = qmv.p[i * qmv.stride];
   for (int i = tid; i < 6 * nb; i += nth) w.um[i] = umv.p[i * umv.stride];
@@ -631,7 +632,7 @@ template <class Real> __device__ __forceinline__ void clamp_slot(const KScene<Re
   }
 }
 template <class Real> __device__ __forceinline__ void clamp_cone(const KScene<Real>& sc, WS<Real>& w, Real* lam) {
-  for (int sl = threadIdx.x; sl < sc.n_slots; sl += blockDim.x)
+  for (int sl = w.tid; sl < sc.n_slots; sl += blockDim.x)
     if (w.srow[sl] >= 0) clamp_slot(sc, lam + w.srow[sl]);
 }
 
@@ -776,7 +777,7 @@ __device__ __forceinline__ void sep_row(const KScene<Real>& sc, WS<Real>& w, con
 // residual and the merit are not formed (the returned merit is 0).
 template <class Real>
 __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, const Real* lam, const StepH<Real>& h, bool dyn = true) {
-  const int tid = threadIdx.x, nth = blockDim.x;
+  const int tid = w.tid, nth = blockDim.x;
   const int nb = sc.nb, m = w.ints[0], mc = w.ints[1];
   const Real hR = h.h;
   // poses at q+ = q- + h G(q-) u
@@ -933,7 +934,7 @@ __device__ __forceinline__ int tri_row(int e) { return (int)(0.5f * (sqrtf((floa
 // 6 rows for 9 products.  One thread per row, forming its own Y and taking its columns after
 // one another, took 9.9 k cycles per Newton iteration of a robot, two threads per row 5.8 k.
 template <class Real> __device__ __forceinline__ void assemble(const KScene<Real>& sc, WS<Real>& w, const StepH<Real>& h) {
-  const int tid = threadIdx.x, nth = blockDim.x;
+  const int tid = w.tid, nth = blockDim.x;
   const int mc = w.ints[1], gstr = tri_size(sc.pg), ss = sc.ss, ldg = sc.ldg;
   const Real hR = h.h;
   // delta = delta_rel * mean diag(h J M^-1 J^T), formed by the evaluation at this iterate
@@ -1242,7 +1243,7 @@ template <int TW> __device__ __forceinline__ void chol_inv_regs(float* A, int n,
 // wheel's slots active; a robot on flat ground has 6 rows per wheel) go two to a warp, larger
 // ones one to a warp, and blocks beyond 32 rows through shared memory.
 template <class Real> __device__ __forceinline__ void factor_groups(const KScene<Real>& sc, WS<Real>& w) {
-  const int tid = threadIdx.x, wid = tid >> 5, nw = blockDim.x >> 5;
+  const int tid = w.tid, wid = tid >> 5, nw = blockDim.x >> 5;
   const int ng = sc.n_groups, gstr = tri_size(sc.pg);
   int big = 0;
   for (int g = 0; g < ng; ++g) big = w.gn[g] > big ? w.gn[g] : big;
@@ -1395,7 +1396,7 @@ template <class Real> __device__ void chol_inv_inplace4(Real* A, int n, Real* co
 // synchronises.
 template <class Real> __device__ __forceinline__ void factor_separator(const KScene<Real>& sc, WS<Real>& w) {
   if (sc.ss > 32) chol_inv_inplace4(w.S, sc.ss, w.prow);
-  else if (threadIdx.x < 32 && sc.ss > 0) chol_inv_regs<32>(w.S, sc.ss, sc.ss, w.prow);
+  else if (w.tid < 32 && sc.ss > 0) chol_inv_regs<32>(w.S, sc.ss, sc.ss, w.prow);
 }
 
 // Two-accumulator dot products (even and odd terms apart, halving the dependent chain):
@@ -1449,7 +1450,7 @@ template <class Real> __device__ __forceinline__ Real dot2col(const Real* T, int
 //   packed).
 // Here all but the last; factor_separator follows.
 template <class Real> __device__ __forceinline__ void factor_eliminate(const KScene<Real>& sc, WS<Real>& w) {
-  const int tid = threadIdx.x, nth = blockDim.x;
+  const int tid = w.tid, nth = blockDim.x;
   const int ldg = sc.ldg, cm = sc.cmax, gstr = tri_size(sc.pg);
   factor_groups(sc, w);
   __syncthreads();
@@ -1516,7 +1517,7 @@ template <class Real> __device__ __forceinline__ void arrow_separator(const KSce
 
 // Groups, backward, by the whole CTA: x_g = Li_g^T (y_g - F_g^T x_s) into v.
 template <class Real> __device__ __forceinline__ void arrow_backward(const KScene<Real>& sc, WS<Real>& w, Real* v) {
-  const int tid = threadIdx.x, nth = blockDim.x;
+  const int tid = w.tid, nth = blockDim.x;
   const int gstr = tri_size(sc.pg), ldg = sc.ldg, cm = sc.cmax, mc = w.ints[1];
   const Real* y = w.tmp;
   Real* z = w.tmp2;
@@ -1549,9 +1550,9 @@ template <class Real> __device__ __forceinline__ void arrow_backward(const KScen
 }
 
 template <class Real> __device__ __forceinline__ void arrow_solve(const KScene<Real>& sc, WS<Real>& w, Real* v) {
-  arrow_forward(sc, w, v, threadIdx.x, blockDim.x, [] { __syncthreads(); });
+  arrow_forward(sc, w, v, w.tid, blockDim.x, [] { __syncthreads(); });
   __syncthreads();
-  if (threadIdx.x < 32) arrow_separator(sc, w, v);
+  if (w.tid < 32) arrow_separator(sc, w, v);
   __syncthreads();
   arrow_backward(sc, w, v);
 }
@@ -1560,7 +1561,7 @@ template <class Real> __device__ __forceinline__ void arrow_solve(const KScene<R
 // component; with ACC exact products and exact partial sums.
 template <bool ACC, class Real>
 __device__ __forceinline__ void jt_apply(const KScene<Real>& sc, WS<Real>& w, const Real* x, Real* out) {
-  for (int task = threadIdx.x; task < 6 * sc.nb; task += blockDim.x) {
+  for (int task = w.tid; task < 6 * sc.nb; task += blockDim.x) {
     const int b = task / 6, k = task - 6 * (task / 6);
     acc2<Real> ca;
     Real acc = Real(0);
@@ -1588,7 +1589,7 @@ template <class Real> __device__ __forceinline__ void minv6(const KScene<Real>& 
 template <class Real>
 __device__ void schur_solve(const KScene<Real>& sc, WS<Real>& w, const Real* b, Real* x, Real* t6, Real* r, const StepH<Real>& h,
                             int sweeps, Real stop_rel = Real(0)) {
-  const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0];
+  const int tid = w.tid, nth = blockDim.x, m = w.ints[0];
   const Real hR = h.h;
   // pass -1 solves for x itself (its correction from x = 0 is A^-1 b), so that one inlined
   // copy of the arrowhead solve serves the first solve and the sweeps
@@ -1652,7 +1653,7 @@ __device__ void schur_solve(const KScene<Real>& sc, WS<Real>& w, const Real* b, 
 // part of v . out; the caller reduces it (the rows are written by their owning threads).
 template <class Real, bool ACC>
 __device__ Real schur_apply(const KScene<Real>& sc, WS<Real>& w, const Real* v, Real* out, Real* t6, const StepH<Real>& h) {
-  const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0];
+  const int tid = w.tid, nth = blockDim.x, m = w.ints[0];
   jt_apply<ACC>(sc, w, v, t6);
   __syncthreads();
   const Real hR = h.h, delta = w.scal[2];
@@ -1699,7 +1700,7 @@ __device__ Real schur_apply(const KScene<Real>& sc, WS<Real>& w, const Real* v, 
 
 // Jacobi preconditioner: the inverse diagonal of A, stored per row by the row's thread
 template <class Real> __device__ void pcr_jacobi(const KScene<Real>& sc, WS<Real>& w, const StepH<Real>& h) {
-  const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0], mc = w.ints[1];
+  const int tid = w.tid, nth = blockDim.x, m = w.ints[0], mc = w.ints[1];
   const Real hR = h.h, delta = w.scal[2];
   Real* pd = w.pcr + 6 * sc.m_max;
   for (int i = tid; i < m; i += nth) {
@@ -1725,7 +1726,7 @@ template <class Real> __device__ __forceinline__ void factor_blocks(const KScene
 // L^-T L^-1 v per block (reads other rows of v: synchronises on entry and between the two
 // triangular products); out is written by the rows' threads.
 template <class Real> __device__ void pcr_precond(const KScene<Real>& sc, WS<Real>& w, const Real* v, Real* out) {
-  const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0], mc = w.ints[1];
+  const int tid = w.tid, nth = blockDim.x, m = w.ints[0], mc = w.ints[1];
   if (sc.pc == PC_JACOBI) {
     const Real* pd = w.pcr + 6 * sc.m_max;
     for (int i = tid; i < m; i += nth) out[i] = pd[i] * v[i];
@@ -1775,7 +1776,7 @@ template <class Real> __device__ void pcr_precond(const KScene<Real>& sc, WS<Rea
 template <class Real, bool ACC>
 __device__ int pcr_solve(const KScene<Real>& sc, WS<Real>& w, const Real* b, Real* x, int iters, Real rtol, Real* t6,
                          const StepH<Real>& h, int* conv) {
-  const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0], M = sc.m_max;
+  const int tid = w.tid, nth = blockDim.x, m = w.ints[0], M = sc.m_max;
   Real *r = w.pcr, *z = r + M, *p = z + M, *Ap = p + M, *Az = Ap + M, *q = Az + M;
   Real bb = Real(0);
   for (int i = tid; i < m; i += nth) { x[i] = Real(0); r[i] = b[i]; bb += b[i] * b[i]; }
@@ -1827,7 +1828,7 @@ __device__ int pcr_solve(const KScene<Real>& sc, WS<Real>& w, const Real* b, Rea
 template <class Real>
 __device__ int pcr_solve_refined(const KScene<Real>& sc, WS<Real>& w, const Real* b, Real* x, int iters, Real rtol,
                                  Real* t6, Real* dx, Real* rt, const StepH<Real>& h, int* conv) {
-  const int tid = threadIdx.x, nth = blockDim.x, m = w.ints[0];
+  const int tid = w.tid, nth = blockDim.x, m = w.ints[0];
   const Real floor = sizeof(Real) == 4 ? Real(1e-4) : Real(0);
   const Real ulp = sizeof(Real) == 4 ? Real(1.1920929e-7) : Real(2.220446049250313e-16);
   Real bb = Real(0);
@@ -1918,7 +1919,7 @@ template <class Real> __device__ __forceinline__ void scene_to_shared(const DevS
 // world launch, or the index a persistent CTA took from the queue).
 template <class Real>
 __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, const StepArgs& a, int item) {
-  const int tid = threadIdx.x, nth = blockDim.x;
+  const int tid = w.tid, nth = blockDim.x;
   const int world = a.list ? a.list[item] : a.world0 + item;
   if (world < 0 || world >= a.n_worlds) return;
   const TapeLayout tl = tape_layout(sc);
@@ -2153,8 +2154,21 @@ template <class Real>
 __global__ void __launch_bounds__(128, sizeof(Real) == 4 ? 4 : 3) step_kernel(const DevScene scp, const StepArgs a) {
   extern __shared__ __align__(16) char smem[];
   __shared__ __align__(16) KScene<Real> ssc;
+  // The CTA's first warp does most of the work that one warp does alone (the separator's
+  // factor and solve, the bodies' sums).  A warp's scheduler follows from its slot on the SM, and
+  // CTAs of two warps would all put their first warps on the same two of the four: every
+  // second CTA takes its warps in the other order (8192 robots: 3.06 -> 2.66 ms with the
+  // adjoint).  The numbering changes no result.  Four warps have a scheduler each; turning
+  // them too made the terrain slower (1.20 -> 1.53 ms).
   scene_to_shared(scp, a.h, ssc);
   WS<Real> w = ws_carve<Real>(smem, ssc);
+  if (threadIdx.x == 0) {
+    unsigned slot;
+    asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
+    w.ints[14] = (int)(slot >> 2);
+  }
+  __syncthreads();
+  w.tid = blockDim.x == 64 ? (int)((threadIdx.x + 32u * (unsigned)w.ints[14]) & 63u) : (int)threadIdx.x;
   // one CTA per world, or persistent: take work items until the queue is exhausted (no CTA
   // waits on another).  One call site for both: a second inlined copy would double the code.
   for (;;) {
@@ -2242,6 +2256,7 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
   scene_to_shared(scp, a.h, ssc);
   const KScene<Real>& sc = ssc;
   WS<Real> w = ws_carve<Real>(smem, sc);
+  w.tid = threadIdx.x;
   ExWS<Real> ex = {};
   if (MODE == ADJ_EXACT) ex = ex_carve<Real>(smem + ws_layout_bytes<Real>(sc), sc);
   const int tid = threadIdx.x, nth = blockDim.x;
