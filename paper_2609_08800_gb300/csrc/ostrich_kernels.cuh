@@ -44,7 +44,6 @@ template <class Real> struct WS {
   int *srow;      // first row of an active slot, -1 of an inactive one
   int *sid, *sftype;
   // per-body row lists
-  int *bgrp, *bsepn;
   uint16_t *bsep;   // offsets in J of the body's parts of the separator rows touching it
   // groups
   int *g0, *gn;
@@ -112,7 +111,7 @@ template <class Real> __host__ __device__ __forceinline__ WS<Real> ws_carve(char
   w.srad = carve<Real>(p, 3 * ns); w.sd = carve<Real>(p, ns); w.swhat = carve<Real>(p, ns);
   w.sedge = carve<Real>(p, 2 * ns);
   w.srow = carve<int>(p, ns); w.sid = carve<int>(p, ns); w.sftype = carve<int>(p, ns);
-  w.bgrp = carve<int>(p, nb); w.bsepn = carve<int>(p, nb); w.bsep = carve<uint16_t>(p, nb * ss);
+  w.bsep = carve<uint16_t>(p, nb * ss);
   w.g0 = carve<int>(p, ng); w.gn = carve<int>(p, ng);
   const int cm = s.cmax > 0 ? s.cmax : 1, ldg = s.ldg > 0 ? s.ldg : 1, esz = ng * cm * ldg;
   // The coupling rows E live from the assembly to F = E L^-T, when the trial multipliers, the
@@ -390,13 +389,6 @@ __device__ __forceinline__ S joint_coord(const KScene<Real>& sc, int j, vec3<S> 
   return dot3(a, (pc + rc) - (pp + rp));
 }
 
-// Joint of the k-th servo.
-template <class Real> __device__ __forceinline__ int servo_joint(const KScene<Real>& sc, int k) {
-  int j = 0, cnt = -1;
-  for (j = 0; j < sc.nj; ++j) if (sc.servo_of[j] >= 0 && ++cnt == k) break;
-  return j;
-}
-
 // ---------------------------------------------------------------------------
 // per-world setup: load inputs, contacts, rows, masses, warm start
 // ---------------------------------------------------------------------------
@@ -432,13 +424,12 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
   for (int i = tid; i < 7 * nb; i += nth) w.qm[i] = qmv.p[i * qmv.stride];
   for (int i = tid; i < 6 * nb; i += nth) w.um[i] = umv.p[i * umv.stride];
   for (int i = tid; i < sc.n_servo; i += nth) w.ubar[i] = ubarv.p[i * ubarv.stride];
+  if (tid == 0) w.ints[7] = 0;
   __syncthreads();
   // contact activation (FP32 predicate) and slot frames in working precision; an item is one
   // slot, or on a heightmap one wheel rim, whose candidate faces fill its nf slots in order.
   // (Rare or long pieces stay loops and single call sites: their code is read once per step
   // and only pushes the Newton loop's out of the instruction cache.)
-  if (tid == 0) w.ints[7] = 0;
-  __syncthreads();
   const bool hm = sc.env == ENV_HEIGHTMAP && !ct_in;
   const int n_rims = hm ? 2 * nb : 0;
 #pragma unroll 1
@@ -494,7 +485,7 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
     }
   }
   // bodies: world inertia at q-, external force, warm-start velocity
-  for (int b = tid; b < nb; b += nth) {
+  for (int b = nth - 1 - tid; b < nb; b += nth) {   // beside the slots' warp
     Real R[9];
     qmat(w.qm + 7 * b + 3, R);
     for (int k = 0; k < 9; ++k) w.R[9 * b + k] = R[k];
@@ -525,7 +516,7 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
   // servo biases b_c of Eq. (8): -target (velocity target) or (x(q-) - target)/h (position
   // target, x the joint coordinate at the step's start; w.R holds R(q-) here)
   for (int k = tid; k < sc.n_servo; k += nth) {
-    const int j = servo_joint(sc, k), bp = sc.jp[j], bc = sc.jc[j];
+    const int j = sc.servo_j[k], bp = sc.jp[j], bc = sc.jc[j];
     if (sc.smode[j] == SERVO_POSITION) {
       const Real x = joint_coord<Real>(sc, j, v3(w.qm[7 * bp], w.qm[7 * bp + 1], w.qm[7 * bp + 2]),
                                        MatRot<Real>{w.R + 9 * bp},
@@ -553,8 +544,7 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
       const int bb = sc.slot_body[sl];
       w.srow[sl] = r0;
       const int lam = 5 * sc.nj + sc.n_servo + 3 * sl;
-      int gb = 0;
-      while (sc.group_body[gb] != bb) ++gb;
+      const int gb = sc.body_group[bb];
       for (int k = 0; k < 3; ++k) {
         const int r = r0 + k;
         w.row[r] = row_word(lam + k, bb, -1, k == 0 ? ROW_NORMAL : ROW_FRIC, k, gb, sl);
@@ -581,32 +571,21 @@ __device__ void world_setup(const KScene<Real>& sc, WS<Real>& w, Src<Real> qmv, 
   {
     const int mc = w.ints[1];
     // separator rows: five per joint, then one per servo
-    for (int a = tid; a < sc.ss; a += nth) {
+    const int ssd = sc.ss > 0 ? sc.ss : 1;
+    for (int a = nth - 1 - tid; a < sc.ss; a += nth) {
       const int r = mc + a;
+      // in its bodies' lists (in row order)
+      for (int side = 0; side < 2; ++side)
+        w.bsep[sc.sep_b[a][side] * ssd + sc.sep_pos[a][side]] = (uint16_t)(12 * r + 6 * side);
       if (a < 5 * sc.nj) {
         const int j = a / 5, k = a - 5 * j;
         w.row[r] = row_word(5 * j + k, sc.jp[j], sc.jc[j], ROW_JOINT, k, 0, j);
       } else {
-        const int j = servo_joint(sc, a - 5 * sc.nj);
+        const int j = sc.servo_j[a - 5 * sc.nj];
         w.row[r] = row_word(5 * sc.nj + sc.servo_of[j], sc.jp[j], sc.jc[j], ROW_SERVO, 0, 0, j);
       }
     }
-    // per-body lists: its group and the separator rows that touch it, in row order
-    const int ssd = sc.ss > 0 ? sc.ss : 1;
-    for (int bb = tid; bb < nb; bb += nth) {
-      int gb = -1;
-      for (int g = 0; g < sc.n_groups; ++g) if (sc.group_body[g] == bb) gb = g;
-      w.bgrp[bb] = gb;
-      int cnt = 0;
-      for (int a2 = 0; a2 < sc.ss; ++a2) {
-        const int j = a2 < 5 * sc.nj ? a2 / 5 : servo_joint(sc, a2 - 5 * sc.nj);
-        if (sc.jp[j] == bb || sc.jc[j] == bb)
-          w.bsep[bb * ssd + cnt++] = (uint16_t)(12 * (mc + a2) + (sc.jp[j] == bb ? 0 : 6));
-      }
-      w.bsepn[bb] = cnt;
-    }
   }
-  __syncthreads();
   // normal-row scaling what = J_n M^-1 J_n^T at q- (geometric Jacobian, E = I)
   for (int sl = tid; sl < sc.n_slots; sl += nth) {
     if (w.srow[sl] < 0) { w.swhat[sl] = 0; continue; }
@@ -688,7 +667,7 @@ __device__ __forceinline__ void minv_row6(const KScene<Real>& sc, const WS<Real>
 // joints.  f(offset of the body's part of the row in J, row).
 template <class Real, class F>
 __device__ __forceinline__ void body_rows(const KScene<Real>& sc, const WS<Real>& w, int b, F&& f) {
-  const int g = w.bgrp[b], r0 = g >= 0 ? w.g0[g] : 0, n = g >= 0 ? w.gn[g] : 0, tot = n + w.bsepn[b];
+  const int g = sc.body_group[b], r0 = g >= 0 ? w.g0[g] : 0, n = g >= 0 ? w.gn[g] : 0, tot = n + sc.body_sepn[b];
   const uint16_t* bs = w.bsep + b * (sc.ss > 0 ? sc.ss : 1) - n;
 #pragma unroll 4
   for (int t = 0; t < tot; ++t) {
@@ -1915,6 +1894,22 @@ template <class Real> __device__ __forceinline__ void scene_to_shared(const DevS
   __syncthreads();
 }
 
+// The thread's number in its CTA's work.  The CTA's first warp does most of the work that one
+// warp does alone (the separator's factor and solve, the bodies' sums).  A warp's scheduler
+// follows from its slot on the SM, and CTAs of two warps would all put their first warps on
+// the same two of the four: every second CTA takes its warps in the other order (8192
+// robots: 3.06 -> 2.66 ms, step + adjoint, for the step's).  The numbering changes no result.
+// Four warps have a scheduler each; turning them too made the terrain slower (1.20 -> 1.53 ms).
+template <class Real> __device__ __forceinline__ void turn_warps(WS<Real>& w) {
+  if (threadIdx.x == 0) {
+    unsigned slot;
+    asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
+    w.ints[14] = (int)(slot >> 2);
+  }
+  __syncthreads();
+  w.tid = blockDim.x == 64 ? (int)((threadIdx.x + 32u * (unsigned)w.ints[14]) & 63u) : (int)threadIdx.x;
+}
+
 // One world's step; `item` is the launch's work index (the CTA index of a one-CTA-per-
 // world launch, or the index a persistent CTA took from the queue).
 template <class Real>
@@ -2154,21 +2149,9 @@ template <class Real>
 __global__ void __launch_bounds__(128, sizeof(Real) == 4 ? 4 : 3) step_kernel(const DevScene scp, const StepArgs a) {
   extern __shared__ __align__(16) char smem[];
   __shared__ __align__(16) KScene<Real> ssc;
-  // The CTA's first warp does most of the work that one warp does alone (the separator's
-  // factor and solve, the bodies' sums).  A warp's scheduler follows from its slot on the SM, and
-  // CTAs of two warps would all put their first warps on the same two of the four: every
-  // second CTA takes its warps in the other order (8192 robots: 3.06 -> 2.66 ms with the
-  // adjoint).  The numbering changes no result.  Four warps have a scheduler each; turning
-  // them too made the terrain slower (1.20 -> 1.53 ms).
   scene_to_shared(scp, a.h, ssc);
   WS<Real> w = ws_carve<Real>(smem, ssc);
-  if (threadIdx.x == 0) {
-    unsigned slot;
-    asm volatile("mov.u32 %0, %%warpid;" : "=r"(slot));
-    w.ints[14] = (int)(slot >> 2);
-  }
-  __syncthreads();
-  w.tid = blockDim.x == 64 ? (int)((threadIdx.x + 32u * (unsigned)w.ints[14]) & 63u) : (int)threadIdx.x;
+  turn_warps(w);
   // one CTA per world, or persistent: take work items until the queue is exhausted (no CTA
   // waits on another).  One call site for both: a second inlined copy would double the code.
   for (;;) {
@@ -2247,19 +2230,23 @@ __device__ Real body_vjp(const KScene<Real>& sc, const WS<Real>& w, int b, int d
 namespace ost {
 
 // One world's adjoint (Sec. III-D) in mode MODE (ADJ_PAPER or ADJ_EXACT).
+// FP32, paper mode: registers capped at 128, so that eight robot worlds of 64 threads run per SM as
+// in the step (8192 robots, step + adjoint: 2.57 -> 2.45 ms although the capped code spills
+// some).  The exact mode's shared memory allows three anyway.
 template <class Real, int MODE>
-__global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, const AdjArgs a) {
+__global__ void __launch_bounds__(128, sizeof(Real) == 4 && MODE == ADJ_PAPER ? 4 : 3) adjoint_kernel(const DevScene scp, const AdjArgs a) {
   extern __shared__ __align__(16) char smem[];
   __shared__ __align__(16) KScene<Real> ssc;
-  __shared__ int bgl[NB_CAP * GROUPS_PER_BODY], bgn[NB_CAP], item0[NB_CAP + 1];
+  __shared__ unsigned char bgl[NB_CAP * GROUPS_PER_BODY];
+  __shared__ int bgn[NB_CAP], item0[NB_CAP + 1];
   __shared__ int ncon[NB_CAP], jpre[NB_CAP + 1], cpre[NB_CAP + 1];
   scene_to_shared(scp, a.h, ssc);
   const KScene<Real>& sc = ssc;
   WS<Real> w = ws_carve<Real>(smem, sc);
-  w.tid = threadIdx.x;
+  turn_warps(w);
   ExWS<Real> ex = {};
   if (MODE == ADJ_EXACT) ex = ex_carve<Real>(smem + ws_layout_bytes<Real>(sc), sc);
-  const int tid = threadIdx.x, nth = blockDim.x;
+  const int tid = w.tid, nth = blockDim.x;
   const int world = a.list ? a.list[blockIdx.x] : a.world0 + blockIdx.x;
   if (world < 0 || world >= a.n_worlds) return;
   const int slot = a.list ? (a.list_slot ? a.list_slot[blockIdx.x] : -1) : 0;
@@ -2284,21 +2271,28 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
   for (int i = tid; i < m; i += nth) w.lk[i] = tp[tl.off_lam + row_lam(w.row[i])];
   __syncthreads();
   evaluate(sc, w, w.uk, w.lk, h, false);   // J (with E at u*), C, delta, poses at q+
-  if (tid == 0) {
-    body_groups(sc, w, bgl, bgn);
-    int acc = 0;
-    for (int b = 0; b < nb; ++b) { item0[b] = acc; acc += 7 * (bgn[b] + 1); }
-    item0[nb] = acc;
-    // work order of the pull-back items by cost: joint groups, contact groups, body terms
-    int aj = 0, ac = 0;
-    for (int b = 0; b < nb; ++b) {
-      int nc = 0;
-      while (nc < bgn[b] && bgl[b * GROUPS_PER_BODY + nc] < sc.n_slots) ++nc;
-      ncon[b] = nc;
-      jpre[b] = aj; aj += 7 * (bgn[b] - nc);
-      cpre[b] = ac; ac += 7 * nc;
+  if (tid < 32) {
+    // a lane per body: its groups, and by prefix sums over the bodies the places of its
+    // pull-back items and their work order by cost (joint groups, contact groups, body terms)
+    const int lane = tid;
+    const bool tr = MODE == ADJ_PAPER && sc.pullback == 1;
+    int nc = 0, ng = 0;
+    bool dual_pos = false;
+    if (lane < nb) {
+      ng = body_groups(sc, w, lane, bgl, nc);
+      for (int k = 0; k < ng; ++k) dual_pos = dual_pos || position_needs_dual(sc, w, bgl[lane * GROUPS_PER_BODY + k], tr);
+      bgn[lane] = ng;
+      ncon[lane] = nc;
     }
-    jpre[nb] = aj; cpre[nb] = ac;
+    const int n_coord = __any_sync(0xffffffffu, dual_pos) ? 7 : 4;
+    int pi = lane < nb ? 7 * (ng + 1) : 0, pj = n_coord * (ng - nc), pc = n_coord * nc;
+    for (int o = 1; o < NB_CAP; o <<= 1) {             // inclusive sums
+      const int ui = __shfl_up_sync(0xffffffffu, pi, o), uj = __shfl_up_sync(0xffffffffu, pj, o);
+      const int uc = __shfl_up_sync(0xffffffffu, pc, o);
+      if (lane >= o) { pi += ui; pj += uj; pc += uc; }
+    }
+    if (lane == 0) { item0[0] = 0; jpre[0] = 0; cpre[0] = 0; }
+    if (lane < nb) { item0[lane + 1] = pi; jpre[lane + 1] = pj; cpre[lane + 1] = pc; }
   }
   if (sc.lin == LIN_DIRECT) {
     cp_async_wait_all();     // this thread's copies of the taped factor; the barrier below
@@ -2491,8 +2485,9 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
                         // sum_b 7 (groups_b + 1) <= 14 m_max items
   // taken in cost order (every joint item, then every contact item, then the body terms)
   // so that the threads' loads even out; each item is stored at its place in the per-body
-  // layout, which fixes the order of the sums below
-  const int n_items = item0[nb], nj_items = jpre[nb], nc_items = cpre[nb];
+  // layout, which fixes the order of the sums below.  n_coord: the four quaternion
+  // coordinates, and the three positions after them where a group has no closed form for those.
+  const int nj_items = jpre[nb], nc_items = cpre[nb], n_items = nj_items + nc_items + 4 * nb;
   for (int e = tid; e < n_items; e += nth) {
     int b = 0, c, k;
     if (e < nj_items) {
@@ -2508,20 +2503,27 @@ __global__ void __launch_bounds__(128, 3) adjoint_kernel(const DevScene scp, con
       k = 1 + (r - c * nc);
     } else {
       const int e3 = e - nj_items - nc_items;
-      b = e3 / 7;
-      c = e3 - 7 * b;
+      b = e3 / 4;
+      c = e3 - 4 * b;
       k = 0;
     }
+    c = c < 4 ? 3 + c : c - 4;
+    const int grp = k ? bgl[b * GROUPS_PER_BODY + k - 1] : 0;
+    if (c < 3 && !position_needs_dual(sc, w, grp, trunc)) continue;
     item[item0[b] + c * (bgn[b] + 1) + k] =
-        k == 0 ? body_vjp(sc, w, b, c, gq, wu, h)
-               : group_vjp_q<Real, MODE>(sc, w, ex, bgl[b * GROUPS_PER_BODY + k - 1], b, c, wl, wu, trunc, h);
+        k == 0 ? body_vjp(sc, w, b, c, gq, wu, h) : group_vjp_q<Real, MODE>(sc, w, ex, grp, b, c, wl, wu, trunc, h);
   }
   __syncthreads();
+  const Real inv_h = Real(1) / hR;
   for (int e = tid; e < nb * 7; e += nth) {
     const int b = e / 7, c = e % 7;
     acc2<Real> acc;        // the terms cancel strongly: compensated sum
     const int base = item0[b] + c * (bgn[b] + 1);
-    for (int k = 0; k <= bgn[b]; ++k) acc.add(item[base + k]);
+    for (int k = 0; k <= bgn[b]; ++k) {
+      const int grp = k ? bgl[b * GROUPS_PER_BODY + k - 1] : 0;
+      if (c >= 3 || (k && position_needs_dual(sc, w, grp, trunc))) acc.add(item[base + k]);
+      else acc.add(k ? group_pull_position<Real, MODE>(sc, w, ex, grp, b, c, wl, inv_h) : gq[7 * b + c]);
+    }
     dout[(size_t)(7 * b + c) * ld + world] = acc.value();
   }
 }

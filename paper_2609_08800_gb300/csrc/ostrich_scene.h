@@ -51,6 +51,10 @@ struct SceneLayout {
   unsigned char sep_n[SEP_CAP], sep_g[SEP_CAP][2], sep_k[SEP_CAP][2];
   unsigned char sep_b[SEP_CAP][2];       // parent and child body of a separator row
   int sep_shared;                        // a separator row lies in two groups' lists
+  // per body its group (-1: none) and the number of separator rows touching it; a separator
+  // row's place in the lists of its two bodies; joint of each servo
+  signed char body_group[NB_CAP];
+  unsigned char body_sepn[NB_CAP], sep_pos[SEP_CAP][2], servo_j[NJ_CAP];
 };
 
 // Everything a kernel needs to know about the scene and the solver settings, passed by
@@ -103,7 +107,7 @@ inline void finish_scene(SceneLayout& s) {
   s.ldg = s.pg | 1;
   s.lds = s.ss | 1;
   int gof[NB_CAP];
-  for (int b = 0; b < NB_CAP; ++b) gof[b] = -1;
+  for (int b = 0; b < NB_CAP; ++b) { gof[b] = -1; s.body_sepn[b] = 0; }
   for (int g = 0; g < s.n_groups; ++g) { gof[s.group_body[g]] = g; s.cpl_n[g] = 0; }
   for (int a = 0; a < s.ss; ++a) {
     int j = a < 5 * s.nj ? a / 5 : -1;
@@ -112,9 +116,11 @@ inline void finish_scene(SceneLayout& s) {
       for (j = 0; j < s.nj; ++j) if (s.servo_of[j] >= 0 && ++cnt == k) break;
     }
     s.sep_n[a] = 0;
+    if (a >= 5 * s.nj) s.servo_j[a - 5 * s.nj] = (unsigned char)j;
     int bodies[2] = {s.jp[j], s.jc[j]};
     s.sep_b[a][0] = (unsigned char)bodies[0];
     s.sep_b[a][1] = (unsigned char)bodies[1];
+    for (int t = 0; t < 2; ++t) s.sep_pos[a][t] = s.body_sepn[bodies[t]]++;
     for (int t = 0; t < 2; ++t) {
       int g = gof[bodies[t]];
       if (g < 0) continue;
@@ -125,6 +131,7 @@ inline void finish_scene(SceneLayout& s) {
       s.sep_n[a]++;
     }
   }
+  for (int b = 0; b < NB_CAP; ++b) s.body_group[b] = (signed char)gof[b];
   s.sep_shared = 0;
   for (int a = 0; a < s.ss; ++a) if (s.sep_n[a] > 1) s.sep_shared = 1;
   s.cmax = 0;
