@@ -759,10 +759,17 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
   const int tid = w.tid, nth = blockDim.x;
   const int nb = sc.nb, m = w.ints[0], mc = w.ints[1];
   const Real hR = h.h;
-  // poses at q+ = q- + h G(q-) u
-  for (int b = tid; b < nb; b += nth) {
-    kin_body<Real, Real>(w.qm + 7 * b, u + 6 * b, h, w.qp + 7 * b);
-    qmat(w.qp + 7 * b + 3, w.R + 9 * b);
+  // poses at q+ = q- + h G(q-) u, a thread per body and axis (column of the rotation)
+  for (int e = tid; e < 3 * nb; e += nth) {
+    const int b = e / 3, ax = e - 3 * b;
+    Real qp[7];
+    kin_body<Real, Real>(w.qm + 7 * b, u + 6 * b, h, qp);
+    const vec3<Real> c = qrot(qp + 3, v3(ax == 0 ? Real(1) : Real(0), ax == 1 ? Real(1) : Real(0),
+                                         ax == 2 ? Real(1) : Real(0)));
+    Real* R = w.R + 9 * b + ax;
+    R[0] = c.x; R[3] = c.y; R[6] = c.z;
+    if (ax == 0)
+      for (int k = 0; k < 7; ++k) w.qp[7 * b + k] = qp[k];
   }
   __syncthreads();
   // contact slots from the first thread on, separator rows from the last: they run beside
@@ -836,6 +843,30 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
   }
   for (int a = nth - 1 - tid; a < sc.ss; a += nth) sep_row(sc, w, u, lam, h, a, mc);
   __syncthreads();
+  // Y = M^-1 J^T of every row and the diagonal J Y of J M^-1 J^T, for the assembly at this
+  // iterate and its damping delta = delta_rel * mean diag(h J Y); from the last thread, beside
+  // the bodies' residuals below
+  for (int i = nth - 1 - tid; i < m; i += nth) {
+    Real* Ji = w.J + 12 * i;
+    const uint32_t rw = w.row[i];
+    Real Yi[6], Jv[6];
+    load6(Ji, Jv);
+    minv_row6(sc, w, row_b0(rw), Jv, Yi);
+    Real d = rowdot(Jv, 0, Yi, 0);
+    if (i < mc) {
+      store6(Ji + 6, Yi);
+    } else {
+      // (the direct adjoint, dyn = false, needs no Y, and its F is on its way to that place)
+      Real* Ys = w.ys + 12 * (i - mc);
+      const bool keep = dyn || sc.lin == LIN_PCR;
+      if (keep) store6(Ys, Yi);
+      load6(Ji + 6, Jv);
+      minv_row6(sc, w, row_b1(rw), Jv, Yi);
+      if (keep) store6(Ys + 6, Yi);
+      d = d + rowdot(Jv, 0, Yi, 0);
+    }
+    w.tmp[i] = d;
+  }
   if (dyn) {
     // Eq. (10): r_dyn = M (u - u-) - h f - h J^T lambda, per body; merit part |M^-1 r_dyn|^2.
     // The inertia and constraint terms nearly cancel at convergence, so the sum is
@@ -857,8 +888,8 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
       rd.add_prod(-hR, w.f[6 * b + k]);
       w.rdyn[6 * b + k] = rd.value();
     }
-    __syncthreads();
   }
+  __syncthreads();
   Real part = Real(0);
   for (int b = tid; b < nb && dyn; b += nth) {
     const Real* rv = w.rdyn + 6 * b;
@@ -867,29 +898,10 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
     Real mr[6] = {rv[0] * mi, rv[1] * mi, rv[2] * mi, iw.x, iw.y, iw.z};
     for (int k = 0; k < 6; ++k) { w.mr[6 * b + k] = mr[k]; part += mr[k] * mr[k]; }
   }
-  // with the merit: Y = M^-1 J^T of every row and delta = delta_rel * mean diag(h J Y) of
-  // these rows, for the assembly at this iterate (scal[2])
   Real dpart = 0;
   for (int i = tid; i < m; i += nth) {
     if (dyn) part += w.r2[i] * w.r2[i];
-    Real* Ji = w.J + 12 * i;
-    Real Yi[6], Jv[6];
-    load6(Ji, Jv);
-    minv_row6(sc, w, row_b0(w.row[i]), Jv, Yi);
-    Real d = rowdot(Jv, 0, Yi, 0);
-    if (i < mc) {
-      store6(Ji + 6, Yi);
-    } else {
-      // (the direct adjoint, dyn = false, needs no Y, and its F is on its way to that place)
-      Real* Ys = w.ys + 12 * (i - mc);
-      const bool keep = dyn || sc.lin == LIN_PCR;
-      if (keep) store6(Ys, Yi);
-      load6(Ji + 6, Jv);
-      minv_row6(sc, w, row_b1(w.row[i]), Jv, Yi);
-      if (keep) store6(Ys + 6, Yi);
-      d = d + rowdot(Jv, 0, Yi, 0);
-    }
-    dpart += hR * d;
+    dpart += hR * w.tmp[i];
   }
   block_sum2(w, part, dpart);
   if (tid == 0) w.scal[2] = m > 0 ? sc.delta_rel * dpart / Real(m) : Real(0);
@@ -902,10 +914,14 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
 // ---------------------------------------------------------------------------
 
 
-// Row of the packed lower triangle that entry e lies in.  (8 e + 1 is the square of 2 a + 1
-// at a row's first entry and below the next odd square in it, and below 2^24 here, so the
-// rounded root's integer part is exact.)
-__device__ __forceinline__ int tri_row(int e) { return (int)(0.5f * (sqrtf((float)(8 * e + 1)) - 1.0f)); }
+// Row a of the packed lower triangle that entry e lies in: (2 a + 1)^2 <= 8 e + 1 < (2 a + 3)^2.
+// Half a unit added under the root keeps it off these squares by more than 1e-5 of its value
+// for every triangle here, far beyond the approximate root's error.
+__device__ __forceinline__ int tri_row(int e) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"((float)(8 * e + 1) + 0.5f));
+  return (int)(0.5f * (r - 1.0f));
+}
 
 // The group blocks A_g, their coupling rows E_g and the separator block, all from J and
 // Y = M^-1 J^T as the evaluation left them, in 3 x 3 (contact against contact, contact against
@@ -943,8 +959,8 @@ template <class Real> __device__ __forceinline__ void assemble(const KScene<Real
 #pragma unroll
       for (int b = 0; b < 3; ++b) ob[b] = 12 * (r0 + 3 * cb + b);
     } else {
-      ca = (e - np) / nk;
-      cb = e - np - ca * nk;
+      ca = 0;
+      for (cb = e - np; cb >= nk; cb -= nk) ++ca;
       const int bg = sc.group_body[g], last = sc.cpl_n[g] - 1;
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
