@@ -124,7 +124,10 @@ ostrich_status ostrich_create(const ostrich_scene_desc* scene, const ostrich_sol
 /* Layout sizes: out[0] n_state, out[1] m_max, out[2] n_slots, out[3] n_servo. */
 ostrich_status ostrich_layout(const ostrich_ctx* ctx, int32_t out[4]);
 
-/* Threads per world (32, 64 or 128) used by both kernels; the autotuner's knob. */
+/* Threads per world (32, 64 or 128) of both kernels; the autotuner's knob.  It fixes the order in
+ * which the sums over a world's rows are taken, hence the results' rounding.  A launch of so
+ * few worlds that all run at once with 128 threads each may use 128 whatever the setting, in
+ * the same order: a world's result does not depend on how many others the launch holds. */
 ostrich_status ostrich_set_threads(ostrich_ctx* ctx, int threads);
 
 /* Launch schedule of ostrich_step (an autotuner knob; results do not depend on it):

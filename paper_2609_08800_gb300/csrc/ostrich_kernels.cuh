@@ -31,6 +31,7 @@ namespace ost {
 // ---------------------------------------------------------------------------
 template <class Real> struct WS {
   int tid;        // this thread's number in the CTA's work (the kernels may turn the warps' order)
+  int sum_nth;    // threads whose partial sums the merit and the damping are added up from
   // bodies
   Real *qm, *um, *ubar, *uk, *ut, *ub, *du, *f, *rdyn, *mr, *Iw, *Iwi, *R, *qp;
   Real *sbc;      // per servo: the bias b_c of Eq. (8) (-target, or (x(q-) - target)/h)
@@ -899,10 +900,11 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
     for (int k = 0; k < 6; ++k) { w.mr[6 * b + k] = mr[k]; part += mr[k] * mr[k]; }
   }
   Real dpart = 0;
-  for (int i = tid; i < m; i += nth) {
-    if (dyn) part += w.r2[i] * w.r2[i];
-    dpart += hR * w.tmp[i];
-  }
+  if (tid < w.sum_nth)
+    for (int i = tid; i < m; i += w.sum_nth) {
+      if (dyn) part += w.r2[i] * w.r2[i];
+      dpart += hR * w.tmp[i];
+    }
   block_sum2(w, part, dpart);
   if (tid == 0) w.scal[2] = m > 0 ? sc.delta_rel * dpart / Real(m) : Real(0);
   __syncthreads();                         // scal[2] is read by the assembly that follows
@@ -2168,6 +2170,7 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 ? 4 : 3) step_kernel(co
   scene_to_shared(scp, a.h, ssc);
   WS<Real> w = ws_carve<Real>(smem, ssc);
   turn_warps(w);
+  w.sum_nth = a.sum_threads;
   // one CTA per world, or persistent: take work items until the queue is exhausted (no CTA
   // waits on another).  One call site for both: a second inlined copy would double the code.
   for (;;) {
@@ -2260,6 +2263,7 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 && MODE == ADJ_PAPER ? 
   const KScene<Real>& sc = ssc;
   WS<Real> w = ws_carve<Real>(smem, sc);
   turn_warps(w);
+  w.sum_nth = a.sum_threads;
   ExWS<Real> ex = {};
   if (MODE == ADJ_EXACT) ex = ex_carve<Real>(smem + ws_layout_bytes<Real>(sc), sc);
   const int tid = w.tid, nth = blockDim.x;
@@ -2562,6 +2566,25 @@ template <class K> cudaError_t ensure_smem(K kernel, size_t smem, int* done_dev,
   return e;
 }
 
+// Threads of a world's CTA in a launch of n worlds for a context set to `threads`.  Few worlds leave
+// most of the chip's schedulers idle, and what counts is one world's latency: four warps then
+// share its rows and tiles (1 robot, step 234 -> 213 us, adjoint 41 -> 39; 608 robots 269 -> 258 us;
+// 2048 robots would take 981 instead of 665), as long as all worlds run at once: four CTAs of
+// 128 threads per SM in FP32, two in FP64, whose arithmetic units more warps do not help beyond
+// that (608 robots: adjoint 213 -> 276 us).  Scenes of at most a warp's rows gain nothing.
+// The sums over all rows keep the order of `threads` (sum_threads), so results do not depend on
+// this.  The conjugate-residual solver and the exact adjoint sum over the whole CTA in more
+// places: they keep their threads.
+template <class Real> int cta_threads(const DevScene& sc, int threads, int n, int* sms_of_dev) {
+  if (threads >= 128 || sc.lin != LIN_DIRECT || sc.m_max <= 32) return threads;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return threads;
+  if (!sms_of_dev[dev] &&
+      cudaDeviceGetAttribute(&sms_of_dev[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return threads;
+  return n <= (sizeof(Real) == 4 ? 4 : 2) * sms_of_dev[dev] ? 128 : threads;
+}
+
 template <class Real>
 cudaError_t launch_step(const DevScene& sc, const StepArgs& a, int threads, cudaStream_t st) {
   static int done_dev[64] = {0};
@@ -2572,26 +2595,29 @@ cudaError_t launch_step(const DevScene& sc, const StepArgs& a, int threads, cuda
   if (e != cudaSuccess) return e;
   int n = a.list ? a.n_list : a.n_worlds - a.world0;
   if (n <= 0) return cudaSuccess;
+  static int sms[64] = {0};
+  StepArgs b = a;
+  b.sum_threads = threads;
+  threads = cta_threads<Real>(sc, threads, n, sms);
   if (a.queue) {
     // persistent: as many CTAs as fit on the device at once, fed from the queue
-    int dev = 0, sms = 0, per_sm = 0;
+    int dev = 0, n_sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem)) != cudaSuccess)
       return e;
     if (per_sm < 1) per_sm = 1;
-    int grid = sms * per_sm < n ? sms * per_sm : n;
+    int grid = n_sms * per_sm < n ? n_sms * per_sm : n;
     if ((e = cudaMemsetAsync(a.queue, 0, sizeof(int), st)) != cudaSuccess) return e;
     if (a.order && a.cost) {
       lpt_order_kernel<<<1, 1024, 0, st>>>(a.cost + a.world0, n, const_cast<int32_t*>(a.order));
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    StepArgs b = a;
     b.n_items = n;
     kernel<<<grid, threads, smem, st>>>(sc, b);
     return cudaGetLastError();
   }
-  kernel<<<n, threads, smem, st>>>(sc, a);
+  kernel<<<n, threads, smem, st>>>(sc, b);
   return cudaGetLastError();
 }
 
@@ -2606,7 +2632,11 @@ cudaError_t launch_adjoint(const DevScene& sc, const AdjArgs& a, int threads, cu
   if (e != cudaSuccess) return e;
   int n = a.list ? a.n_list : a.n_worlds - a.world0;
   if (n <= 0) return cudaSuccess;
-  kernel<<<n, threads, smem, st>>>(sc, a);
+  static int sms[64] = {0};
+  AdjArgs b = a;
+  b.sum_threads = threads;
+  if (mode == ADJ_PAPER) threads = cta_threads<Real>(sc, threads, n, sms);
+  kernel<<<n, threads, smem, st>>>(sc, b);
   return cudaGetLastError();
 }
 

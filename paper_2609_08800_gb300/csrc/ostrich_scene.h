@@ -150,6 +150,7 @@ struct StepArgs {
   const void* state_in; const void* controls; void* state_out; void* impulses;
   int32_t* ids; uint32_t* status; int32_t* iters; void* tape;
   int ld, n_worlds, world0; double h;
+  int sum_threads = 0;       // threads per world whose summation order the launch keeps (set by the launcher)
   double* trace = nullptr;   // optional diagnostic: merit of each iterate, (budget + 2) per world
   const int32_t* list = nullptr; const int32_t* list_slot = nullptr; int n_list = 0, tape_slots = 0;
   // persistent schedule (queue != nullptr): gridDim CTAs take the work items 0 .. n_items-1
@@ -160,6 +161,7 @@ struct StepArgs {
 struct AdjArgs {
   const void* tape; const void* dL_dnext; void* dL_dstate; void* dL_dcontrols;
   int ld, n_worlds, world0; double h;
+  int sum_threads = 0;       // as in StepArgs
   const int32_t* list = nullptr; const int32_t* list_slot = nullptr; int n_list = 0, tape_slots = 0;
   // optional physical-parameter gradients: dL/dk_p per servo (n_servo x ld), dL/dm per
   // body (nb x ld), dL/dI per body-frame principal moment (3 nb x ld), or null
