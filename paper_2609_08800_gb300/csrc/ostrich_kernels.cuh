@@ -750,12 +750,89 @@ __device__ __forceinline__ void sep_row(const KScene<Real>& sc, WS<Real>& w, con
   w.r2[i] = r; w.rhat[i] = r; w.C[i] = C;
 }
 
+// The rows of contact slot sl: the normal's, the two of friction, or all three.
+template <bool NORM, bool FRIC, class Real>
+__device__ __forceinline__ void slot_rows(const KScene<Real>& sc, WS<Real>& w, const Real* u, const Real* lam,
+                                          const StepH<Real>& h, int sl) {
+  const Real hR = h.h;
+  int i = w.srow[sl];
+  int b = sc.slot_body[sl];
+  int local = sl - sc.slot_base[b];
+  vec3<Real> p = v3(w.qp[7 * b], w.qp[7 * b + 1], w.qp[7 * b + 2]);
+  vec3<Real> n = v3(w.sn[3 * sl], w.sn[3 * sl + 1], w.sn[3 * sl + 2]);
+  vec3<Real> t1 = v3(w.st1[3 * sl], w.st1[3 * sl + 1], w.st1[3 * sl + 2]);
+  vec3<Real> t2 = v3(w.st2[3 * sl], w.st2[3 * sl + 1], w.st2[3 * sl + 2]);
+  vec3<Real> x = slot_point<Real>(sc, b, local, p, w.qp + 7 * b + 3, n);
+  vec3<Real> lev = x - p;
+  vec3<Real> wk = v3(u[6 * b + 3], u[6 * b + 4], u[6 * b + 5]);
+  vec3<Real> dirs[3] = {n, t1, t2};
+  Real vel[3];
+  const MapE<Real> Ek(wk, h);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    if (k == 0 ? !NORM : !FRIC) continue;
+    vec3<Real> ang = Ek(cross3(lev, dirs[k]));
+    Real* Jr = w.J + 12 * (i + k);
+    Jr[0] = dirs[k].x; Jr[1] = dirs[k].y; Jr[2] = dirs[k].z; Jr[3] = ang.x; Jr[4] = ang.y; Jr[5] = ang.z;
+    vel[k] = dirs[k].x * u[6 * b] + dirs[k].y * u[6 * b + 1] + dirs[k].z * u[6 * b + 2] + ang.x * u[6 * b + 3] +
+             ang.y * u[6 * b + 4] + ang.z * u[6 * b + 5];
+  }
+  const Real kap = sc.kappa, eps = sc.eps;
+  const Real hw = hR * w.swhat[sl];
+  const Real ln = lam[i];
+  if (NORM) {
+    // normal row, Eq. (4): phi_eps(c_n/h + kappa lambda_n, h what lambda_n)
+    Real cn = dot3(n, x) - w.sd[sl];
+    Real a = cn / hR + kap * ln, bb = hw * ln;
+    // At an active contact b = h what lambda_n is large (~10 m/s) and a ~ 0, so the
+    // textbook forms a + b - s, 1 - a/s and 1 - b/s cancel; in FP32 that leaves ~1e-6
+    // m/s of noise in the row, which the small eigenvalue (~kappa) of the impulse split
+    // between redundant contacts amplifies to ~1e-3 N and the Newton iteration stalls.
+    // The same quantities in forms free of cancellation (exact rearrangements):
+    // a + b - s = (2ab - eps^2)/(a + b + s) for a + b > 0;  1 - a/s = (b^2 + eps^2)/(s (s + a))
+    // for a > 0;  1 - b/s likewise.
+    Real s = ssqrt(a * a + bb * bb + eps * eps);
+    const Real apb = a + bb;
+    Real phi = apb > Real(0) ? (Real(2) * a * bb - eps * eps) / (apb + s) : apb - s;
+    Real fa = a > Real(0) ? (bb * bb + eps * eps) / (s * (s + a)) : Real(1) - a / s;
+    Real fb = bb > Real(0) ? (a * a + eps * eps) / (s * (s + bb)) : Real(1) - bb / s;
+    Real scl = fa > Real(1e-12) ? fa : Real(1e-12);
+    w.r2[i] = phi; w.rhat[i] = phi / scl; w.C[i] = kap + hw * fb / scl;
+  }
+  if (!FRIC) return;
+  // friction rows, Eq. (7): J_f u + (W + kappa) lambda_f with W from the FB reading
+  const Real l1 = lam[i + 1], l2 = lam[i + 2];
+  Real vt = ssqrt(vel[1] * vel[1] + vel[2] * vel[2] + eps * eps);
+  Real lfn = ssqrt(l1 * l1 + l2 * l2 + eps * eps);
+  Real lnp = ln > Real(0) ? ln : Real(0);
+  Real g = hw * (sc.mu * lnp - lfn);
+  Real sg = ssqrt(vt * vt + g * g + eps * eps);
+  // W's numerator max(0, vt - phi_eps(vt, g)) is sg - g >= 0; for g > 0 (sticking) it is
+  // the small difference of two large numbers, taken as (vt^2 + eps^2)/(sg + g)
+  Real num = g > Real(0) ? (vt * vt + eps * eps) / (sg + g) : sg - g;
+  Real den = sc.mu * lnp; if (den < Real(1e-12)) den = Real(1e-12);
+  Real W = num / den;
+  Real rf1 = vel[1] + (W + kap) * l1, rf2 = vel[2] + (W + kap) * l2;
+  Real wgt = hw / (hw + W);
+  w.r2[i + 1] = rf1 * wgt; w.r2[i + 2] = rf2 * wgt;
+  w.rhat[i + 1] = rf1; w.rhat[i + 2] = rf2;
+  w.C[i + 1] = W + kap; w.C[i + 2] = W + kap;
+  // radial part of the friction block: rho e e^T, e = lambda_f/|lambda_f|
+  Real rho = Real(0);
+  if (num > Real(0)) {
+    Real fbg = num / sg;                  // 1 - g/sg
+    rho = fbg * hw * lfn / den;
+  }
+  Real e1 = l1 / lfn, e2 = l2 / lfn;
+  w.srad[3 * sl] = rho * e1 * e1; w.srad[3 * sl + 1] = rho * e1 * e2; w.srad[3 * sl + 2] = rho * e2 * e2;
+}
+
 // ---------------------------------------------------------------------------
 // one residual / Jacobian evaluation at iterate (u, lam); returns the merit
 // ---------------------------------------------------------------------------
 // dyn = false (the adjoint): the rows, their compliance and delta only; the dynamics
 // residual and the merit are not formed (the returned merit is 0).
-template <class Real>
+template <bool FEW, class Real>
 __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, const Real* lam, const StepH<Real>& h, bool dyn = true) {
   const int tid = w.tid, nth = blockDim.x;
   const int nb = sc.nb, m = w.ints[0], mc = w.ints[1];
@@ -774,73 +851,22 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
   }
   __syncthreads();
   // contact slots from the first thread on, separator rows from the last: they run beside
-  // one another in different warps
-  for (int sl = tid; sl < sc.n_slots; sl += nth) {
-      if (w.srow[sl] < 0) continue;
-      int i = w.srow[sl];
-      int b = sc.slot_body[sl];
-      int local = sl - sc.slot_base[b];
-      vec3<Real> p = v3(w.qp[7 * b], w.qp[7 * b + 1], w.qp[7 * b + 2]);
-      vec3<Real> n = v3(w.sn[3 * sl], w.sn[3 * sl + 1], w.sn[3 * sl + 2]);
-      vec3<Real> t1 = v3(w.st1[3 * sl], w.st1[3 * sl + 1], w.st1[3 * sl + 2]);
-      vec3<Real> t2 = v3(w.st2[3 * sl], w.st2[3 * sl + 1], w.st2[3 * sl + 2]);
-      vec3<Real> x = slot_point<Real>(sc, b, local, p, w.qp + 7 * b + 3, n);
-      vec3<Real> lev = x - p;
-      vec3<Real> wk = v3(u[6 * b + 3], u[6 * b + 4], u[6 * b + 5]);
-      vec3<Real> dirs[3] = {n, t1, t2};
-      Real vel[3];
-      const MapE<Real> Ek(wk, h);
-      for (int k = 0; k < 3; ++k) {
-        vec3<Real> ang = Ek(cross3(lev, dirs[k]));
-        Real* Jr = w.J + 12 * (i + k);
-        Jr[0] = dirs[k].x; Jr[1] = dirs[k].y; Jr[2] = dirs[k].z; Jr[3] = ang.x; Jr[4] = ang.y; Jr[5] = ang.z;
-        vel[k] = dirs[k].x * u[6 * b] + dirs[k].y * u[6 * b + 1] + dirs[k].z * u[6 * b + 2] + ang.x * u[6 * b + 3] +
-                 ang.y * u[6 * b + 4] + ang.z * u[6 * b + 5];
-      }
-      const Real kap = sc.kappa, eps = sc.eps;
-      const Real hw = hR * w.swhat[sl];
-      // normal row, Eq. (4): phi_eps(c_n/h + kappa lambda_n, h what lambda_n)
-      Real cn = dot3(n, x) - w.sd[sl];
-      Real ln = lam[i], l1 = lam[i + 1], l2 = lam[i + 2];
-      Real a = cn / hR + kap * ln, bb = hw * ln;
-      // At an active contact b = h what lambda_n is large (~10 m/s) and a ~ 0, so the
-      // textbook forms a + b - s, 1 - a/s and 1 - b/s cancel; in FP32 that leaves ~1e-6
-      // m/s of noise in the row, which the small eigenvalue (~kappa) of the impulse split
-      // between redundant contacts amplifies to ~1e-3 N and the Newton iteration stalls.
-      // The same quantities in forms free of cancellation (exact rearrangements):
-      // a + b - s = (2ab - eps^2)/(a + b + s) for a + b > 0;  1 - a/s = (b^2 + eps^2)/(s (s + a))
-      // for a > 0;  1 - b/s likewise.
-      Real s = ssqrt(a * a + bb * bb + eps * eps);
-      const Real apb = a + bb;
-      Real phi = apb > Real(0) ? (Real(2) * a * bb - eps * eps) / (apb + s) : apb - s;
-      Real fa = a > Real(0) ? (bb * bb + eps * eps) / (s * (s + a)) : Real(1) - a / s;
-      Real fb = bb > Real(0) ? (a * a + eps * eps) / (s * (s + bb)) : Real(1) - bb / s;
-      Real scl = fa > Real(1e-12) ? fa : Real(1e-12);
-      w.r2[i] = phi; w.rhat[i] = phi / scl; w.C[i] = kap + hw * fb / scl;
-      // friction rows, Eq. (7): J_f u + (W + kappa) lambda_f with W from the FB reading
-      Real vt = ssqrt(vel[1] * vel[1] + vel[2] * vel[2] + eps * eps);
-      Real lfn = ssqrt(l1 * l1 + l2 * l2 + eps * eps);
-      Real lnp = ln > Real(0) ? ln : Real(0);
-      Real g = hw * (sc.mu * lnp - lfn);
-      Real sg = ssqrt(vt * vt + g * g + eps * eps);
-      // W's numerator max(0, vt - phi_eps(vt, g)) is sg - g >= 0; for g > 0 (sticking) it is
-      // the small difference of two large numbers, taken as (vt^2 + eps^2)/(sg + g)
-      Real num = g > Real(0) ? (vt * vt + eps * eps) / (sg + g) : sg - g;
-      Real den = sc.mu * lnp; if (den < Real(1e-12)) den = Real(1e-12);
-      Real W = num / den;
-      Real rf1 = vel[1] + (W + kap) * l1, rf2 = vel[2] + (W + kap) * l2;
-      Real wgt = hw / (hw + W);
-      w.r2[i + 1] = rf1 * wgt; w.r2[i + 2] = rf2 * wgt;
-      w.rhat[i + 1] = rf1; w.rhat[i + 2] = rf2;
-      w.C[i + 1] = W + kap; w.C[i + 2] = W + kap;
-      // radial part of the friction block: rho e e^T, e = lambda_f/|lambda_f|
-      Real rho = Real(0);
-      if (num > Real(0)) {
-        Real fbg = num / sg;                  // 1 - g/sg
-        rho = fbg * hw * lfn / den;
-      }
-      Real e1 = l1 / lfn, e2 = l2 / lfn;
-      w.srad[3 * sl] = rho * e1 * e1; w.srad[3 * sl + 1] = rho * e1 * e2; w.srad[3 * sl + 2] = rho * e2 * e2;
+  // one another in different warps.  Where warps would idle (few worlds), a slot's friction and
+  // its normal (its position's arithmetic twice) run in different warps, the lighter normals
+  // beside the separator rows: their roots and quotients are this phase's serial chain, and
+  // in FP64 the time of the warp's arithmetic unit (step and adjoint: 1 robot 213 -> 209 us,
+  // 22 in FP64 1605 -> 1534, 37 boxes in FP64 881 -> 817).  With the chip full it would be more
+  // work for the same units (8192 robots 2.35 -> 2.38 ms).
+  const int half = nth >> 1;
+  if (FEW && half >= 32 && sc.n_slots <= half) {
+    const int sl = tid < half ? tid : tid - half;
+    if (sl < sc.n_slots && w.srow[sl] >= 0) {
+      if (tid < half) slot_rows<false, true>(sc, w, u, lam, h, sl);
+      else slot_rows<true, false>(sc, w, u, lam, h, sl);
+    }
+  } else {
+    for (int sl = tid; sl < sc.n_slots; sl += nth)
+      if (w.srow[sl] >= 0) slot_rows<true, true>(sc, w, u, lam, h, sl);
   }
   for (int a = nth - 1 - tid; a < sc.ss; a += nth) sep_row(sc, w, u, lam, h, a, mc);
   __syncthreads();
@@ -1930,7 +1956,7 @@ template <class Real> __device__ __forceinline__ void turn_warps(WS<Real>& w) {
 
 // One world's step; `item` is the launch's work index (the CTA index of a one-CTA-per-
 // world launch, or the index a persistent CTA took from the queue).
-template <class Real>
+template <class Real, bool FEW>
 __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, const StepArgs& a, int item) {
   const int tid = w.tid, nth = blockDim.x;
   const int world = a.list ? a.list[item] : a.world0 + item;
@@ -1975,7 +2001,7 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
   for (;;) {
     // the loop's one evaluation: of the trial iterate, the warm start or the returned
     // iterate; step control: the full step (Sec. III-C) or backtracking on the merit
-    const Real mt = evaluate(sc, w, w.ut, w.lt, h);
+    const Real mt = evaluate<FEW>(sc, w, w.ut, w.lt, h);
     if (phase == 1 && !(mt < merit) && ai + 1 < n_alpha) {
       ++ai;
       alpha *= Real(0.5);
@@ -2163,7 +2189,9 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
 
 // At most 128 threads per world, registers capped at 128 in FP32: eight robot worlds of 64
 // threads per SM then, which their 24.9 KB of workspace allows too.
-template <class Real>
+// FEW: see few_worlds; a kernel of its own, because as a branch of this one its code cost the
+// large launches 1 %.
+template <class Real, bool FEW>
 __global__ void __launch_bounds__(128, sizeof(Real) == 4 ? 4 : 3) step_kernel(const DevScene scp, const StepArgs a) {
   extern __shared__ __align__(16) char smem[];
   __shared__ __align__(16) KScene<Real> ssc;
@@ -2183,7 +2211,7 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 ? 4 : 3) step_kernel(co
       if (it >= a.n_items) break;
       if (a.order) it = a.order[it];
     }
-    step_world<Real>(ssc, w, a, it);
+    step_world<Real, FEW>(ssc, w, a, it);
     if (!a.queue) break;
   }
 }
@@ -2290,7 +2318,7 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 && MODE == ADJ_PAPER ? 
   for (int i = tid; i < 6 * nb; i += nth) w.uk[i] = tp[tl.off_u + i];
   for (int i = tid; i < m; i += nth) w.lk[i] = tp[tl.off_lam + row_lam(w.row[i])];
   __syncthreads();
-  evaluate(sc, w, w.uk, w.lk, h, false);   // J (with E at u*), C, delta, poses at q+
+  evaluate<false>(sc, w, w.uk, w.lk, h, false);   // J (with E at u*), C, delta, poses at q+
   if (tid < 32) {
     // a lane per body: its groups, and by prefix sums over the bodies the places of its
     // pull-back items and their work order by cost (joint groups, contact groups, body terms)
@@ -2566,39 +2594,46 @@ template <class K> cudaError_t ensure_smem(K kernel, size_t smem, int* done_dev,
   return e;
 }
 
-// Threads of a world's CTA in a launch of n worlds for a context set to `threads`.  Few worlds leave
-// most of the chip's schedulers idle, and what counts is one world's latency: four warps then
+// Whether a launch of n worlds is few for the chip: most of its schedulers idle, all worlds run
+// at once, and what counts is one world's latency.  Four CTAs of 128 threads per SM in FP32, two
+// in FP64, whose arithmetic units more warps do not help beyond that (608 robots: adjoint
+// 213 -> 276 us).
+template <class Real> bool few_worlds(int n, int* sms_of_dev) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+  if (!sms_of_dev[dev] &&
+      cudaDeviceGetAttribute(&sms_of_dev[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return false;
+  return n <= (sizeof(Real) == 4 ? 4 : 2) * sms_of_dev[dev];
+}
+
+// Threads of a world's CTA in a launch of few worlds for a context set to `threads`: four warps
 // share its rows and tiles (1 robot, step 234 -> 213 us, adjoint 41 -> 39; 608 robots 269 -> 258 us;
-// 2048 robots would take 981 instead of 665), as long as all worlds run at once: four CTAs of
-// 128 threads per SM in FP32, two in FP64, whose arithmetic units more warps do not help beyond
-// that (608 robots: adjoint 213 -> 276 us).  Scenes of at most a warp's rows gain nothing.
+// 2048 robots would take 981 instead of 665).  Scenes of at most a warp's rows gain nothing.
 // The sums over all rows keep the order of `threads` (sum_threads), so results do not depend on
 // this.  The conjugate-residual solver and the exact adjoint sum over the whole CTA in more
 // places: they keep their threads.
-template <class Real> int cta_threads(const DevScene& sc, int threads, int n, int* sms_of_dev) {
-  if (threads >= 128 || sc.lin != LIN_DIRECT || sc.m_max <= 32) return threads;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return threads;
-  if (!sms_of_dev[dev] &&
-      cudaDeviceGetAttribute(&sms_of_dev[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return threads;
-  return n <= (sizeof(Real) == 4 ? 4 : 2) * sms_of_dev[dev] ? 128 : threads;
+inline int few_threads(const DevScene& sc, int threads) {
+  if (sc.lin != LIN_DIRECT) return threads;
+  const int t = sc.m_max <= 32 ? 64 : 128;
+  return threads > t ? threads : t;
 }
 
 template <class Real>
 cudaError_t launch_step(const DevScene& sc, const StepArgs& a, int threads, cudaStream_t st) {
-  static int done_dev[64] = {0};
-  static size_t done_size[64] = {0};
-  auto kernel = step_kernel<Real>;
-  size_t smem = ws_bytes<Real>(sc);
-  cudaError_t e = ensure_smem(kernel, smem, done_dev, done_size);
-  if (e != cudaSuccess) return e;
-  int n = a.list ? a.n_list : a.n_worlds - a.world0;
-  if (n <= 0) return cudaSuccess;
+  static int done_dev[2][64] = {{0}};
+  static size_t done_size[2][64] = {{0}};
   static int sms[64] = {0};
+  int n = a.list ? a.n_list : a.n_worlds - a.world0;
+  const bool few = few_worlds<Real>(n, sms);
+  auto kernel = few ? step_kernel<Real, true> : step_kernel<Real, false>;
+  size_t smem = ws_bytes<Real>(sc);
+  cudaError_t e = ensure_smem(kernel, smem, done_dev[few], done_size[few]);
+  if (e != cudaSuccess) return e;
+  if (n <= 0) return cudaSuccess;
   StepArgs b = a;
   b.sum_threads = threads;
-  threads = cta_threads<Real>(sc, threads, n, sms);
+  if (few) threads = few_threads(sc, threads);
   if (a.queue) {
     // persistent: as many CTAs as fit on the device at once, fed from the queue
     int dev = 0, n_sms = 0, per_sm = 0;
@@ -2635,7 +2670,7 @@ cudaError_t launch_adjoint(const DevScene& sc, const AdjArgs& a, int threads, cu
   static int sms[64] = {0};
   AdjArgs b = a;
   b.sum_threads = threads;
-  if (mode == ADJ_PAPER) threads = cta_threads<Real>(sc, threads, n, sms);
+  if (mode == ADJ_PAPER && few_worlds<Real>(n, sms)) threads = few_threads(sc, threads);
   kernel<<<n, threads, smem, st>>>(sc, b);
   return cudaGetLastError();
 }

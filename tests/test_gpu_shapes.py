@@ -4,8 +4,8 @@
   rows one warp's registers hold (their factor's order and that of the whole CTA);
 * hinged boxes with every corner active: contact groups of 24 rows (one block per warp; the
   usual ones go two to a warp up to 16 rows), two groups sharing the joint's rows;
-* few worlds run with four warps each, many with the context's threads: the results of a
-  world are bit-identical either way.
+* few worlds run with more warps each (normals and friction in different ones), many with the
+  context's threads: the results of a world are bit-identical either way.
 
 Tolerances are those of the parity tests of the same precision (test_gpu_parity.py): FP64
 1e-7 / 1e-6 / 1e-6, FP32 1e-4 / 1e-3 / 1e-3 for worlds whose iterate solves the step.
@@ -82,19 +82,24 @@ def test_full_contact_groups_match_oracle(ostrich, threads):  # noqa: F811
 
 
 @pytest.mark.parametrize("dtype,per_sm", [("f32", 4), ("f64", 2)])
-def test_results_do_not_depend_on_the_launch(ostrich, dtype, per_sm):  # noqa: F811
-    """The first worlds of a launch one world larger than what runs with four warps each,
-    against the same worlds alone."""
-    sc = S.robot_box_scene()
+@pytest.mark.parametrize("kind,solver", [("robot", 0), ("box", 0), ("robot", 1)])
+def test_results_do_not_depend_on_the_launch(ostrich, dtype, per_sm, kind, solver):  # noqa: F811
+    """The first worlds of a launch one world larger than what runs with four warps each (two
+    for the box, with normals and friction apart), against the same worlds alone."""
+    sc = S.robot_box_scene() if kind == "robot" else S.box_drop_scene()
     W, n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + 1, 6
     tdt = torch.float64 if dtype == "f64" else torch.float32
-    st = np.repeat(S.robot_box_states(sc, n, seed=3), -(-W // n), axis=1)[:, :W]
+    if kind == "robot":
+        st = S.robot_box_states(sc, n, seed=3)
+    else:
+        st = np.concatenate([S.box_drop_state(sc, 0.2 * k, -1e-3 * k) for k in range(n)], axis=1)
+    st = np.repeat(st, -(-W // n), axis=1)[:, :W]
     st = st[:, np.argsort(np.arange(W) % n, kind="stable")]      # worlds of a kind side by side
     ub = S.random_controls(sc.n_servos, W, seed=3)
     g = np.random.default_rng(4).normal(size=st.shape)
     outs = []
     for cols in (np.arange(W), np.arange(0, W, W // n)[:n]):
-        ctx = ostrich.Context(sc, S.SolverConfig(tol=1e-4), len(cols), dtype=dtype, tape_slots=1)
+        ctx = ostrich.Context(sc, S.SolverConfig(tol=1e-4, linear_solver=solver), len(cols), dtype=dtype, tape_slots=1)
         dev = [torch.tensor(np.ascontiguousarray(a[:, cols]), dtype=tdt, device="cuda") for a in (st, ub, g)]
         r = ctx.step(dev[0], dev[1], H, tape_slot=0)
         ds, du = ctx.adjoint(0, dev[2], H)
