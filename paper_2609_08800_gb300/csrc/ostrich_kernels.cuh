@@ -898,22 +898,73 @@ __device__ Real evaluate(const KScene<Real>& sc, WS<Real>& w, const Real* u, con
     // Eq. (10): r_dyn = M (u - u-) - h f - h J^T lambda, per body; merit part |M^-1 r_dyn|^2.
     // The inertia and constraint terms nearly cancel at convergence, so the sum is
     // accumulated with exact products and exact partial sums (acc2).
-    for (int task = tid; task < 6 * nb; task += nth) {
-      const int b = task / 6, k = task - 6 * (task / 6);
-      acc2<Real> rd;
-      body_rows(sc, w, b, [&](int off, int i) { rd.add_prod(w.J[off + k], -hR * lam[i]); });
-      if (k < 3) {
-        const Real m_ = sc.mass[b];
-        rd.add_prod(m_, u[6 * b + k]);
-        rd.add_prod(-m_, w.um[6 * b + k]);
-      } else {
-        for (int c = 0; c < 3; ++c) {
-          rd.add_prod(w.Iw[9 * b + 3 * (k - 3) + c], u[6 * b + 3 + c]);
-          rd.add_prod(-w.Iw[9 * b + 3 * (k - 3) + c], w.um[6 * b + 3 + c]);
+    if constexpr (FEW && sizeof(Real) == 8) {
+      // FP64: what counts is the number of instructions of a warp, each some 60 cycles of its
+      // arithmetic unit whatever the lanes in use.  Four threads a sum, four terms a turn: each
+      // forms its own term's product and the errors of its product and of its partial sum; the
+      // sum itself and that of the errors all four form alike, term by term in acc2's order (19
+      // instructions for four terms instead of 40, and the same bits).  Terms past the end are
+      // zero and change nothing.  From the last thread on, beside the rows above.  The phase
+      // takes 12.3 instead of 17.9 k cycles for a box, 23.7 instead of 27.9 k for a robot; with
+      // more worlds, whose warps fill the units, it is the slower one (583 robots + 1 %).
+      const int seg = 3 - (tid & 3), lane3 = (threadIdx.x & 31) | 3;
+      for (int base = 0; base < 24 * nb; base += nth) {
+        const int e = (base + nth - 1 - tid) >> 2, b = e / 6, k = e - 6 * b;
+        const bool on = e < 6 * nb;
+        const int g = on ? sc.body_group[b] : -1, r0 = g >= 0 ? w.g0[g] : 0, n = g >= 0 ? w.gn[g] : 0;
+        const int tot = on ? n + sc.body_sepn[b] : 0, nm = k < 3 ? 2 : 6, T = on ? tot + nm + 1 : 0;
+        const uint16_t* bs = w.bsep + (on ? b : 0) * (sc.ss > 0 ? sc.ss : 1) - n;
+        Real s = Real(0), cc = Real(0);
+        for (int t0 = 0; __any_sync(0xffffffffu, t0 < T); t0 += 4) {
+          const int t = t0 + seg, r = t - tot;
+          Real x = Real(0), y = Real(0);
+          if (t < tot) {
+            const unsigned off = t < n ? 12 * (r0 + t) : bs[t];
+            x = w.J[off + k];
+            y = -hR * lam[off / 12u];
+          } else if (on && r < nm) {
+            x = k < 3 ? sc.mass[b] : w.Iw[9 * b + 3 * (k - 3) + (r >> 1)];
+            const int q = 6 * b + (k < 3 ? k : 3 + (r >> 1));
+            if (r & 1) { x = -x; y = w.um[q]; } else { y = u[q]; }
+          } else if (on && r == nm) {
+            x = -hR;
+            y = w.f[6 * b + k];
+          }
+          const Real p = rn_mul(x, y), ep = rn_fma(x, y, -p);
+          Real sb = Real(0), sa = Real(0);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const Real t1 = rn_add(s, __shfl_sync(0xffffffffu, p, lane3 - q));
+            if (seg == q) { sb = s; sa = t1; }
+            s = t1;
+          }
+          const Real bp = rn_sub(sa, sb), es = rn_add(rn_sub(sb, rn_sub(sa, bp)), rn_sub(p, bp));
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            cc = rn_add(cc, __shfl_sync(0xffffffffu, es, lane3 - q));
+            cc = rn_add(cc, __shfl_sync(0xffffffffu, ep, lane3 - q));
+          }
         }
+        if (on && seg == 0) w.rdyn[6 * b + k] = rn_add(s, cc);
       }
-      rd.add_prod(-hR, w.f[6 * b + k]);
-      w.rdyn[6 * b + k] = rd.value();
+    } else {
+      for (int task = tid; task < 6 * nb; task += nth) {
+        const int b = task / 6, k = task - 6 * (task / 6);
+        acc2<Real> rd;
+        body_rows(sc, w, b, [&](int off, int i) { rd.add_prod(w.J[off + k], -hR * lam[i]); });
+        if (k < 3) {
+          const Real m_ = sc.mass[b];
+          rd.add_prod(m_, u[6 * b + k]);
+          rd.add_prod(-m_, w.um[6 * b + k]);
+        } else {
+          for (int c = 0; c < 3; ++c) {
+            rd.add_prod(w.Iw[9 * b + 3 * (k - 3) + c], u[6 * b + 3 + c]);
+            rd.add_prod(-w.Iw[9 * b + 3 * (k - 3) + c], w.um[6 * b + 3 + c]);
+          }
+        }
+        rd.add_prod(-hR, w.f[6 * b + k]);
+        w.rdyn[6 * b + k] = rd.value();
+      }
     }
   }
   __syncthreads();
@@ -1169,19 +1220,40 @@ template <int NR, class Real> __device__ __forceinline__ void load_column(const 
 // of chol_inv_inplace in the same order.
 //
 // FP64: its multiply-adds bound it (two a clock per SM), so rows past the end are left out.
-template <int TW> __device__ __forceinline__ void chol_inv_regs(double* A, int n, int nmax, double* buf) {
-  const int lane = threadIdx.x & (TW - 1);
+// The reciprocal root is some 1000 cycles of the warp's arithmetic unit, half of a pivot.
+// PAIR: a second warp (chol_roots), on another unit, takes the root of the next diagonal --
+// which lane k + 1 forms from its own entries alone (a - c c) -- while this one updates the
+// rows.  They meet at the named barriers bar and bar + 1 of their 64 threads, both nmax - 1
+// times, and exchange through xch (4 values).  The 24 x 24
+// separator of a robot: 53.2 -> 42.9 k cycles.
+__device__ __forceinline__ void pair_sync(int id) {
+  __syncwarp();
+  asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory");
+}
+
+template <int TW, bool PAIR = false>
+__device__ __forceinline__ void chol_inv_regs(double* A, int n, int nmax, double* buf, double* xch = nullptr,
+                                              int bar = 0) {
+  const int lane = threadIdx.x & (TW - 1), half = (threadIdx.x & 31) / TW;
   double a[TW];
   load_column(A, n, lane, a);
   double* row = A + lane;
+  double inv;
 #pragma unroll 1
   for (int k = 0; k < nmax; ++k) {
-    const double akk = __shfl_sync(0xffffffffu, a[0], k, TW);
-    const double inv = pivot_rsqrt(akk > 0.0 ? akk : 1e-30);
+    if (!PAIR || k == 0) {
+      const double akk = __shfl_sync(0xffffffffu, a[0], k, TW);
+      inv = pivot_rsqrt(akk > 0.0 ? akk : 1e-30);
+    } else {
+      pair_sync(bar + 1);
+      inv = xch[2 + half];
+    }
     const bool piv = lane == k;
     const double c = piv ? inv : a[0] * inv;
     double* bk = buf + (k & 1 ? TW : 0);
     if (lane > k) bk[lane - k - 1] = c;
+    if (PAIR && lane == k + 1) xch[half] = rn_fma(-c, c, a[1]);
+    if (PAIR && k + 1 < nmax) pair_sync(bar);
     if (lane <= k && k < n) *row = c;
     row += k + 1;
     __syncwarp();
@@ -1194,6 +1266,18 @@ template <int TW> __device__ __forceinline__ void chol_inv_regs(double* A, int n
         for (int r = 0; r < 4; ++r)
           if (q + r + 1 < TW) a[q + r] = rn_fma(-l[r], c, piv ? 0.0 : a[q + r + 1]);
       }
+  }
+}
+
+// The second warp of a pair: the reciprocal roots of the pivots after the first.
+template <int TW> __device__ __forceinline__ void chol_roots(int nmax, double* xch, int bar) {
+  const int half = (threadIdx.x & 31) / TW;
+#pragma unroll 1
+  for (int k = 1; k < nmax; ++k) {
+    pair_sync(bar);
+    const double d = xch[half], inv = pivot_rsqrt(d > 0.0 ? d : 1e-30);
+    if ((threadIdx.x & (TW - 1)) == 0) xch[2 + half] = inv;
+    pair_sync(bar + 1);
   }
 }
 
@@ -1264,12 +1348,34 @@ template <int TW> __device__ __forceinline__ void chol_inv_regs(float* A, int n,
 
 // The inverse factors of the contact groups' blocks.  Blocks of up to 16 rows (five of a
 // wheel's slots active; a robot on flat ground has 6 rows per wheel) go two to a warp, larger
-// ones one to a warp, and blocks beyond 32 rows through shared memory.
-template <class Real> __device__ __forceinline__ void factor_groups(const KScene<Real>& sc, WS<Real>& w) {
+// ones one to a warp, and blocks beyond 32 rows through shared memory.  With few worlds in FP64
+// the second half of the warps takes the roots of the first half's pivots, where that leaves
+// every warp at most one block (or two of 16 rows).
+template <bool FEW, class Real> __device__ __forceinline__ void factor_groups(const KScene<Real>& sc, WS<Real>& w) {
   const int tid = w.tid, wid = tid >> 5, nw = blockDim.x >> 5;
   const int ng = sc.n_groups, gstr = tri_size(sc.pg);
   int big = 0;
   for (int g = 0; g < ng; ++g) big = w.gn[g] > big ? w.gn[g] : big;
+  if constexpr (FEW && sizeof(Real) == 8) {
+    const int hw = nw >> 1, per = big <= 16 ? 2 : 1;
+    if (big <= 32 && ng <= per * hw) {
+      const int job = wid < hw ? wid : wid - hw, bar = 1 + 2 * job, half = per == 2 ? (tid >> 4) & 1 : 0;
+      const int g0 = per * job, g = g0 + half, na = g0 < ng ? w.gn[g0] : 0;
+      const int nb = per == 2 && g0 + 1 < ng ? w.gn[g0 + 1] : 0, nmax = na > nb ? na : nb;
+      Real* xch = w.prow + 64 * (hw + job);
+      Real* A = w.G + (g < ng ? g : 0) * gstr;
+      const int n = g < ng ? w.gn[g] : 0;
+      if (wid >= 2 * hw || nmax == 0) return;
+      if (per == 2) {
+        if (wid < hw) chol_inv_regs<16, true>(A, n, nmax, w.prow + 64 * wid + 32 * half, xch, bar);
+        else chol_roots<16>(nmax, xch, bar);
+      } else {
+        if (wid < hw) chol_inv_regs<32, true>(A, n, nmax, w.prow + 64 * wid, xch, bar);
+        else chol_roots<32>(nmax, xch, bar);
+      }
+      return;
+    }
+  }
   if (big <= 16) {
     const int half = (tid >> 4) & 1;
     Real* buf = w.prow + 64 * wid + 32 * half;
@@ -1415,9 +1521,16 @@ template <class Real> __device__ void chol_inv_inplace4(Real* A, int n, Real* co
 }
 
 // L_s^-1 of the separator block in place over S: in one warp's registers up to 32 rows (the
-// CTA's other warps do not join), else by the whole CTA through shared memory.  The caller
-// synchronises.
-template <class Real> __device__ __forceinline__ void factor_separator(const KScene<Real>& sc, WS<Real>& w) {
+// CTA's other warps do not join; with few worlds in FP64 the last of four warps takes the
+// pivots' roots), else by the whole CTA through shared memory.  The caller synchronises.
+template <bool FEW, class Real> __device__ __forceinline__ void factor_separator(const KScene<Real>& sc, WS<Real>& w) {
+  if constexpr (FEW && sizeof(Real) == 8) {
+    if (blockDim.x == 128 && sc.ss > 0 && sc.ss <= 32) {
+      if (w.tid < 32) chol_inv_regs<32, true>(w.S, sc.ss, sc.ss, w.prow, w.prow + 64 * 3, 1);
+      else if (w.tid >= 96) chol_roots<32>(sc.ss, w.prow + 64 * 3, 1);
+      return;
+    }
+  }
   if (sc.ss > 32) chol_inv_inplace4(w.S, sc.ss, w.prow);
   else if (w.tid < 32 && sc.ss > 0) chol_inv_regs<32>(w.S, sc.ss, sc.ss, w.prow);
 }
@@ -1472,10 +1585,10 @@ template <class Real> __device__ __forceinline__ Real dot2col(const Real* T, int
 //   Lsi = L_s^-1 with L_s L_s^T = S - sum_g F_g F_g^T, the reduced separator (stored in S,
 //   packed).
 // Here all but the last; factor_separator follows.
-template <class Real> __device__ __forceinline__ void factor_eliminate(const KScene<Real>& sc, WS<Real>& w) {
+template <bool FEW, class Real> __device__ __forceinline__ void factor_eliminate(const KScene<Real>& sc, WS<Real>& w) {
   const int tid = w.tid, nth = blockDim.x;
   const int ldg = sc.ldg, cm = sc.cmax, gstr = tri_size(sc.pg);
-  factor_groups(sc, w);
+  factor_groups<FEW>(sc, w);
   __syncthreads();
   // F_g[k][j] = sum_{l <= j} E_g[k][l] Li_g[j][l], two threads per contact row
   const int mc = w.ints[1];
@@ -1739,9 +1852,9 @@ template <class Real> __device__ void pcr_jacobi(const KScene<Real>& sc, WS<Real
 // Block-Jacobi preconditioner: each contact group's block and the (unreduced) separator
 // block of A, as assembled, factored in place to their inverse Cholesky factors (G, S)
 template <class Real> __device__ __forceinline__ void factor_blocks(const KScene<Real>& sc, WS<Real>& w) {
-  factor_groups(sc, w);
+  factor_groups<false>(sc, w);
   __syncthreads();
-  factor_separator(sc, w);
+  factor_separator<false>(sc, w);
   __syncthreads();
 }
 
@@ -2063,9 +2176,9 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
     if (direct || sc.pc == PC_BLOCK) {
       assemble(sc, w, h);
       if (direct) {
-        factor_eliminate(sc, w);
+        factor_eliminate<FEW>(sc, w);
         if (fin) {
-          factor_separator(sc, w);
+          factor_separator<FEW>(sc, w);
           break;
         }
       } else {
@@ -2080,7 +2193,11 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
     const bool beside = direct && nth > 32 && sc.ss <= 32;
     Real* rhs = direct ? w.dl : w.rhs;
     const int t0 = beside ? tid - 32 : tid, T = beside ? 32 : nth;
-    if (beside && tid < 32) factor_separator(sc, w);
+    if constexpr (FEW && sizeof(Real) == 8) {
+      if (beside && (tid < 32 || tid >= 96)) factor_separator<FEW>(sc, w);
+    } else {
+      if (beside && tid < 32) factor_separator<FEW>(sc, w);
+    }
     if (t0 >= 0 && t0 < T) {
       for (int i = t0; i < m; i += T) {
         const Real* Ji = w.J + 12 * i;
@@ -2100,7 +2217,7 @@ __device__ __forceinline__ void step_world(const KScene<Real>& sc, WS<Real>& w, 
     if (direct) {
       if (!beside) {
         arrow_forward(sc, w, w.dl, tid, nth, [] { __syncthreads(); });
-        factor_separator(sc, w);
+        factor_separator<FEW>(sc, w);
         __syncthreads();
       }
       if (tid < 32) arrow_separator(sc, w, w.dl);
@@ -2349,8 +2466,8 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 && MODE == ADJ_PAPER ? 
     // PCR mode tapes no factor: the exact mode's GMRES preconditioner is the direct factor,
     // formed here at the taped iterate
     assemble(sc, w, h);
-    factor_eliminate(sc, w);
-    factor_separator(sc, w);
+    factor_eliminate<false>(sc, w);
+    factor_separator<false>(sc, w);
     __syncthreads();
   } else if (sc.pc == PC_BLOCK) {
     // the PCR operator and preconditioner of the forward pass, at the taped iterate
