@@ -48,8 +48,8 @@ template <class Real> struct WS {
   uint16_t *bsep;   // offsets in J of the body's parts of the separator rows touching it
   // groups
   int *g0, *gn;
-  // Schur storage (block-arrowhead, inverse form): G group blocks, E coupling rows,
-  // H = E G, S reduced separator; prow a pivot-row buffer per warp
+  // Schur storage (block-arrowhead, inverse form): G group blocks, E coupling rows, H their
+  // F = E L^-T, S reduced separator; prow the factors' exchange rows, 64 values per warp
   Real *G, *E, *H, *S, *prow, *tmp, *tmp2;
   // scratch
   Real *red;
@@ -332,20 +332,6 @@ __device__ __forceinline__ void joint_rows_each(const KScene<Real>& sc, int j, v
     const vec3<S> a3 = cross3(b2, e1);
     f(4, z, a3, z, scale(a3, S(-1.0)), dot3(b2, e1));
   }
-}
-
-// The same five rows held in one structure (for callers that need them all at once)
-template <class S> struct JRows {
-  vec3<S> lin_p[5], ang_p[5], lin_c[5], ang_c[5];
-  S c[5];
-};
-
-template <class S, class RP, class RC, class Real>
-__device__ __forceinline__ void joint_rows_geom(const KScene<Real>& sc, int j, vec3<S> pp, const RP& rotp, vec3<S> pc,
-                                                const RC& rotc, JRows<S>& o) {
-  joint_rows_each<S>(sc, j, pp, rotp, pc, rotc, [&](int k, vec3<S> lp, vec3<S> ap, vec3<S> lc, vec3<S> ac, S c) {
-    o.lin_p[k] = lp; o.ang_p[k] = ap; o.lin_c[k] = lc; o.ang_c[k] = ac; o.c[k] = c;
-  });
 }
 
 // Servo row of joint j (Eq. (8)): Jacobian parts before E of the joint rate, the relative
@@ -1224,8 +1210,8 @@ template <int NR, class Real> __device__ __forceinline__ void load_column(const 
 // PAIR: a second warp (chol_roots), on another unit, takes the root of the next diagonal --
 // which lane k + 1 forms from its own entries alone (a - c c) -- while this one updates the
 // rows.  They meet at the named barriers bar and bar + 1 of their 64 threads, both nmax - 1
-// times, and exchange through xch (4 values).  The 24 x 24
-// separator of a robot: 53.2 -> 42.9 k cycles.
+// times, and exchange through xch (4 values).  The 24 x 24 separator of a robot: 53.2 -> 42.9 k
+// cycles.
 __device__ __forceinline__ void pair_sync(int id) {
   __syncwarp();
   asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory");

@@ -31,7 +31,6 @@ struct SceneLayout {
   int smode[NJ_CAP];   // SERVO_VELOCITY / SERVO_POSITION
   // solver settings
   int budget, kmin, ls, pullback;
-  int refine;     // iterative-refinement sweeps after each forward (Newton-step) Schur solve
   int refine_adj; // iterative-refinement sweeps after the adjoint's Schur solve
   // linear solver of Eq. (12): LIN_DIRECT, or LIN_PCR (matrix-free preconditioned conjugate
   // residual with preconditioner pc; pcr_iters iterations per Newton step; the adjoint's
@@ -45,7 +44,7 @@ struct SceneLayout {
   // static coupling between groups and separator rows (the separator rows are always
   // present): group g couples to separator rows cpl_row[g][0 .. cpl_n[g]); separator row
   // a belongs to the lists of sep_n[a] <= 2 groups, at (sep_g[a][i], sep_k[a][i])
-  int ldg, lds, cmax;                    // odd row lengths of the coupling blocks (ldg); cmax coupling rows
+  int ldg, cmax;                         // odd row lengths of the coupling blocks (ldg); cmax coupling rows
   int cpl_n[NB_CAP];
   unsigned char cpl_row[NB_CAP][SEP_CAP];
   unsigned char sep_n[SEP_CAP], sep_g[SEP_CAP][2], sep_k[SEP_CAP][2];
@@ -105,7 +104,6 @@ inline void finish_scene(SceneLayout& s) {
     }
   s.ss = 5 * s.nj + s.n_servo;
   s.ldg = s.pg | 1;
-  s.lds = s.ss | 1;
   int gof[NB_CAP];
   for (int b = 0; b < NB_CAP; ++b) { gof[b] = -1; s.body_sepn[b] = 0; }
   for (int g = 0; g < s.n_groups; ++g) { gof[s.group_body[g]] = g; s.cpl_n[g] = 0; }

@@ -78,7 +78,6 @@ inline ostrich_status build_scene(const ostrich_scene_desc* d, const ostrich_sol
   // matrix-free product (8 sweeps); the forward Newton iteration corrects an inexact
   // step by itself (without refinement it takes the same number of iterations to the
   // same residuals), so its solves are not refined.
-  s.refine = 0;
   s.refine_adj = dtype == OSTRICH_F32 ? 8 : 0;
   // the direct factor by default; PCR is selected on a context (ostrich_set_linear_solver)
   s.lin = LIN_DIRECT; s.pc = PC_JACOBI; s.pcr_iters = 16; s.pcr_iters_adj = 256;
