@@ -2731,7 +2731,9 @@ cudaError_t launch_step(const DevScene& sc, const StepArgs& a, int threads, cuda
   const bool few = few_worlds<Real>(n, sms);
   auto kernel = few ? step_kernel<Real, true> : step_kernel<Real, false>;
   size_t smem = ws_bytes<Real>(sc);
-  cudaError_t e = ensure_smem(kernel, smem, done_dev[few], done_size[few]);
+  // both kernels at once: a launch of another number of worlds may be under capture
+  cudaError_t e = ensure_smem(step_kernel<Real, false>, smem, done_dev[0], done_size[0]);
+  if (e == cudaSuccess) e = ensure_smem(step_kernel<Real, true>, smem, done_dev[1], done_size[1]);
   if (e != cudaSuccess) return e;
   if (n <= 0) return cudaSuccess;
   StepArgs b = a;
