@@ -144,30 +144,28 @@ template <class Real> __host__ __device__ __forceinline__ size_t ws_layout_bytes
 }
 template <class Real> size_t ws_bytes(const DevScene& s) { return ws_layout_bytes<Real>(s); }
 
-// deterministic block reduction (fixed tree); result broadcast through w.red[0]
+// Deterministic block sum (fixed tree), the same in every thread, through w.red[8..].  One
+// barrier: between the reads of one call and the writes of the next lies another barrier of
+// the caller's, and block_sum2 has places of its own, so that the two may alternate.
 template <class Real> __device__ Real block_sum(WS<Real>& w, Real v) {
   const int tid = w.tid, lane = tid & 31, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) w.red[8 + wid] = v;
   __syncthreads();
-  if (lane == 0) w.red[wid] = v;
-  __syncthreads();
-  if (tid == 0) {
-    Real acc = Real(0);
-    for (int i = 0; i < nw; ++i) acc += w.red[i];
-    w.red[32] = acc;
-  }
-  __syncthreads();
-  return w.red[32];
+  Real acc = Real(0);
+  for (int i = 0; i < nw; ++i) acc += w.red[8 + i];
+  return acc;
 }
 
-// two deterministic block sums at once (fixed tree, as block_sum): results in a, b
+// Two deterministic block sums at once (fixed tree, as block_sum): results in a, b.  The same
+// rule on barriers.  (512 robots by conjugate residuals, whose iterations hold one of each: 1291 ->
+// 1267 us with one barrier instead of three and two; 8192 robots directly 2371 -> 2351.)
 template <class Real> __device__ void block_sum2(WS<Real>& w, Real& a, Real& b) {
   const int tid = w.tid, lane = tid & 31, wid = tid >> 5, nw = (blockDim.x + 31) >> 5;
   for (int o = 16; o > 0; o >>= 1) {
     a += __shfl_xor_sync(0xffffffffu, a, o);
     b += __shfl_xor_sync(0xffffffffu, b, o);
   }
-  __syncthreads();
   if (lane == 0) { w.red[wid] = a; w.red[16 + wid] = b; }
   __syncthreads();
   Real sa = Real(0), sb = Real(0);
