@@ -1203,7 +1203,10 @@ template <int NR, class Real> __device__ __forceinline__ void load_column(const 
 // pivot).  Row k of L^-1 is then final and goes to A.  Every entry receives the operations
 // of chol_inv_inplace in the same order.
 //
-// FP64: its multiply-adds bound it (two a clock per SM), so rows past the end are left out.
+// FP64: its multiply-adds bound it (two a clock per SM), so rows past the end are left out.  Of
+// two blocks in a warp the shorter one goes on with the longer one's pivots: on its own, which
+// are zero, its lanes would go the other way at the test for a positive pivot, and the warp
+// through the root twice (37 boxes, step and adjoint: 754 -> 707 us).
 // The reciprocal root is some 1000 cycles of the warp's arithmetic unit, half of a pivot.
 // PAIR: a second warp (chol_roots), on another unit, takes the root of the next diagonal --
 // which lane k + 1 forms from its own entries alone (a - c c) -- while this one updates the
@@ -1226,7 +1229,7 @@ __device__ __forceinline__ void chol_inv_regs(double* A, int n, int nmax, double
 #pragma unroll 1
   for (int k = 0; k < nmax; ++k) {
     if (!PAIR || k == 0) {
-      const double akk = __shfl_sync(0xffffffffu, a[0], k, TW);
+      const double akk = __shfl_sync(0xffffffffu, a[0], TW == 32 ? k : (n > k ? half : half ^ 1) * TW + k);
       inv = pivot_rsqrt(akk > 0.0 ? akk : 1e-30);
     } else {
       pair_sync(bar + 1);
@@ -1254,12 +1257,12 @@ __device__ __forceinline__ void chol_inv_regs(double* A, int n, int nmax, double
 }
 
 // The second warp of a pair: the reciprocal roots of the pivots after the first.
-template <int TW> __device__ __forceinline__ void chol_roots(int nmax, double* xch, int bar) {
+template <int TW> __device__ __forceinline__ void chol_roots(int n, int nmax, double* xch, int bar) {
   const int half = (threadIdx.x & 31) / TW;
 #pragma unroll 1
   for (int k = 1; k < nmax; ++k) {
     pair_sync(bar);
-    const double d = xch[half], inv = pivot_rsqrt(d > 0.0 ? d : 1e-30);
+    const double d = xch[TW == 32 || n > k ? half : half ^ 1], inv = pivot_rsqrt(d > 0.0 ? d : 1e-30);
     if ((threadIdx.x & (TW - 1)) == 0) xch[2 + half] = inv;
     pair_sync(bar + 1);
   }
@@ -1352,10 +1355,10 @@ template <bool FEW, class Real> __device__ __forceinline__ void factor_groups(co
       if (wid >= 2 * hw || nmax == 0) return;
       if (per == 2) {
         if (wid < hw) chol_inv_regs<16, true>(A, n, nmax, w.prow + 64 * wid + 32 * half, xch, bar);
-        else chol_roots<16>(nmax, xch, bar);
+        else chol_roots<16>(n, nmax, xch, bar);
       } else {
         if (wid < hw) chol_inv_regs<32, true>(A, n, nmax, w.prow + 64 * wid, xch, bar);
-        else chol_roots<32>(nmax, xch, bar);
+        else chol_roots<32>(n, nmax, xch, bar);
       }
       return;
     }
@@ -1511,7 +1514,7 @@ template <bool FEW, class Real> __device__ __forceinline__ void factor_separator
   if constexpr (FEW && sizeof(Real) == 8) {
     if (blockDim.x == 128 && sc.ss > 0 && sc.ss <= 32) {
       if (w.tid < 32) chol_inv_regs<32, true>(w.S, sc.ss, sc.ss, w.prow, w.prow + 64 * 3, 1);
-      else if (w.tid >= 96) chol_roots<32>(sc.ss, w.prow + 64 * 3, 1);
+      else if (w.tid >= 96) chol_roots<32>(sc.ss, sc.ss, w.prow + 64 * 3, 1);
       return;
     }
   }
