@@ -2401,7 +2401,7 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 && MODE == ADJ_PAPER ? 
   __shared__ __align__(16) KScene<Real> ssc;
   __shared__ unsigned char bgl[NB_CAP * GROUPS_PER_BODY];
   __shared__ int bgn[NB_CAP], item0[NB_CAP + 1];
-  __shared__ int ncon[NB_CAP], jpre[NB_CAP + 1], cpre[NB_CAP + 1];
+  __shared__ int ncon[NB_CAP], jpre[NB_CAP + 1], cpre[NB_CAP + 1], n_first;
   scene_to_shared(scp, a.h, ssc);
   const KScene<Real>& sc = ssc;
   WS<Real> w = ws_carve<Real>(smem, sc);
@@ -2436,7 +2436,7 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 && MODE == ADJ_PAPER ? 
   evaluate<false>(sc, w, w.uk, w.lk, h, false);   // J (with E at u*), C, delta, poses at q+
   if (tid < 32) {
     // a lane per body: its groups, and by prefix sums over the bodies the places of its
-    // pull-back items and their work order by cost (joint groups, contact groups, body terms)
+    // pull-back items and the joint and contact groups before it
     const int lane = tid;
     const bool tr = MODE == ADJ_PAPER && sc.pullback == 1;
     int nc = 0, ng = 0;
@@ -2447,14 +2447,14 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 && MODE == ADJ_PAPER ? 
       bgn[lane] = ng;
       ncon[lane] = nc;
     }
-    const int n_coord = __any_sync(0xffffffffu, dual_pos) ? 7 : 4;
-    int pi = lane < nb ? 7 * (ng + 1) : 0, pj = n_coord * (ng - nc), pc = n_coord * nc;
+    dual_pos = __any_sync(0xffffffffu, dual_pos);
+    int pi = lane < nb ? 7 * (ng + 1) : 0, pj = ng - nc, pc = nc;
     for (int o = 1; o < NB_CAP; o <<= 1) {             // inclusive sums
       const int ui = __shfl_up_sync(0xffffffffu, pi, o), uj = __shfl_up_sync(0xffffffffu, pj, o);
       const int uc = __shfl_up_sync(0xffffffffu, pc, o);
       if (lane >= o) { pi += ui; pj += uj; pc += uc; }
     }
-    if (lane == 0) { item0[0] = 0; jpre[0] = 0; cpre[0] = 0; }
+    if (lane == 0) { item0[0] = 0; jpre[0] = 0; cpre[0] = 0; n_first = dual_pos ? 7 : 4; }
     if (lane < nb) { item0[lane + 1] = pi; jpre[lane + 1] = pj; cpre[lane + 1] = pc; }
   }
   if (sc.lin == LIN_DIRECT) {
@@ -2644,39 +2644,53 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 && MODE == ADJ_PAPER ? 
   // body's own terms), each a dual-number evaluation along that coordinate; the items of a
   // coordinate are summed in a fixed order
   const bool trunc = MODE == ADJ_PAPER && sc.pullback == 1;
-  Real* item = w.G;     // the factor (G, E, H, S, one carved run) is no longer needed;
-                        // sum_b 7 (groups_b + 1) <= 14 m_max items
+  Real* item = w.G;     // the factor (G, H, S, one carved run; E lies over dl = wl and is not part
+                        // of it) is no longer needed; sum_b 7 (groups_b + 1) <= 14 m_max items
   // taken in cost order (every joint item, then every contact item, then the body terms)
   // so that the threads' loads even out; each item is stored at its place in the per-body
-  // layout, which fixes the order of the sums below.  n_coord: the four quaternion
-  // coordinates, and the three positions after them where a group has no closed form for those.
-  const int nj_items = jpre[nb], nc_items = cpre[nb], n_items = nj_items + nc_items + 4 * nb;
-  for (int e = tid; e < n_items; e += nth) {
-    int b = 0, c, k;
-    if (e < nj_items) {
-      while (e >= jpre[b + 1]) ++b;
-      const int nj = bgn[b] - ncon[b], r = e - jpre[b];
-      c = r / nj;
-      k = 1 + ncon[b] + (r - c * nj);
-    } else if (e < nj_items + nc_items) {
-      const int e2 = e - nj_items;
-      while (e2 >= cpre[b + 1]) ++b;
-      const int nc = ncon[b], r = e2 - cpre[b];
-      c = r / nc;
-      k = 1 + (r - c * nc);
-    } else {
-      const int e3 = e - nj_items - nc_items;
-      b = e3 / 4;
-      c = e3 - 4 * b;
-      k = 0;
+  // layout, which fixes the order of the sums below.  First the four quaternion coordinates,
+  // and the three positions after them where a group has no closed form for those.  A
+  // non-finite item means a non-finite value among what the duals multiply: a zero derivative
+  // times it is NaN along the positions too, which their closed form would lose, so that
+  // world takes a second pass, over all positions.
+  int c0 = 0, nco = n_first;
+  bool all_dual = false;
+  for (;;) {
+    const int nbc = c0 ? 3 : 4, nj_items = nco * jpre[nb], nc_items = nco * cpre[nb];
+    const int n_items = nj_items + nc_items + nbc * nb;
+    bool lost = false;
+    for (int e = tid; e < n_items; e += nth) {
+      int b = 0, c, k;
+      if (e < nj_items) {
+        while (e >= nco * jpre[b + 1]) ++b;
+        const int nj = bgn[b] - ncon[b], r = e - nco * jpre[b];
+        c = r / nj;
+        k = 1 + ncon[b] + (r - c * nj);
+      } else if (e < nj_items + nc_items) {
+        const int e2 = e - nj_items;
+        while (e2 >= nco * cpre[b + 1]) ++b;
+        const int nc = ncon[b], r = e2 - nco * cpre[b];
+        c = r / nc;
+        k = 1 + (r - c * nc);
+      } else {
+        const int e3 = e - nj_items - nc_items;
+        b = e3 / nbc;
+        c = e3 - nbc * b;
+        k = 0;
+      }
+      c += c0;
+      c = c < 4 ? 3 + c : c - 4;
+      const int grp = k ? bgl[b * GROUPS_PER_BODY + k - 1] : 0;
+      if (c < 3 && !all_dual && !position_needs_dual(sc, w, grp, trunc)) continue;
+      const Real v =
+          k == 0 ? body_vjp(sc, w, b, c, gq, wu, h) : group_vjp_q<Real, MODE>(sc, w, ex, grp, b, c, wl, wu, trunc, h);
+      item[item0[b] + c * (bgn[b] + 1) + k] = v;
+      lost = lost || !isfinite(v);
     }
-    c = c < 4 ? 3 + c : c - 4;
-    const int grp = k ? bgl[b * GROUPS_PER_BODY + k - 1] : 0;
-    if (c < 3 && !position_needs_dual(sc, w, grp, trunc)) continue;
-    item[item0[b] + c * (bgn[b] + 1) + k] =
-        k == 0 ? body_vjp(sc, w, b, c, gq, wu, h) : group_vjp_q<Real, MODE>(sc, w, ex, grp, b, c, wl, wu, trunc, h);
+    if (!__syncthreads_or(lost) || all_dual) break;
+    all_dual = true;
+    c0 = 4; nco = 3;
   }
-  __syncthreads();
   const Real inv_h = Real(1) / hR;
   for (int e = tid; e < nb * 7; e += nth) {
     const int b = e / 7, c = e % 7;
@@ -2684,7 +2698,7 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 && MODE == ADJ_PAPER ? 
     const int base = item0[b] + c * (bgn[b] + 1);
     for (int k = 0; k <= bgn[b]; ++k) {
       const int grp = k ? bgl[b * GROUPS_PER_BODY + k - 1] : 0;
-      if (c >= 3 || (k && position_needs_dual(sc, w, grp, trunc))) acc.add(item[base + k]);
+      if (c >= 3 || all_dual || (k && position_needs_dual(sc, w, grp, trunc))) acc.add(item[base + k]);
       else acc.add(k ? group_pull_position<Real, MODE>(sc, w, ex, grp, b, c, wl, inv_h) : gq[7 * b + c]);
     }
     dout[(size_t)(7 * b + c) * ld + world] = acc.value();
