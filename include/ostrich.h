@@ -130,6 +130,12 @@ ostrich_status ostrich_layout(const ostrich_ctx* ctx, int32_t out[4]);
  * the same order: a world's result does not depend on how many others the launch holds. */
 ostrich_status ostrich_set_threads(ostrich_ctx* ctx, int threads);
 
+/* Threads per world that a step of n worlds (n_worlds, or a list's n_list) runs with on the
+ * current device: the context's, or more in a small launch.  Where it is not the context's,
+ * timing such a launch says nothing about that setting.  Without a device the context's; 0
+ * for a NULL context or n < 1. */
+int ostrich_launch_threads(const ostrich_ctx* ctx, int n);
+
 /* Launch schedule of ostrich_step (an autotuner knob; results do not depend on it):
  * 0 one CTA per world (default); 1 persistent: as many CTAs as fit on the device take
  * worlds from a device work counter, heaviest first by each world's Newton iterations in

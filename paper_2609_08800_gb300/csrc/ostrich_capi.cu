@@ -16,6 +16,7 @@ namespace ost {
 template <class Real> cudaError_t launch_step(const DevScene&, const StepArgs&, int, cudaStream_t);
 template <class Real> cudaError_t launch_adjoint(const DevScene&, const AdjArgs&, int, cudaStream_t);
 template <class Real> size_t adj_smem_bytes(const DevScene&, int);
+template <class Real> int step_threads(const DevScene&, int, int);
 }  // namespace ost
 
 struct ostrich_ctx {
@@ -108,6 +109,12 @@ ostrich_status ostrich_set_threads(ostrich_ctx* c, int threads) {
   if (threads != 32 && threads != 64 && threads != 128) return fail(c, OSTRICH_EINVAL, "threads must be 32, 64 or 128");
   c->threads = threads;
   return OSTRICH_OK;
+}
+
+int ostrich_launch_threads(const ostrich_ctx* c, int n) {
+  if (!c || n < 1) return 0;
+  return c->dtype == OSTRICH_F64 ? ost::step_threads<double>(c->sc, c->threads, n)
+                                 : ost::step_threads<float>(c->sc, c->threads, n);
 }
 
 ostrich_status ostrich_set_schedule(ostrich_ctx* c, int schedule) {

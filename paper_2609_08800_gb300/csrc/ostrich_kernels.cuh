@@ -20,6 +20,7 @@
 // define OST_REAL) so that the two compile in parallel.
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <atomic>
 #include "ostrich_scene.h"
 #include "ostrich_math.cuh"
 #include "ostrich_contacts.cuh"
@@ -2727,13 +2728,15 @@ template <class K> cudaError_t ensure_smem(K kernel, size_t smem, int* done_dev,
 // at once, and what counts is one world's latency.  Four CTAs of 128 threads per SM in FP32, two
 // in FP64, whose arithmetic units more warps do not help beyond that (608 robots: adjoint
 // 213 -> 276 us).
-template <class Real> bool few_worlds(int n, int* sms_of_dev) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
-  if (!sms_of_dev[dev] &&
-      cudaDeviceGetAttribute(&sms_of_dev[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return false;
-  return n <= (sizeof(Real) == 4 ? 4 : 2) * sms_of_dev[dev];
+template <class Real> bool few_worlds(int n) {
+  static std::atomic<int> sms[64];
+  int dev = 0, k = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return false; }
+  if (!(k = sms[dev].load(std::memory_order_relaxed))) {
+    if (cudaDeviceGetAttribute(&k, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) { cudaGetLastError(); return false; }
+    sms[dev].store(k, std::memory_order_relaxed);
+  }
+  return n <= (sizeof(Real) == 4 ? 4 : 2) * k;
 }
 
 // Threads of a world's CTA in a launch of few worlds for a context set to `threads`: four warps
@@ -2748,13 +2751,17 @@ inline int few_threads(const DevScene& sc, int threads) {
   return threads > t ? threads : t;
 }
 
+// Threads per world of a step of n worlds for a context set to `threads`.
+template <class Real> int step_threads(const DevScene& sc, int threads, int n) {
+  return few_worlds<Real>(n) ? few_threads(sc, threads) : threads;
+}
+
 template <class Real>
 cudaError_t launch_step(const DevScene& sc, const StepArgs& a, int threads, cudaStream_t st) {
   static int done_dev[2][64] = {{0}};
   static size_t done_size[2][64] = {{0}};
-  static int sms[64] = {0};
   int n = a.list ? a.n_list : a.n_worlds - a.world0;
-  const bool few = few_worlds<Real>(n, sms);
+  const bool few = few_worlds<Real>(n);
   auto kernel = few ? step_kernel<Real, true> : step_kernel<Real, false>;
   size_t smem = ws_bytes<Real>(sc);
   // both kernels at once: a launch of another number of worlds may be under capture
@@ -2798,10 +2805,9 @@ cudaError_t launch_adjoint(const DevScene& sc, const AdjArgs& a, int threads, cu
   if (e != cudaSuccess) return e;
   int n = a.list ? a.n_list : a.n_worlds - a.world0;
   if (n <= 0) return cudaSuccess;
-  static int sms[64] = {0};
   AdjArgs b = a;
   b.sum_threads = threads;
-  if (mode == ADJ_PAPER && few_worlds<Real>(n, sms)) threads = few_threads(sc, threads);
+  if (mode == ADJ_PAPER && few_worlds<Real>(n)) threads = few_threads(sc, threads);
   kernel<<<n, threads, smem, st>>>(sc, b);
   return cudaGetLastError();
 }
@@ -2817,6 +2823,7 @@ template <class Real> size_t ws_used(const DevScene& s) {
 
 template cudaError_t launch_step<OST_REAL>(const DevScene&, const StepArgs&, int, cudaStream_t);
 template cudaError_t launch_adjoint<OST_REAL>(const DevScene&, const AdjArgs&, int, cudaStream_t);
+template int step_threads<OST_REAL>(const DevScene&, int, int);
 template size_t ws_bytes<OST_REAL>(const DevScene&);
 template size_t ws_used<OST_REAL>(const DevScene&);
 template size_t adj_smem_bytes<OST_REAL>(const DevScene&, int);

@@ -69,6 +69,8 @@ def lib():
         L.ostrich_create.restype = ctypes.c_int
         L.ostrich_layout.argtypes = [_vp, ctypes.POINTER(ctypes.c_int32)]
         L.ostrich_set_threads.argtypes = [_vp, ctypes.c_int]
+        L.ostrich_launch_threads.argtypes = [_vp, ctypes.c_int]
+        L.ostrich_launch_threads.restype = ctypes.c_int
         L.ostrich_set_schedule.argtypes = [_vp, ctypes.c_int]
         L.ostrich_step.argtypes = [_vp, _vp, _vp, ctypes.c_double, _vp, _vp, _vp, _vp, _vp, ctypes.c_int, _vp]
         L.ostrich_adjoint.argtypes = [_vp, ctypes.c_int, _vp, ctypes.c_double, _vp, _vp, _vp]
@@ -278,6 +280,10 @@ class Context:
     def set_threads(self, threads):
         self._check(lib().ostrich_set_threads(self._h, int(threads)), "ostrich_set_threads")
         self.threads = int(threads)
+
+    def launch_threads(self, n=None):
+        """Threads per world that a step of n worlds (default: all) runs with."""
+        return int(lib().ostrich_launch_threads(self._h, self.n_worlds if n is None else int(n)))
 
     def set_schedule(self, schedule):
         """0: one CTA per world; 1: persistent CTAs, heaviest worlds first."""

@@ -90,17 +90,26 @@ SCHEDULES = (0, 1)
 
 def tune(ctx, state, controls, h, candidates=CANDIDATES, reps=3, persist=True, path=None, schedules=SCHEDULES):
     """Time each (threads, schedule) candidate on (state, controls), set the fastest on ctx,
-    record it.  Returns (best threads, {threads: ms} at the best schedule)."""
-    times = {}
+    record it.  Returns (best threads, {threads: ms} at the best schedule).
+
+    A launch of few worlds may run with more threads than the context's, so that several
+    candidates launch the same kernel and their times differ by noise alone.  Of those the
+    context's own setting is kept (it fixes the order of the sums), and nothing is recorded:
+    the table is read for full batches, about which such times say nothing."""
+    own = getattr(ctx, "threads", 64)
+    times, launched = {}, {}
     for sch in schedules:
         ctx.set_schedule(sch)
         for t in candidates:
             ctx.set_threads(t)
+            launched[t] = ctx.launch_threads()
             times[(t, sch)] = time_step(ctx, state, controls, h, reps)
     best_t, best_s = min(times, key=times.get)
+    if own in launched and launched[own] == launched[best_t]:
+        best_t = own
     ctx.set_threads(best_t)
     ctx.set_schedule(best_s)
-    if persist:
+    if persist and all(launched[t] == t for t in candidates):
         store(key(ctx), {"threads": best_t, "schedule": best_s,
                          "ms": {f"{t}/{sch}": round(v, 4) for (t, sch), v in times.items()},
                          "worlds": ctx.n_worlds}, path)
