@@ -203,11 +203,24 @@ template <class Real> size_t ex_bytes(const DevScene& s) {
   return used;
 }
 
-// Shared memory of one world in the adjoint kernel of a mode.
+// Per body the constraint groups touching it and where its pull-back items lie (adjoint_kernel).
+struct AdjLists {
+  unsigned char bgl[NB_CAP * GROUPS_PER_BODY];   // groups of each body (body_groups)
+  int bgn[NB_CAP], ncon[NB_CAP];                 // their number, that of the contacts among them
+  int item0[NB_CAP + 1];                         // first item of each body
+  int jpre[NB_CAP + 1], cpre[NB_CAP + 1];        // joint and contact groups of the bodies before
+  int n_first;                                   // coordinates of the first pass over the items
+};
+
+// Dynamic shared memory of one world in the adjoint kernel of a mode.
 template <class Real> size_t adj_smem_bytes(const DevScene& s, int mode) {
   size_t b = ws_bytes<Real>(s);
   if (mode == ADJ_EXACT) b = (b + ex_bytes<Real>(s) + 15) & ~(size_t)15;
   return b;
+}
+// All shared memory of its CTA: beside that the static scene and lists.
+template <class Real> size_t adj_smem_total(const DevScene& s, int mode) {
+  return adj_smem_bytes<Real>(s, mode) + ((sizeof(KScene<Real>) + 15) & ~(size_t)15) + sizeof(AdjLists);
 }
 
 // Groups touching body b: slot indices (active slots of the body) then n_slots + j for its

@@ -15,7 +15,8 @@
 namespace ost {
 template <class Real> cudaError_t launch_step(const DevScene&, const StepArgs&, int, cudaStream_t);
 template <class Real> cudaError_t launch_adjoint(const DevScene&, const AdjArgs&, int, cudaStream_t);
-template <class Real> size_t adj_smem_bytes(const DevScene&, int);
+template <class Real> size_t ws_bytes(const DevScene&);
+template <class Real> size_t adj_smem_total(const DevScene&, int);
 template <class Real> int step_threads(const DevScene&, int, int);
 }  // namespace ost
 
@@ -51,6 +52,14 @@ static ostrich_status cuda_fail(ostrich_ctx* c, cudaError_t e, const char* where
   if (c) std::snprintf(c->err, sizeof(c->err), "%s: %s", where, cudaGetErrorString(e));
   return OSTRICH_ECUDA;
 }
+
+// Whether a world of the scene fits a CTA of the adjoint of a mode.
+static bool adjoint_fits(const ost::DevScene& s, int dtype, int mode) {
+  return (dtype == OSTRICH_F64 ? ost::adj_smem_total<double>(s, mode) : ost::adj_smem_total<float>(s, mode)) <=
+         ost::SMEM_CTA_MAX;
+}
+
+static const char* const too_large = "the adjoint's working set exceeds shared memory";
 
 static size_t elem_size(int dtype) { return dtype == OSTRICH_F64 ? sizeof(double) : sizeof(float); }
 
@@ -192,6 +201,7 @@ ostrich_status ostrich_adjoint_list(ostrich_ctx* c, const void* dL_dnext, double
   if (!c->tape) return fail(c, OSTRICH_ETAPE, "the context has no tape");
   if (!dL_dnext || !dL_dstate) return fail(c, OSTRICH_EINVAL, "gradient pointers missing");
   if (!(h > 0)) return fail(c, OSTRICH_EINVAL, "h must be positive");
+  if (!adjoint_fits(c->sc, c->dtype, c->adj_mode)) return fail(c, OSTRICH_EINVAL, too_large);
   if (n_list < 0 || n_list > c->n_worlds) return fail(c, OSTRICH_EINVAL, "n_list outside [0, n_worlds]");
   if (n_list > 0 && (!worlds || !tape_slots)) return fail(c, OSTRICH_EINVAL, "worlds or tape_slots list missing");
   if (n_list == 0) return OSTRICH_OK;
@@ -210,9 +220,8 @@ ostrich_status ostrich_adjoint_list(ostrich_ctx* c, const void* dL_dnext, double
 ostrich_status ostrich_set_adjoint_mode(ostrich_ctx* c, int mode, int32_t* krylov_iters) {
   if (!c) return OSTRICH_EINVAL;
   if (mode != OSTRICH_ADJ_PAPER && mode != OSTRICH_ADJ_EXACT) return fail(c, OSTRICH_EINVAL, "unknown adjoint mode");
-  const size_t smem = c->dtype == OSTRICH_F64 ? ost::adj_smem_bytes<double>(c->sc, mode)
-                                              : ost::adj_smem_bytes<float>(c->sc, mode);
-  if (smem > ost::SMEM_CTA_MAX) return fail(c, OSTRICH_EINVAL, "the exact adjoint's working set exceeds shared memory");
+  if (mode == OSTRICH_ADJ_EXACT && !adjoint_fits(c->sc, c->dtype, mode))
+    return fail(c, OSTRICH_EINVAL, "the exact adjoint's working set exceeds shared memory");
   c->adj_mode = mode;
   c->krylov = krylov_iters;
   return OSTRICH_OK;
@@ -227,11 +236,8 @@ ostrich_status ostrich_set_linear_solver(ostrich_ctx* c, int solver, int precond
   ost::DevScene s = c->sc;
   s.lin = solver; s.pc = precond; s.pcr_iters = iters; s.pcr_iters_adj = adj_iters;
   s.pcr_rtol_adj = adj_rtol > 0 ? adj_rtol : (c->dtype == OSTRICH_F32 ? 1e-10 : 1e-12);
-  const bool f64 = c->dtype == OSTRICH_F64;
-  const size_t ws = f64 ? ost::ws_bytes<double>(s) : ost::ws_bytes<float>(s);
-  const size_t used = f64 ? ost::ws_used<double>(s) : ost::ws_used<float>(s);
-  const size_t adj = f64 ? ost::adj_smem_bytes<double>(s, c->adj_mode) : ost::adj_smem_bytes<float>(s, c->adj_mode);
-  if (ws > ost::SMEM_CTA_MAX || used > ws || adj > ost::SMEM_CTA_MAX)
+  const size_t step = c->dtype == OSTRICH_F64 ? ost::step_smem_total<double>(s) : ost::step_smem_total<float>(s);
+  if (step > ost::SMEM_CTA_MAX || (c->adj_mode == OSTRICH_ADJ_EXACT && !adjoint_fits(s, c->dtype, c->adj_mode)))
     return fail(c, OSTRICH_EINVAL, "the PCR working set exceeds shared memory");
   c->sc = s;
   std::fill(c->slot_written.begin(), c->slot_written.end(), (unsigned char)0);
@@ -252,6 +258,7 @@ ostrich_status ostrich_adjoint_params(ostrich_ctx* c, int tape_slot, const void*
   if (!c->slot_written[tape_slot]) return fail(c, OSTRICH_ETAPE, "tape slot holds no recorded step");
   if (h != c->slot_h[tape_slot]) return fail(c, OSTRICH_EINVAL, "h differs from the recorded step");
   if (!dL_dnext || !dL_dstate) return fail(c, OSTRICH_EINVAL, "gradient pointers missing");
+  if (!adjoint_fits(c->sc, c->dtype, c->adj_mode)) return fail(c, OSTRICH_EINVAL, too_large);
   ost::AdjArgs a;
   a.tape = slot_ptr(c, tape_slot); a.dL_dnext = dL_dnext; a.dL_dstate = dL_dstate; a.dL_dcontrols = dL_dcontrols;
   a.ld = c->ld; a.n_worlds = c->n_worlds; a.world0 = 0; a.h = h;

@@ -144,6 +144,10 @@ template <class Real> __host__ __device__ __forceinline__ size_t ws_layout_bytes
   return (used + 15) & ~(size_t)15;
 }
 template <class Real> size_t ws_bytes(const DevScene& s) { return ws_layout_bytes<Real>(s); }
+// All shared memory of a CTA of the step kernels: the working set beside their static scene.
+template <class Real> size_t step_smem_total(const DevScene& s) {
+  return ws_bytes<Real>(s) + ((sizeof(KScene<Real>) + 15) & ~(size_t)15);
+}
 
 // Deterministic block sum (fixed tree), the same in every thread, through w.red[8..].  One
 // barrier: between the reads of one call and the writes of the next lies another barrier of
@@ -2400,9 +2404,9 @@ template <class Real, int MODE>
 __global__ void __launch_bounds__(128, sizeof(Real) == 4 && MODE == ADJ_PAPER ? 4 : 3) adjoint_kernel(const DevScene scp, const AdjArgs a) {
   extern __shared__ __align__(16) char smem[];
   __shared__ __align__(16) KScene<Real> ssc;
-  __shared__ unsigned char bgl[NB_CAP * GROUPS_PER_BODY];
-  __shared__ int bgn[NB_CAP], item0[NB_CAP + 1];
-  __shared__ int ncon[NB_CAP], jpre[NB_CAP + 1], cpre[NB_CAP + 1], n_first;
+  __shared__ __align__(16) AdjLists al;
+  unsigned char* bgl = al.bgl;
+  int *bgn = al.bgn, *item0 = al.item0, *ncon = al.ncon, *jpre = al.jpre, *cpre = al.cpre;
   scene_to_shared(scp, a.h, ssc);
   const KScene<Real>& sc = ssc;
   WS<Real> w = ws_carve<Real>(smem, sc);
@@ -2455,7 +2459,7 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 && MODE == ADJ_PAPER ? 
       const int uc = __shfl_up_sync(0xffffffffu, pc, o);
       if (lane >= o) { pi += ui; pj += uj; pc += uc; }
     }
-    if (lane == 0) { item0[0] = 0; jpre[0] = 0; cpre[0] = 0; n_first = dual_pos ? 7 : 4; }
+    if (lane == 0) { item0[0] = 0; jpre[0] = 0; cpre[0] = 0; al.n_first = dual_pos ? 7 : 4; }
     if (lane < nb) { item0[lane + 1] = pi; jpre[lane + 1] = pj; cpre[lane + 1] = pc; }
   }
   if (sc.lin == LIN_DIRECT) {
@@ -2654,7 +2658,7 @@ __global__ void __launch_bounds__(128, sizeof(Real) == 4 && MODE == ADJ_PAPER ? 
   // non-finite item means a non-finite value among what the duals multiply: a zero derivative
   // times it is NaN along the positions too, which their closed form would lose, so that
   // world takes a second pass, over all positions.
-  int c0 = 0, nco = n_first;
+  int c0 = 0, nco = al.n_first;
   bool all_dual = false;
   for (;;) {
     const int nbc = c0 ? 3 : 4, nj_items = nco * jpre[nb], nc_items = nco * cpre[nb];
@@ -2812,20 +2816,11 @@ cudaError_t launch_adjoint(const DevScene& sc, const AdjArgs& a, int threads, cu
   return cudaGetLastError();
 }
 
-
-// Bytes the carve of one world actually consumes from a 16-byte aligned base; the
-// context refuses a scene for which this exceeds ws_bytes (checked on the host).
-template <class Real> size_t ws_used(const DevScene& s) {
-  size_t used = 0;
-  ws_carve<Real>(nullptr, s, &used);
-  return used;
-}
-
 template cudaError_t launch_step<OST_REAL>(const DevScene&, const StepArgs&, int, cudaStream_t);
 template cudaError_t launch_adjoint<OST_REAL>(const DevScene&, const AdjArgs&, int, cudaStream_t);
 template int step_threads<OST_REAL>(const DevScene&, int, int);
 template size_t ws_bytes<OST_REAL>(const DevScene&);
-template size_t ws_used<OST_REAL>(const DevScene&);
-template size_t adj_smem_bytes<OST_REAL>(const DevScene&, int);
+template size_t step_smem_total<OST_REAL>(const DevScene&);
+template size_t adj_smem_total<OST_REAL>(const DevScene&, int);
 
 }  // namespace ost

@@ -20,6 +20,7 @@
 namespace ost {
 template <class Real> cudaError_t launch_step(const DevScene&, const StepArgs&, int, cudaStream_t);
 template <class Real> cudaError_t launch_adjoint(const DevScene&, const AdjArgs&, int, cudaStream_t);
+template <class Real> size_t adj_smem_total(const DevScene&, int);
 }  // namespace ost
 
 static __device__ __align__(256) unsigned char g_noalloc_tape[OSTRICH_NOALLOC_SCRATCH_BYTES];
@@ -61,6 +62,7 @@ extern "C" ostrich_status ostrich_step_adjoint_noalloc(const ostrich_scene_desc*
   if (scene->env == OSTRICH_ENV_HEIGHTMAP) return OSTRICH_EINVAL;
   ost::DevScene s;
   if (ost::build_scene(scene, cfg, OSTRICH_F32, s) != OSTRICH_OK) return OSTRICH_EINVAL;
+  if (ost::adj_smem_total<float>(s, OSTRICH_ADJ_PAPER) > ost::SMEM_CTA_MAX) return OSTRICH_EINVAL;
   if (s.n_servo > 0 && !controls) return OSTRICH_EINVAL;
   ost::TapeLayout tl = ost::tape_layout(s);
   const size_t need = (size_t)n_worlds * (size_t)tl.total * sizeof(float);
@@ -86,6 +88,7 @@ extern "C" ostrich_status ostrich_noalloc_capacity(const ostrich_scene_desc* sce
   if (scene->env == OSTRICH_ENV_HEIGHTMAP) return OSTRICH_EINVAL;
   ost::DevScene s;
   if (ost::build_scene(scene, cfg, OSTRICH_F32, s) != OSTRICH_OK) return OSTRICH_EINVAL;
+  if (ost::adj_smem_total<float>(s, OSTRICH_ADJ_PAPER) > ost::SMEM_CTA_MAX) return OSTRICH_EINVAL;
   const size_t rec = (size_t)ost::tape_layout(s).total * sizeof(float);
   *max_worlds = (int32_t)((size_t)OSTRICH_NOALLOC_SCRATCH_BYTES / rec);
   if (record_bytes) *record_bytes = rec;

@@ -11,10 +11,9 @@
 #include "ostrich_scene.h"
 
 namespace ost {
-template <class Real> size_t ws_bytes(const DevScene&);
-template <class Real> size_t ws_used(const DevScene&);
+template <class Real> size_t step_smem_total(const DevScene&);
 
-// Shared-memory limit of one CTA on sm_103a (the working set of one world must fit).
+// Shared-memory limit of one CTA on sm_103a, for a kernel's dynamic and static variables together.
 constexpr size_t SMEM_CTA_MAX = 227 * 1024;
 
 // Fills s from d and cfg for element type dtype (OSTRICH_F32 / OSTRICH_F64).  The
@@ -82,9 +81,8 @@ inline ostrich_status build_scene(const ostrich_scene_desc* d, const ostrich_sol
   // the direct factor by default; PCR is selected on a context (ostrich_set_linear_solver)
   s.lin = LIN_DIRECT; s.pc = PC_JACOBI; s.pcr_iters = 16; s.pcr_iters_adj = 256;
   s.pcr_rtol_adj = dtype == OSTRICH_F32 ? 1e-10 : 1e-12;
-  const size_t smem = dtype == OSTRICH_F64 ? ws_bytes<double>(s) : ws_bytes<float>(s);
-  const size_t used = dtype == OSTRICH_F64 ? ws_used<double>(s) : ws_used<float>(s);
-  if (smem > SMEM_CTA_MAX || used > smem) return OSTRICH_EINVAL;
+  if ((dtype == OSTRICH_F64 ? step_smem_total<double>(s) : step_smem_total<float>(s)) > SMEM_CTA_MAX)
+    return OSTRICH_EINVAL;
   return OSTRICH_OK;
 }
 
