@@ -125,9 +125,10 @@ ostrich_status ostrich_create(const ostrich_scene_desc* scene, const ostrich_sol
 ostrich_status ostrich_layout(const ostrich_ctx* ctx, int32_t out[4]);
 
 /* Threads per world (32, 64 or 128) of both kernels; the autotuner's knob.  It fixes the order in
- * which the sums over a world's rows are taken, hence the results' rounding.  A launch of so
- * few worlds that all run at once with 128 threads each may use 128 whatever the setting, in
- * the same order: a world's result does not depend on how many others the launch holds. */
+ * which the sums over a world's rows are taken, hence the results' rounding.  A launch of few
+ * worlds (at most four per SM in FP32, two in FP64) under the direct solver runs with at
+ * least 128 threads per world (64 in scenes of at most 32 rows), in the same order: a
+ * world's result does not depend on how many others the launch holds. */
 ostrich_status ostrich_set_threads(ostrich_ctx* ctx, int threads);
 
 /* Threads per world that a step of n worlds (n_worlds, or a list's n_list) runs with on the
@@ -276,7 +277,7 @@ void ostrich_destroy(ostrich_ctx* ctx);
  * adds no computation to ostrich_step / ostrich_adjoint.
  *
  * One forward step of n_worlds worlds (as ostrich_step, without impulses, ids or
- * status; one CTA of 64 threads per world) followed at once by the adjoint of that step
+ * status; as a context of 64 threads per world) followed at once by the adjoint of that step
  * (as ostrich_adjoint), with the tape in a fixed library array of
  * OSTRICH_NOALLOC_SCRATCH_BYTES instead of a context.  Arrays are caller-owned device
  * pointers in the layout above (ld >= n_worlds; 0 means n_worlds).  No context is

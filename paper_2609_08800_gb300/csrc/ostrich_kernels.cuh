@@ -56,7 +56,7 @@ template <class Real> struct WS {
   Real *red;
   int *ints;      // [0] rows, [1] contact rows, [7] contact-generation status bits (4: candidates beyond
                   // the slots), [8], [9] decisions of the exact adjoint, [14] turn of the warps, [15] work item
-  Real *scal;     // [0] merit cur, [1] best merit, [2] delta, [3] merit trial
+  Real *scal;     // [2] delta, the damping at the iterate evaluated last
   Real *pcr;      // PCR mode: r, z, p, A p, A z, P A p and the Jacobi diagonal, m_max each
 };
 
@@ -790,7 +790,7 @@ __device__ __forceinline__ void slot_rows(const KScene<Real>& sc, WS<Real>& w, c
       fb = bb > Real(0) ? (a * a + eps * eps) / (s * (s + bb)) : Real(1) - bb / s;
     } else {
       // one quotient for either form: a warp with lanes of both kinds would go through two
-      // (step and adjoint: 8192 robots 2356 -> 2336 us, 1001 robots on the plane 263 -> 258)
+      // (step and adjoint: 8192 robots 2351 -> 2336 us, 1001 robots on the plane 261 -> 259)
       fa = (a > Real(0) ? bb * bb + eps * eps : a) / (a > Real(0) ? s * (s + a) : s);
       fb = (bb > Real(0) ? a * a + eps * eps : bb) / (bb > Real(0) ? s * (s + bb) : s);
       if (!(a > Real(0))) fa = Real(1) - fa;
@@ -2012,9 +2012,10 @@ __device__ int pcr_solve_refined(const KScene<Real>& sc, WS<Real>& w, const Real
 // ---------------------------------------------------------------------------
 // forward step kernel
 // ---------------------------------------------------------------------------
-// The scene lives in shared memory during a launch, in working precision: kernels index its
-// per-body and per-row tables with thread-dependent indices, which the constant (parameter)
-// cache would serialise across a warp.
+// The scene lives in a CTA's shared memory, in working precision: kernels index its per-body and
+// per-row tables with thread-dependent indices, which the constant (parameter) cache would
+// serialise across a warp.  Every CTA forms it as it starts (once per world, or once per
+// persistent CTA), each value by one thread, the servo compliance by a division in FP64.
 template <class Real> __device__ __forceinline__ void scene_to_shared(const DevScene& src, double h, KScene<Real>& dst) {
   const SceneLayout& sl = src;
   SceneLayout& dl = dst;
@@ -2728,10 +2729,16 @@ template <class K> cudaError_t ensure_smem(K kernel, size_t smem, int* done_dev,
   return e;
 }
 
-// Whether a launch of n worlds is few for the chip: most of its schedulers idle, all worlds run
-// at once, and what counts is one world's latency.  Four CTAs of 128 threads per SM in FP32, two
-// in FP64, whose arithmetic units more warps do not help beyond that (608 robots: adjoint
-// 213 -> 276 us).
+// Whether a launch of n worlds is few for the chip: at most four per SM in FP32, two in FP64.
+// Most of its schedulers would idle, and what counts is one world's latency.  The line, by
+// the robot's step without and with all that follows from it (us): FP32, 1 world 149 / 136, two
+// per SM 253 / 235, four 273 / 260, five 306 / 387; FP64, one per SM 1413 / 1092, two 1552 / 1215,
+// three 1506 / 1450, but four 1901 / 2249 and their adjoint 207 / 275 (its arithmetic units
+// are full).  Boxes: FP32 four per SM 139 / 128, FP64 two 682 / 556.  The line takes no account of
+// how many worlds a scene's workspace lets run at once: where they run in turns there is
+// the more to gain (eight chained boxes, FP32, 58 KB, three per SM at once: four per SM 2194 /
+// 1895; FP64, 114 KB, one at once: two per SM 13170 / 9425).  A context of 128 threads with
+// 64 slots gains nothing in FP32 (terrain, four per SM 267 / 275).
 template <class Real> bool few_worlds(int n) {
   static std::atomic<int> sms[64];
   int dev = 0, k = 0;
@@ -2744,8 +2751,7 @@ template <class Real> bool few_worlds(int n) {
 }
 
 // Threads of a world's CTA in a launch of few worlds for a context set to `threads`: four warps
-// share its rows and tiles (1 robot, step 234 -> 213 us, adjoint 41 -> 39; 608 robots 269 -> 258 us;
-// 2048 robots would take 981 instead of 665).  Scenes of at most a warp's rows gain nothing.
+// share its rows and tiles.  Scenes of at most a warp's rows gain nothing from more than two.
 // The sums over all rows keep the order of `threads` (sum_threads), so results do not depend on
 // this.  The conjugate-residual solver and the exact adjoint sum over the whole CTA in more
 // places: they keep their threads.

@@ -57,8 +57,8 @@ struct SceneLayout {
 };
 
 // Everything a kernel needs to know about the scene and the solver settings, passed by
-// value as a kernel parameter.  The physical values are doubles here; a launch turns them
-// once into its own precision (KScene).
+// value as a kernel parameter.  The physical values are doubles here; a CTA turns them into
+// its kernel's precision as it starts (KScene).
 struct DevScene : SceneLayout {
   double mu, g;
   double box[5];                 // x0, x1, y0, y1, H
@@ -74,10 +74,12 @@ struct DevScene : SceneLayout {
 // The time step and half of it in working precision.
 template <class Real> struct StepH { Real h, hh; };
 
-// The scene of one launch in working precision, in shared memory: the layout, the physical
+// A CTA's copy of the scene in working precision, in shared memory: the layout, the physical
 // values rounded to Real, and the quotients that the kernels would otherwise form again for
 // every row (1/m, 1/I, the servo compliance).  On this chip a double-precision operation or
-// conversion costs tens of cycles, so none is left on the FP32 kernels' path.
+// conversion costs tens of cycles: the FP32 kernels have them as a CTA starts, in the test of
+// a step's last merit and in the exact adjoint's stopping tests, but not in the Newton
+// loop (unless it records a merit trace) or the paper's adjoint.
 template <class Real> struct KScene : SceneLayout {
   Real mu, g, box[5], hsp, hox, hoy;
   Real mass[NB_CAP], minv[NB_CAP], inertia[NB_CAP][3], iinv[NB_CAP][3], half[NB_CAP][3], radius[NB_CAP], hw[NB_CAP];
